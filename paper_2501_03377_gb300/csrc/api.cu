@@ -36,6 +36,7 @@ void run_precond_f64(const tpcg_plan* pl, const double* R, double* Z, SolveState
 void run_precond_cmp(const tpcg_plan* p, const Geom& g, const double* R, double* Z, SolveState* st);
 int run_precond_tc(const tpcg_plan* pl, float* Z, SolveState* st);
 int tc_plan_setup(tpcg_plan* pl);
+int oz_plan_setup(tpcg_plan* pl);
 void tc_plan_release(tpcg_plan* pl);
 int tc_launches_per_apply(const tpcg_plan* pl);
 void tc_apply_grain(tpcg_plan* pl);
@@ -153,6 +154,7 @@ void free_plan(tpcg_plan* p) {
     for (int d = 0; d < 2; ++d) {
       cudaFree(p->d_W64[a][d]);
       cudaFree(p->d_Wt16[a][d]);
+      cudaFree(p->d_oz[a][d]);
     }
     cudaFree(p->d_lam64[a]);
     cudaFree(p->d_lam32[a]);
@@ -681,7 +683,7 @@ int tpcg_plan_create(int nx, int ny, int nz, const int bc[3], const double h[3],
     for (int i = 0; i < kFxCount && !rc; ++i)
       if ((size_t)p->fx_blocks[i] * 4 > p->partial_slots) rc = TPCG_ERR_UNSUPPORTED;
   }
-  if (!rc && prec != TPCG_FP64) rc = tc_plan_setup(p);
+  if (!rc) rc = (prec != TPCG_FP64) ? tc_plan_setup(p) : oz_plan_setup(p);
   // the set-up copies ran on the legacy stream; wait for them only (not for other streams' work)
   if (!rc && cudaStreamSynchronize(0) != cudaSuccess) rc = TPCG_ERR_CUDA;
   if (rc) {

@@ -115,6 +115,8 @@ __global__ void __launch_bounds__(256) k_modeprod_f64(ModeArgsF64 a) {
   }
 }
 
+bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, double* Y, const double* R, SolveState* st);
+
 // Runs the whole FP64 preconditioner: R (FP64, unpadded) -> Z (FP64).  With
 // st != nullptr the last pass also performs the PCG finalize.
 void run_precond_f64(const tpcg_plan* pl, const double* R, double* Z, SolveState* st) {
@@ -122,12 +124,17 @@ void run_precond_f64(const tpcg_plan* pl, const double* R, double* Z, SolveState
   const double* in = R;
   for (int s = 0; s < ns; ++s) {
     const StageParams& p = pl->stages[s];
+    double* out = (s == ns - 1) ? Z : (double*)pl->d_T[s & 1];
+    if (run_pass_oz(pl, p, in, out, R, st)) {
+      in = out;
+      continue;
+    }
     ModeArgsF64 a{};
     a.p = p;
     a.X = in;
     a.Wm = pl->d_W64[p.axis][p.dir];
     const bool last = (s == ns - 1);
-    a.Y = last ? Z : (double*)pl->d_T[s & 1];
+    a.Y = out;
     a.lamA = pl->d_lam64[p.lamA];
     a.lamB = pl->d_lam64[p.lamB];
     a.lamC = pl->d_lam64[p.lamC];
