@@ -115,20 +115,24 @@ __global__ void __launch_bounds__(256) k_modeprod_f64(ModeArgsF64 a) {
   }
 }
 
-bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, double* Y, const double* R, SolveState* st);
+bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, double* Y, const double* R, SolveState* st,
+                 bool after_pass);
 
 // Runs the whole FP64 preconditioner: R (FP64, unpadded) -> Z (FP64).  With
 // st != nullptr the last pass also performs the PCG finalize.
 void run_precond_f64(const tpcg_plan* pl, const double* R, double* Z, SolveState* st) {
   const int ns = (int)pl->stages.size();
   const double* in = R;
+  bool after_pass = false;
   for (int s = 0; s < ns; ++s) {
     const StageParams& p = pl->stages[s];
     double* out = (s == ns - 1) ? Z : (double*)pl->d_T[s & 1];
-    if (run_pass_oz(pl, p, in, out, R, st)) {
+    if (run_pass_oz(pl, p, in, out, R, st, after_pass)) {
+      after_pass = true;
       in = out;
       continue;
     }
+    after_pass = false;
     ModeArgsF64 a{};
     a.p = p;
     a.X = in;

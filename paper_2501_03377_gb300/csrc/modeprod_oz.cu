@@ -68,6 +68,7 @@ struct OzArgs {
   long long oa, ob, oc;
   int vec_in, vec_out;  // 16-byte row loads; 32-byte runs of eight output rows
   int iters;            // tiles per CTA
+  int first;            // the kernel before this one on the stream is not a pass
   int scale, singular;
   const double* lamA;
   const double* lamB;
@@ -137,6 +138,7 @@ __device__ __forceinline__ double scaled_i64(long long v, int e) {
 
 template <bool FINAL>
 __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
+  if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
   if (a.st && a.st->done) return;  // (uniform over the grid)
   // Programmatic dependent launch: the next pass sets up on SMs this grid has left and waits
   // (griddepcontrol.wait) before it touches this pass's output.
@@ -496,8 +498,11 @@ int oz_plan_setup(tpcg_plan* p) {
   return cudaGetLastError() == cudaSuccess ? TPCG_OK : TPCG_ERR_CUDA;
 }
 
-// One mode-product pass; false when its axis has no digit images.
-bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, double* Y, const double* R, SolveState* st) {
+// One mode-product pass; false when its axis has no digit images.  `after_pass`: the previous kernel on the stream
+// is another of these passes.  Every other kernel may be the one that sets the state's `done` word, so the pass
+// behind it waits for it before it looks.
+bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, double* Y, const double* R, SolveState* st,
+                 bool after_pass) {
   const uint8_t* img = p->d_oz[sp.axis][sp.dir];
   if (!img) return false;
   OzArgs a{};
@@ -520,6 +525,7 @@ bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, dou
                ((uintptr_t)Y & 31) == 0)
                   ? 1
                   : 0;
+  a.first = after_pass ? 0 : 1;
   a.scale = sp.scale;
   a.singular = p->singular ? 1 : 0;
   a.lamA = p->d_lam64[sp.lamA];

@@ -41,6 +41,7 @@ constexpr int kBlk = 16384;  // one 128-row x 64-element K tile of a K-major ope
 constexpr int kTubeCols = 128;  // columns of one tube tile (two MN-major atoms of 64)
 
 struct SlabArgs {
+  int first;  // first launch of an application: the kernel before it may set the state's `done` word
   int n, q, t;             // grid nx, ny, nz
   // frontal pair
   int MB1, N1, KT1;        // step 1: 128-row blocks of n', N = q padded to 16, K tiles (64) of n
@@ -136,6 +137,7 @@ template <class InT, class OutT, bool FINAL>
 __global__ void __launch_bounds__(kFrontalThreads, 1)
     k_frontal_pair(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA1,
                    const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmO, SlabArgs a) {
+  if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
   if (a.st && a.st->done) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
@@ -478,6 +480,7 @@ template <class InT, bool PAIR>
 __global__ void __launch_bounds__(kSlabThreads, 1)
     k_tube_pair(const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmW1,
                 const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmO, SlabArgs a) {
+  if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
   if (a.st && a.st->done) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
@@ -1009,6 +1012,7 @@ int run_precond_slab(const tpcg_plan* p, float* Z, SolveState* st) {
     const bool last = (i == ns - 1);
     if (last && (void*)Z != p->d_Z) return TPCG_ERR_INVALID_ARG;  // the output map names the plan's Z
     a.st = st;
+    a.first = i == 0 ? 1 : 0;
     a.partials = p->d_partials;
     LaunchScope ls(p, kKModeTC);
     if (sp->fp16) slab_launch<__half>(L, a, last && st != nullptr, p->stream);

@@ -85,6 +85,7 @@ struct KShape<Bf16Pair> {
 };
 
 struct TcArgs {
+  int first;  // first pass of an application: the kernel before it may set the state's `done` word
   int C, KT, Cout, VR, Np, MB, acc_cols, tmem_cols, NS;
   int rows, B;
   int B1;  // fused pair: the row split (a, b) of the forward pass, for G
@@ -194,6 +195,7 @@ template <int FORM, class InT, class OutT, bool FINAL>
 __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     k_modeprod_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                   const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmO, TcArgs a) {
+  if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
   if (a.st && a.st->done) return;
   // Programmatic dependent launch: the next pass may start its prologue (barriers, TMEM, eigenbasis
   // load) on SMs this grid frees; it waits (griddepcontrol.wait) before touching this pass's output.
@@ -747,6 +749,7 @@ template <class InT>
 __global__ void __launch_bounds__(kPairThreads, 1)
     k_modeprod_pair(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW1,
                     const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmO, TcArgs a) {
+  if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
   if (a.st && a.st->done) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
@@ -1044,6 +1047,7 @@ constexpr int kPairSplitThreads = (2 + kPairSplitEpi) * 32;
 __global__ void __launch_bounds__(kPairSplitThreads, 1)
     k_modeprod_pair_split(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW1,
                           const __grid_constant__ CUtensorMap tmW2, TcArgs a) {
+  if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
   if (a.st && a.st->done) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
@@ -1859,6 +1863,7 @@ int run_precond_tc(const tpcg_plan* p, float* Z, SolveState* st) {
     a.out = last ? (void*)Z : s.out;
     if (last && (void*)Z != p->d_Z) a.tstore = 0;  // the output map names the plan's Z buffer
     a.st = st;
+    a.first = si == 0 ? 1 : 0;
     a.Rt = reinterpret_cast<const uint16_t*>(p->d_Rlp);
     a.partials = p->d_partials;
     LaunchScope ls(p, kKModeTC);
