@@ -66,7 +66,10 @@ extern "C" {
  * In every form the residual r = eta - L ups, the CG inner products, alpha,
  * beta, the solution update and the null-space (mean) projection are FP64;
  * only the three forward and three backward mode products change.        */
-#define TPCG_FP64         0  /* mode products in FP64 (CUDA cores)                   */
+#define TPCG_FP64         0  /* mode products accurate to FP64: axes of at most 256
+                                points as exact FP16 digit slices on the tensor
+                                cores (55-bit operands, one rounding to FP64 per
+                                product), longer ones on the FP64 pipe              */
 #define TPCG_MIXED_TF32   1  /* TF32 tensor-core mode products (FP32 containers rounded
                                 to nearest even at the 10-bit TF32 mantissa), FP32
                                 accumulation and FP32 intermediates: FP32's range,

@@ -37,6 +37,7 @@ void run_precond_cmp(const tpcg_plan* p, const Geom& g, const double* R, double*
 int run_precond_tc(const tpcg_plan* pl, float* Z, SolveState* st);
 int tc_plan_setup(tpcg_plan* pl);
 int oz_plan_setup(tpcg_plan* pl);
+bool oz_axis_ok(int l);
 void tc_plan_release(tpcg_plan* pl);
 int tc_launches_per_apply(const tpcg_plan* pl);
 void tc_apply_grain(tpcg_plan* pl);
@@ -159,6 +160,7 @@ void free_plan(tpcg_plan* p) {
     cudaFree(p->d_lam64[a]);
     cudaFree(p->d_lam32[a]);
   }
+  cudaFree(p->d_G);
   cudaFree(p->d_R);
   cudaFree(p->d_P[0]);
   if (p->prec == TPCG_FP64) cudaFree(p->d_P[1]);  // mixed forms: one allocation for the ring
@@ -544,17 +546,21 @@ int tpcg_plan_create(int nx, int ny, int nz, const int bc[3], const double h[3],
   for (int m = 0; m < 3 && !rc; ++m) {
     const int l = lens[m];
     const AxisBasis& A = p->ax[m];
-    std::vector<double> VT((size_t)l * l);
-    for (int i = 0; i < l; ++i)
-      for (int j = 0; j < l; ++j) VT[(size_t)j * l + i] = A.V[(size_t)i * l + j];
     std::vector<float> lam32(A.lam.begin(), A.lam.end());
     lam32.resize((size_t)pad_to(l, 16) + 16, 0.0f);  // 16-wide epilogue reads stay in bounds
-    if ((rc = dalloc(p, &p->d_W64[m][0], (size_t)l * l))) break;
-    if ((rc = dalloc(p, &p->d_W64[m][1], (size_t)l * l))) break;
+    // FP64 matrices of the axes whose FP64 products run on the FP64 pipe; the others keep digit images
+    const bool f64 = prec == TPCG_FP64 && !oz_axis_ok(l);
+    if (f64 && (rc = dalloc(p, &p->d_W64[m][0], (size_t)l * l))) break;
+    if (f64 && (rc = dalloc(p, &p->d_W64[m][1], (size_t)l * l))) break;
     if ((rc = dalloc(p, &p->d_lam64[m], (size_t)l))) break;
     if ((rc = dalloc(p, &p->d_lam32[m], lam32.size()))) break;
-    cudaMemcpy(p->d_W64[m][0], A.V.data(), sizeof(double) * l * l, cudaMemcpyHostToDevice);   // W = V
-    cudaMemcpy(p->d_W64[m][1], VT.data(), sizeof(double) * l * l, cudaMemcpyHostToDevice);    // W = V^T
+    if (f64) {
+      std::vector<double> VT((size_t)l * l);
+      for (int i = 0; i < l; ++i)
+        for (int j = 0; j < l; ++j) VT[(size_t)j * l + i] = A.V[(size_t)i * l + j];
+      cudaMemcpy(p->d_W64[m][0], A.V.data(), sizeof(double) * l * l, cudaMemcpyHostToDevice);   // W = V
+      cudaMemcpy(p->d_W64[m][1], VT.data(), sizeof(double) * l * l, cudaMemcpyHostToDevice);    // W = V^T
+    }
     cudaMemcpy(p->d_lam64[m], A.lam.data(), sizeof(double) * l, cudaMemcpyHostToDevice);
     cudaMemcpy(p->d_lam32[m], lam32.data(), sizeof(float) * lam32.size(), cudaMemcpyHostToDevice);
     if (prec == TPCG_MIXED_TF32) {
@@ -638,18 +644,12 @@ int tpcg_plan_create(int nx, int ny, int nz, const int bc[3], const double h[3],
     rc = dalloc(p, &r, p->lp_plane ? 2 * p->lp_plane : (size_t)nz * ny * p->pitch16[0] * lp_elem);
     p->d_Rlp = r;
   }
-  for (int i = 0; i < 2 && !rc; ++i) {
-    if (prec == TPCG_FP64) {
-      double* t = nullptr;
-      rc = dalloc(p, &t, p->t_elems);
-      p->d_T[i] = t;
-    } else {
-      uint16_t* t = nullptr;
-      const size_t words = p->t_plane ? 2 * p->t_plane : p->t_elems * lp_elem;
-      rc = dalloc(p, &t, words);
-      p->d_T[i] = t;
-      if (!rc) cudaMemset(t, 0, words * 2);
-    }
+  for (int i = 0; i < 2 && !rc && prec != TPCG_FP64; ++i) {  // (FP64 form: its intermediates use W and Z)
+    uint16_t* t = nullptr;
+    const size_t words = p->t_plane ? 2 * p->t_plane : p->t_elems * lp_elem;
+    rc = dalloc(p, &t, words);
+    p->d_T[i] = t;
+    if (!rc) cudaMemset(t, 0, words * 2);
   }
   if (!rc) rc = dalloc(p, &p->d_state, 1);
   {

@@ -5,8 +5,9 @@
 // last forward pass and the PCG reductions (<R, Z>, sum Z) fused into the
 // epilogue of the last backward pass.
 //
-// FP64 has no tensor-core path on this part, so this is a register-blocked
-// SIMT GEMM: 64 x 64 output tiles, 16-deep K slabs staged in shared memory,
+// Axes of at most 256 points run as digit slices on the tensor cores
+// (modeprod_oz.cu).  Longer ones run here, on the FP64 pipe: a register-blocked
+// SIMT GEMM, 64 x 64 output tiles, 16-deep K slabs staged in shared memory,
 // 4 x 4 outputs per thread.
 #include "tpcg_dev.cuh"
 
@@ -126,7 +127,9 @@ void run_precond_f64(const tpcg_plan* pl, const double* R, double* Z, SolveState
   bool after_pass = false;
   for (int s = 0; s < ns; ++s) {
     const StageParams& p = pl->stages[s];
-    double* out = (s == ns - 1) ? Z : (double*)pl->d_T[s & 1];
+    // intermediates (N elements each) alternate between W, idle during an application, and the plan's Z; the last
+    // pass reads W (an even number of passes)
+    double* out = (s == ns - 1) ? Z : ((s & 1) ? (double*)pl->d_Z : pl->d_W);
     if (run_pass_oz(pl, p, in, out, R, st, after_pass)) {
       after_pass = true;
       in = out;

@@ -30,14 +30,22 @@
 // The whole contraction of a row sits in one tile, so a row's scale is found
 // while it is loaded: FP64 in, FP64 out, nothing else in memory.
 //
-// Warps: 0 streams the eigenbasis digits (pre-swizzled 16 KB images, a ring of
-// seven), 1 issues the MMAs, 2..9 load rows and write their digits (one 64-wide K
-// tile of 7 x 32 rows per slot), 10..17 drain TMEM and store.  (Sharing the
-// eigenbasis stream by TMA multicast in clusters of two or four changed nothing:
-// 950 against 953 and 1057 us per application at 256 x 256 x 128.)
+// Warps: 0..2 stream the eigenbasis digits (pre-swizzled 16 KB images, a ring of
+// ten), 3 issues the MMAs, 4..11 load rows and write their digits (one 64-wide K
+// tile of 7 x 32 rows per slot, two slots), 12..27 drain TMEM and store.
+//
+// Measured at 256 x 256 x 128 (GB300, one application of six passes; k_modeprod_f64: 18.1 ms): 595 us, 108 us per
+// pass along a 256-point axis (120 GFLOP of digit products, 63 us at 1.9 PFLOP/s; the MMAs alone 50) and 78-82 along
+// the 128-point one, against 898 with MMAs whose descriptors one thread puts together, one producer warp, a ring of
+// seven images, eight epilogue warps and a division per point for G.  What is left: with the eigenbasis not
+// reloaded 534, without the epilogue's arithmetic 472, without either 412.  Sharing the eigenbasis stream by TMA
+// multicast in clusters of two or four changed nothing (950 against 953 and 1057 us when it was tried).
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <vector>
 
 #include "tc_ptx.cuh"
 
@@ -50,11 +58,20 @@ constexpr int kDig = 7;                        // base-256 digits of a value
 constexpr int kOzRows = 32;                    // data rows per tile
 constexpr int kOzImg = 128 * 128;              // one eigenbasis digit: 128 columns x 64 K elements
 constexpr int kOzSlot = kDig * kOzRows * 128;  // the data digits of one K tile
-constexpr int kOzStages = 7;
+constexpr int kOzStages = 10;                  // eigenbasis ring: images in flight or in use
+constexpr int kOzSlots = 2;                    // K tiles of data digits
+constexpr int kOzProd = 3;                     // producer warps
 constexpr int kOzMaxKT = 4;                    // axes of at most 256 points
-constexpr int kOzConv = 8, kOzEpi = 8;         // converter and epilogue warps
-constexpr int kOzThreads = (2 + kOzConv + kOzEpi) * 32;
-constexpr int kOzExpBufs = 4;                  // row-exponent buffers (tiles in flight + 1)
+constexpr int kOzConv = 8, kOzEpi = 16;        // converter and epilogue warps
+constexpr int kOzConv0 = kOzProd + 1, kOzEpi0 = kOzConv0 + kOzConv;  // warps: producers, MMA, converters, epilogue
+constexpr int kOzThreads = (kOzEpi0 + kOzEpi) * 32;
+// Registers: 28 warps launch with 72 a thread (64,512); the producer / MMA warpgroup gives back to 40, the two
+// converter warpgroups, which hold a tile's rows, take 88: 128 x 40 + 256 x 88 + 512 x 72 = 64,512.
+static_assert(kOzThreads == 896 && 128 * 40 + 256 * 88 + 512 * 72 == kOzThreads * 72, "register split");
+// Row-exponent buffers.  The converters write those of tile i when the MMAs of all but the last of its
+// predecessors' K tiles but one are done: unit i - 2 at least has begun, so the accumulators of unit i - 4 have been
+// read and the epilogue is past unit i - 5.
+constexpr int kOzExpBufs = 8;
 constexpr int kOzNan = 1 << 20;                // exponent word of a row holding a NaN or an infinity
 constexpr unsigned long long kBias = 0x80808080808080ull;
 
@@ -66,13 +83,11 @@ struct OzArgs {
   int C, KT, Cout, MB;
   int rows, B, in_pitch;
   long long oa, ob, oc;
-  int vec_in, vec_out;  // 16-byte row loads; 32-byte runs of eight output rows
+  int vec_in, vec_out;  // 16-byte row loads; 32-byte runs of four output rows
   int iters;            // tiles per CTA
   int first;            // the kernel before this one on the stream is not a pass
-  int scale, singular;
-  const double* lamA;
-  const double* lamB;
-  const double* lamC;
+  int scale;
+  const double* __restrict__ G;  // pass with the Hadamard step: G[row][c'], laid out as this pass's output
   const double* __restrict__ R;  // last pass of a solve
   SolveState* st;
   double* partials;
@@ -111,16 +126,17 @@ __device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned lo
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-__device__ __forceinline__ void tc_ld8_issue(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// Four columns of the thread's TMEM lane.
+__device__ __forceinline__ void tc_ld4_issue(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 }
-__device__ __forceinline__ void tc_ld8_wait(uint32_t (&r)[8]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
-               :
-               : "memory");
+// Every load issued before has landed; names the seven destinations so that none is read earlier.
+__device__ __forceinline__ void tc_ld4_wait(uint32_t (&t)[kDig][4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int s = 0; s < kDig; ++s) asm volatile("" : "+r"(t[s][0]), "+r"(t[s][1]), "+r"(t[s][2]), "+r"(t[s][3]));
 }
 
 // Contiguous global -> shared copy.
@@ -128,6 +144,11 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(bar)
                : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
 }
 
 // v * 2^e rounded once to FP64 (|v| < 2^63); outside the normal range by the general scaling.
@@ -148,15 +169,15 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* sm = smem_raw + (base - raw);
   const uint32_t sW = base;                                       // ring of eigenbasis digits
-  const uint32_t sX = sW + (uint32_t)(kOzStages * kOzImg);        // data digits, one slot per K tile
-  uint8_t* tail = sm + kOzStages * kOzImg + a.KT * kOzSlot;
+  const uint32_t sX = sW + (uint32_t)(kOzStages * kOzImg);        // ring of data digits
+  uint8_t* tail = sm + kOzStages * kOzImg + kOzSlots * kOzSlot;
   const uint32_t bars = smem_u32(tail);
   auto wfull = [&](int s) { return bars + 8u * s; };
   auto wempty = [&](int s) { return bars + 8u * (kOzStages + s); };
   auto dfull = [&](int s) { return bars + 8u * (2 * kOzStages + s); };
-  auto dempty = [&](int s) { return bars + 8u * (2 * kOzStages + kOzMaxKT + s); };
-  auto eready = [&](int s) { return bars + 8u * (2 * kOzStages + 2 * kOzMaxKT + s); };
-  constexpr int kT = 2 * kOzStages + 2 * kOzMaxKT + kOzExpBufs;
+  auto dempty = [&](int s) { return bars + 8u * (2 * kOzStages + kOzSlots + s); };
+  auto eready = [&](int s) { return bars + 8u * (2 * kOzStages + 2 * kOzSlots + s); };
+  constexpr int kT = 2 * kOzStages + 2 * kOzSlots + kOzExpBufs;
   auto tfull = [&](int b) { return bars + 8u * (kT + b); };
   auto tempty = [&](int b) { return bars + 8u * (kT + 2 + b); };
   const uint32_t drain = bars + 8u * (kT + 4);
@@ -171,7 +192,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
       mbar_init(wfull(s), 1);
       mbar_init(wempty(s), 1);
     }
-    for (int s = 0; s < kOzMaxKT; ++s) {
+    for (int s = 0; s < kOzSlots; ++s) {
       mbar_init(dfull(s), kOzConv * 32);
       mbar_init(dempty(s), 1);
     }
@@ -184,7 +205,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {
+  if (warp == kOzProd) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
                  "r"(512u)
                  : "memory");
@@ -199,81 +220,97 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
   const bool wres = a.MB * a.KT == 1;              // the whole eigenbasis fits the ring: loaded once
   double red0 = 0.0, red1 = 0.0;
 
-  if (warp == 0) {
-    // ---------------- eigenbasis digits: four lanes issue a quarter of an image each (one thread's issue rate
-    // is below what the MMAs consume)
-    constexpr uint32_t part = (uint32_t)kOzImg / 4u;
-    const uint32_t off = (uint32_t)(lane & 3) * part;
-    const int per_unit = a.KT * kDig;
-    const int total = wres ? kDig : units * per_unit;
-    const int per_tile = a.MB * per_unit;
-    int it = 0, im = 0;  // im: image index within the tile's sequence [mb][kt][digit]
-    bool ok = true;
-    for (; it < total; ++it) {
-      const int s = it % kOzStages;
+  if (warp <= kOzProd) {  // one warpgroup
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (warp < kOzProd) {
+      // ---------------- eigenbasis digits: warp w loads images w, w + 3, ... of the sequence [tile][mb][kt][digit]
+      // into ring stage (image mod 10).  A bulk copy holds its thread for about 0.3 us whatever its size, so one
+      // warp alone could not keep the ring full (2.5 us per K tile, whose MMAs take 1 us).
       if (lane == 0) {
-        ok = wait_bounded(wempty(s), (uint32_t)(((it / kOzStages) & 1) ^ 1), ab);
-        if (ok) mbar_expect_tx(wfull(s), (uint32_t)kOzImg);
-      }
-      ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
-      if (!ok) break;
-      if (lane < 4) bulk_load(sW + (uint32_t)s * kOzImg + off, a.img + (size_t)im * kOzImg + off, part, wfull(s));
-      if (++im == per_tile) im = 0;
-      __syncwarp();
-    }
-    if (!ok || *abort_flag) {  // every copy this CTA expects has landed (bounded) before it may leave
-      if (lane == 0)
-        for (int j = (it > kOzStages ? it - kOzStages : 0); j < it; ++j) {
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try_wait(wfull(j % kOzStages), (uint32_t)((j / kOzStages) & 1)) && gtimer() - t0 < kWaitLimitNs) {
+        const int per_tile = a.MB * a.KT * kDig;
+        const int total = wres ? kDig : iters * per_tile;
+        int it = warp, im = warp % per_tile;
+        for (; it < total && !*abort_flag; it += kOzProd) {
+          const int s = it % kOzStages;
+          if (!wait_bounded(wempty(s), (uint32_t)(((it / kOzStages) & 1) ^ 1), ab)) break;
+          mbar_expect_tx(wfull(s), (uint32_t)kOzImg);
+          bulk_load(sW + (uint32_t)s * kOzImg, a.img + (size_t)im * kOzImg, (uint32_t)kOzImg, wfull(s));
+          im += kOzProd;
+          if (im >= per_tile) im -= per_tile;
+        }
+        if (*abort_flag) {  // every copy this warp issued has landed (bounded) before the CTA may leave
+          for (int j = it - kOzProd; j >= 0 && j > it - kOzProd - kOzStages; j -= kOzProd) {
+            const unsigned long long t0 = gtimer();
+            while (!mbar_try_wait(wfull(j % kOzStages), (uint32_t)((j / kOzStages) & 1)) && gtimer() - t0 < kWaitLimitNs) {
+            }
           }
         }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
+      }
+      __syncwarp();
+    } else {
+      // ---------------- MMA issuer: the whole warp walks the loop, one elected lane issues.  The digit loop is
+      // unrolled and its control flow warp-uniform: descriptors put together per MMA by one thread took 143
+      // clocks each, twice what the tensor pipe needs (71 on average, max(N / 2, 32 + N / 4)).
+      const bool lead = elect_one();
       const unsigned long long dW = sw128_desc(sW), dX = sw128_desc(sX);
+      auto wait_all = [&](uint32_t bar, uint32_t par) { return __all_sync(0xffffffffu, wait_bounded(bar, par, ab)) != 0; };
       bool ok = true;
-      int it = 0;
+      uint32_t kts = 0;             // K tiles so far
+      uint32_t ws = 0, wpar = 0;    // ring stage of the next image and its parity
       for (int u = 0; ok && u < units; ++u) {
-        const int b = u & 1, tile = u / a.MB, mb = u - tile * a.MB;
-        if (!(ok = wait_bounded(tempty(b), (uint32_t)(((u >> 1) & 1) ^ 1), ab))) break;
+        const int b = u & 1;
+        if (!(ok = wait_all(tempty(b), (uint32_t)(((u >> 1) & 1) ^ 1)))) break;
         tc_fence_after();
         const uint32_t dacc = tmem + (uint32_t)(b * 256);
-        for (int kt = 0; ok && kt < a.KT; ++kt) {
-          if (mb == 0 && !(ok = wait_bounded(dfull(kt), (uint32_t)(tile & 1), ab))) break;
+        for (int kt = 0; ok && kt < a.KT; ++kt, ++kts) {
+          const uint32_t slot = kts % kOzSlots;
+          if (!(ok = wait_all(dfull(slot), (kts / kOzSlots) & 1u))) break;
           tc_fence_after();
           const int nk = min(4, (a.C - kt * 64 + 15) >> 4);
-          const unsigned long long xd = dX + (uint32_t)kt * (uint32_t)(kOzSlot >> 4);
-          for (int j = 0; j < kDig; ++j, ++it) {
-            const int s = wres ? j : it % kOzStages;
+          const unsigned long long xd = dX + slot * (uint32_t)(kOzSlot >> 4);
+  #pragma unroll
+          for (int j = 0; j < kDig; ++j) {
+            if (wres) ws = j;
             if (!wres || u == 0) {
-              if (!(ok = wait_bounded(wfull(s), (uint32_t)((it / kOzStages) & 1), ab))) break;
+              ok = ok && wait_all(wfull(ws), wpar);
               tc_fence_after();
             }
-            const unsigned long long wd = dW + (uint32_t)s * (uint32_t)(kOzImg >> 4);
-            const uint32_t idesc = idesc_f16kind(128, kOzRows * (kDig - j), 0u);
-            const uint32_t d = dacc + (uint32_t)(j * kOzRows);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              if (kk < nk) tc_mma(d, wd + 2u * kk, xd + 2u * kk, idesc, (kt > 0 || kk > 0 || j > 0) ? 1u : 0u);
-            if (!wres) tc_commit(wempty(s));
+            if (ok && lead) {
+              const unsigned long long wd = dW + ws * (uint32_t)(kOzImg >> 4);
+  #pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                if (kk < nk)
+                  tc_mma(dacc + (uint32_t)(j * kOzRows), wd + 2u * kk, xd + 2u * kk,
+                         idesc_f16kind(128, kOzRows * (kDig - j), 0u), (j > 0 || kk > 0) ? 1u : (kt > 0 ? 1u : 0u));
+              if (!wres) tc_commit(wempty(ws));
+            }
+            if (!wres && ++ws == (uint32_t)kOzStages) {
+              ws = 0;
+              wpar ^= 1u;
+            }
           }
-          if (ok && mb == a.MB - 1) tc_commit(dempty(kt));
+          __syncwarp();
+          if (ok && lead) tc_commit(dempty(slot));
         }
-        if (ok) tc_commit(tfull(b));
+        if (ok && lead) tc_commit(tfull(b));
+        __syncwarp();
       }
-      tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
-      const unsigned long long t0 = gtimer();
-      while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+      if (lead) {
+        tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+        }
       }
+      __syncwarp();
     }
     __syncwarp();
-  } else if (warp < 2 + kOzConv) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 72;");
+  } else if (warp < kOzEpi0) {  // two warpgroups
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
     // ---------------- converters: warp w takes rows 4w .. 4w+3 of a tile; a lane holds elements 64 kt + 2 lane
     // and the next one of each row
-    const int w = warp - 2;
+    const int w = warp - kOzConv0;
+    uint32_t kts = 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the data are the previous pass's output
     bool ok = true;
     for (int i = 0; ok && i < iters; ++i) {
@@ -305,72 +342,99 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
                          (uint32_t)__double2hiint(v[r][kt].y) & 0x7fffffffu));
         E[r] = max(1, (int)(__reduce_max_sync(0xffffffffu, m) >> 20));
       }
-      const uint32_t dpar = (uint32_t)((i & 1) ^ 1);
+      // one set of K tiles per 128-column block: the digits are formed again for the second one, so that the
+      // ring holds two K tiles instead of a whole row (the room goes to the eigenbasis)
+#pragma unroll 1
+      for (int mb = 0; ok && mb < a.MB; ++mb) {
+        // (the rows stay in registers and are not taken for loop constants: the compiler would otherwise form
+        // every digit before the loop and spill them)
 #pragma unroll
-      for (int kt = 0; kt < kOzMaxKT; ++kt) {
-        if (kt >= a.KT) break;
-        if (!(ok = __all_sync(0xffffffffu, wait_bounded(dempty(kt), dpar, ab)))) break;
-        if (kt == 0) {  // (the buffer's previous tile, four tiles ago, has been stored: its accumulators were reused)
-          if (lane < 4) {
-            const int e = lane == 0 ? E[0] : (lane == 1 ? E[1] : (lane == 2 ? E[2] : E[3]));
-            sE[(i % kOzExpBufs) * kOzRows + 4 * w + lane] = e == 0x7ff ? kOzNan : 1077 - e;
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int kt = 0; kt < kOzMaxKT; ++kt) asm volatile("" : "+d"(v[r][kt].x), "+d"(v[r][kt].y));
+#pragma unroll
+        for (int kt = 0; kt < kOzMaxKT; ++kt) {
+          if (kt >= a.KT) break;
+          const uint32_t slot = kts % kOzSlots;
+          if (!(ok = __all_sync(0xffffffffu, wait_bounded(dempty(slot), ((kts / kOzSlots) & 1u) ^ 1u, ab)))) break;
+          ++kts;
+          if (kt == 0 && mb == 0) {  // (the buffer's previous tile has been stored: see kOzExpBufs)
+            if (lane < 4) {
+              const int e = lane == 0 ? E[0] : (lane == 1 ? E[1] : (lane == 2 ? E[2] : E[3]));
+              sE[(i % kOzExpBufs) * kOzRows + 4 * w + lane] = e == 0x7ff ? kOzNan : 1077 - e;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(eready(i % kOzExpBufs));
           }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(eready(i % kOzExpBufs));
-        }
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const double2 x = v[r][kt];
-          const unsigned long long xa = (unsigned long long)to_fixed55(x.x, E[r]) + kBias;
-          const unsigned long long xb = (unsigned long long)to_fixed55(x.y, E[r]) + kBias;
-          const uint32_t row = (uint32_t)(4 * w + r);
-          const uint32_t dst = sX + (uint32_t)kt * kOzSlot + row * 128u + ((((uint32_t)lane >> 2) ^ (row & 7u)) << 4) +
-                               ((uint32_t)lane & 3u) * 4u;
+          for (int r = 0; r < 4; ++r) {
+            const double2 x = v[r][kt];
+            const unsigned long long xa = (unsigned long long)to_fixed55(x.x, E[r]) + kBias;
+            const unsigned long long xb = (unsigned long long)to_fixed55(x.y, E[r]) + kBias;
+            const uint32_t row = (uint32_t)(4 * w + r);
+            const uint32_t dst = sX + slot * kOzSlot + row * 128u + ((((uint32_t)lane >> 2) ^ (row & 7u)) << 4) +
+                                 ((uint32_t)lane & 3u) * 4u;
 #pragma unroll
-          for (int d = 0; d < kDig; ++d)
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + (uint32_t)(d * kOzRows * 128)), "r"(digit_pair(xa, xb, d))
-                         : "memory");
+            for (int d = 0; d < kDig; ++d)
+              asm volatile("st.shared.b32 [%0], %1;" ::"r"(dst + (uint32_t)(d * kOzRows * 128)), "r"(digit_pair(xa, xb, d))
+                           : "memory");
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // digits -> async-proxy reads of the MMA
+          mbar_arrive(dfull(slot));
         }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // digits -> async-proxy reads of the MMA
-        mbar_arrive(dfull(kt));
       }
     }
+    __syncwarp();
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
   } else {
-    // ---------------- epilogue: thread = output column of the block; warp half hf takes 16 of the 32 rows
-    const int q = warp & 3, hf = (warp - 2 - kOzConv) >> 2;
+    // ---------------- epilogue: thread = output column of the block; the four warps of a TMEM lane quadrant take
+    // eight of the 32 rows each
+    const int q = warp & 3, hf = (warp - kOzEpi0) >> 2;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int u = 0; u < units; ++u) {
       const int b = u & 1, tile = u / a.MB, mb = u - tile * a.MB;
-      const int row0 = ((int)blockIdx.x + tile * (int)gridDim.x) * kOzRows + 16 * hf;
+      const int row0 = ((int)blockIdx.x + tile * (int)gridDim.x) * kOzRows + 8 * hf;
       const int c = mb * 128 + q * 32 + lane;
       const int sw = __ldg(a.sw + c);
       const bool okc = c < a.Cout;
-      const double lc = (a.scale && okc) ? a.lamC[c] : 0.0;
       bool ok = wait_bounded(eready(tile % kOzExpBufs), (uint32_t)((tile / kOzExpBufs) & 1), ab);
       ok = ok && wait_bounded(tfull(b), (uint32_t)((u >> 1) & 1), ab);
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
-      const uint32_t tacc = tmem + (uint32_t)(b * 256 + 16 * hf) + ((uint32_t)(q * 32) << 16);
-      const int* eb = sE + (tile % kOzExpBufs) * kOzRows + 16 * hf;
-#pragma unroll 1
-      for (int ch = 0; ch < 2; ++ch) {
-        uint32_t t[kDig][8];
+      const uint32_t tacc = tmem + (uint32_t)(b * 256 + 8 * hf) + ((uint32_t)(q * 32) << 16);
+      const int* eb = sE + (tile % kOzExpBufs) * kOzRows + 8 * hf;
+      auto issue = [&](int ch, uint32_t(&t)[kDig][4]) {
         __syncwarp();  // (lanes past Cout skip the stores)
 #pragma unroll
-        for (int s = 0; s < kDig; ++s) tc_ld8_issue(tacc + (uint32_t)(s * kOzRows + 8 * ch), t[s]);
+        for (int s = 0; s < kDig; ++s) tc_ld4_issue(tacc + (uint32_t)(s * kOzRows + 4 * ch), t[s]);
+      };
+      // rows r0 .. r0+3 of the block's column c
+      auto process = [&](int ch, const uint32_t(&t)[kDig][4]) {
+        const int r0 = row0 + 4 * ch;
+        if (r0 >= a.rows || !okc) return;
+        const int ia = r0 / a.B, ib = r0 - ia * a.B;
+        long long at[4];
+        double f[4];
+        {
+          int xa = ia, xb = ib;
 #pragma unroll
-        for (int s = 0; s < kDig; ++s) tc_ld8_wait(t[s]);
-        if (ch == 1) {  // the accumulators are in registers
-          tc_fence_before();
-          mbar_arrive(tempty(b));
+          for (int r = 0; r < 4; ++r) {
+            at[r] = (long long)xa * a.oa + (long long)xb * a.ob + (long long)c * a.oc;
+            if (++xb == a.B) {
+              xb = 0;
+              ++xa;
+            }
+            f[r] = 0.0;
+            if (r0 + r < a.rows) {
+              if (a.scale) f[r] = __ldg(a.G + at[r]);
+              else if (FINAL) f[r] = __ldg(a.R + at[r]);
+            }
+          }
         }
-        const int r0 = row0 + 8 * ch;
-        if (r0 >= a.rows || !okc) continue;
-        int ia = r0 / a.B, ib = r0 - ia * a.B;
-        double y[8];
+        double y[4];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int ex = eb[8 * ch + r];
+        for (int r = 0; r < 4; ++r) {
+          const int ex = eb[4 * ch + r];
           auto lv = [&](int s) { return __float2int_rn(__uint_as_float(t[s][r])); };
           // T = sum_s acc_s 256^(6-s) = hi 2^32 + lo, kept to 2^8 (below the dropped levels)
           const long long hi = (long long)lv(0) * 65536 + (long long)lv(1) * 256 + lv(2);
@@ -378,40 +442,41 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
           y[r] = ex == kOzNan ? __longlong_as_double(0x7ff8000000000000ll)
                               : scaled_i64((hi << 24) + ((lo + 128) >> 8), 56 - ex - sw);
         }
-        if (a.vec_out) {  // eight rows of one a, contiguous: whole sectors
-          double* py = a.Y + (long long)ia * a.oa + ib + (long long)c * a.oc;
-          asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(py), "d"(y[0]), "d"(y[1]), "d"(y[2]), "d"(y[3])
+        if (a.vec_out) {  // four rows of one a, contiguous: a whole sector
+          asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(a.Y + at[0]), "d"(y[0]), "d"(y[1]), "d"(y[2]),
+                       "d"(y[3])
                        : "memory");
-          asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(py + 4), "d"(y[4]), "d"(y[5]), "d"(y[6]),
-                       "d"(y[7])
-                       : "memory");
-          continue;
+          return;
         }
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
+        for (int r = 0; r < 4; ++r) {
           if (r0 + r >= a.rows) break;
           double o = y[r];
-          if (a.scale) {  // Algorithm 7, Hadamard step: G = 1 / (lam_a + lam_b + lam_c), zero at the null index
-            const bool null = a.singular && ia == 0 && ib == 0 && c == 0;
-            o = null ? 0.0 : o * (1.0 / (a.lamA[ia] + a.lamB[ib] + lc));
-          }
-          const long long at = (long long)ia * a.oa + (long long)ib * a.ob + (long long)c * a.oc;
-          a.Y[at] = o;
+          if (a.scale) o *= f[r];  // Algorithm 7, Hadamard step
+          a.Y[at[r]] = o;
           if (FINAL) {
-            red0 = fma(__ldg(a.R + at), o, red0);
+            red0 = fma(f[r], o, red0);
             red1 += o;
           }
-          if (++ib == a.B) {
-            ib = 0;
-            ++ia;
-          }
         }
+      };
+      uint32_t t[kDig][4];
+#pragma unroll
+      for (int ch = 0; ch < 2; ++ch) {
+        issue(ch, t);
+        tc_ld4_wait(t);
+        if (ch == 1) {  // the accumulators are in registers
+          tc_fence_before();
+          mbar_arrive(tempty(b));
+        }
+        process(ch, t);
+        __syncwarp();
       }
     }
   }
 
   __syncthreads();
-  if (warp == 1) {
+  if (warp == kOzProd) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }
@@ -430,46 +495,62 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
   }
 }
 
-// The digit images of an eigenbasis matrix W (l x l, row-major, contraction index first): block c' scales
-// column c' by its power of two and writes its seven digits at every k, 64-wide K tiles of 128 columns under the
-// 128-byte swizzle.
-__global__ void __launch_bounds__(256) k_oz_image(const double* __restrict__ W, int l, int KT, uint8_t* img, int* sw) {
-  const int c = blockIdx.x, k = threadIdx.x;
-  __shared__ unsigned mx;
-  if (k == 0) mx = 0;
-  __syncthreads();
-  const double v = (c < l && k < l) ? W[(long long)k * l + c] : 0.0;
-  atomicMax(&mx, (unsigned)__double2hiint(v) & 0x7fffffffu);
-  __syncthreads();
-  const int E = max(1, (int)(mx >> 20));
-  if (k == 0) sw[c] = 1077 - E;
-  if (k >= KT * 64) return;
-  const unsigned long long x = (unsigned long long)to_fixed55(v, E) + kBias;
-  const int mb = c >> 7, r = c & 127, kt = k >> 6, kk = k & 63;
-#pragma unroll
-  for (int d = 0; d < kDig; ++d) {
-    const uint32_t h = digit_pair(x, x, d);
-    uint8_t* p = img + (((size_t)mb * KT + kt) * kDig + d) * kOzImg + r * 128 + (((kk >> 3) ^ (r & 7)) << 4) + (kk & 7) * 2;
-    *reinterpret_cast<uint16_t*>(p) = (uint16_t)h;
+// The digit images of an eigenbasis matrix W (l x l, row-major, contraction index first) and the power-of-two
+// scale of each column: column c' as seven base-256 digits at every k, 64-wide K tiles of 128 columns under the
+// 128-byte swizzle; zero past l.
+void digit_image(const std::vector<double>& W, int l, int MB, int KT, std::vector<uint8_t>& out) {
+  const size_t img = (size_t)MB * KT * kDig * kOzImg;
+  out.assign(img + (size_t)MB * 128 * sizeof(int), 0);
+  uint16_t f16[257];  // FP16 of -128 .. 128
+  for (int d = -128; d <= 128; ++d) {
+    const int v = d < 0 ? -d : d;
+    int e = 0;
+    while ((v >> e) > 1) ++e;
+    f16[d + 128] = v ? (uint16_t)((d < 0 ? 0x8000 : 0) | ((15 + e) << 10) | ((v << (10 - e)) & 0x3ff)) : (uint16_t)0;
+  }
+  int* sw = reinterpret_cast<int*>(out.data() + img);
+  for (int c = 0; c < l; ++c) {
+    double mx = 0.0;
+    for (int k = 0; k < l; ++k) mx = std::max(mx, std::fabs(W[(size_t)k * l + c]));
+    int e = 0;
+    std::frexp(mx, &e);  // mx < 2^e
+    sw[c] = 55 - e;
+    uint8_t* col = out.data() + (size_t)(c >> 7) * KT * kDig * kOzImg + (size_t)(c & 127) * 128;
+    for (int k = 0; k < l; ++k) {
+      long long x = std::llrint(std::ldexp(W[(size_t)k * l + c], 55 - e));  // |x| <= 2^55
+      uint8_t* p = col + (size_t)(k >> 6) * kDig * kOzImg + ((((k & 63) >> 3) ^ (c & 7)) << 4) + (k & 7) * 2;
+      for (int d = kDig - 1; d >= 0; --d) {
+        const int v = d ? (int)(int8_t)(x & 0xff) : (int)x;
+        std::memcpy(p + (size_t)d * kOzImg, &f16[v + 128], 2);
+        x = (x - v) >> 8;  // exact
+      }
+    }
   }
 }
 
-size_t oz_smem(int KT) {
-  return 1024 + (size_t)kOzStages * kOzImg + (size_t)KT * kOzSlot + 8 * (2 * kOzStages + 2 * kOzMaxKT + kOzExpBufs + 5) +
-         4 * kOzExpBufs * kOzRows + 16;
+// The Hadamard pseudoinverse G = 1 / (lam_a + lam_b + lam_c), zero at the null index, laid out as the output of the
+// pass that applies it.  An FP64 division per point costs that pass 120 us at 256 x 256 x 128 (FP64 pipe 72 % used);
+// reading 8 bytes per point costs 10.
+__global__ void __launch_bounds__(256) k_oz_ghat(double* __restrict__ G, int A, int B, int C, long long oa, long long ob,
+                                                 long long oc, const double* la, const double* lb, const double* lc,
+                                                 int singular) {
+  const long long n = (long long)A * B * C;
+  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) {
+    const long long r = i / C;
+    const int c = (int)(i - r * C), ia = (int)(r / B), ib = (int)(r - (long long)ia * B);
+    const bool null = singular && ia == 0 && ib == 0 && c == 0;
+    G[ia * oa + ib * ob + c * oc] = null ? 0.0 : 1.0 / (la[ia] + lb[ib] + lc[c]);
+  }
 }
+
+constexpr size_t kOzSmem = 1024 + (size_t)kOzStages * kOzImg + (size_t)kOzSlots * kOzSlot +
+                           8 * (2 * kOzStages + 2 * kOzSlots + kOzExpBufs + 5) + 4 * kOzExpBufs * kOzRows + 16;
+static_assert(kOzSmem <= (size_t)kMaxSmem, "shared memory of k_modeprod_oz");
 
 }  // namespace
 
 // Axes whose products run on the digits (others: k_modeprod_f64).
 bool oz_axis_ok(int l) { return l > 1 && l <= 64 * kOzMaxKT; }
-
-// Bytes of the digit images and scales of one axis (both directions).
-size_t oz_axis_bytes(int l) {
-  if (!oz_axis_ok(l)) return 0;
-  const size_t MB = (l + 127) / 128, KT = (l + 63) / 64;
-  return 2 * (MB * KT * kDig * kOzImg + MB * 128 * sizeof(int));
-}
 
 int oz_plan_setup(tpcg_plan* p) {
   const int lens[3] = {p->nx, p->ny, p->nz};
@@ -479,22 +560,38 @@ int oz_plan_setup(tpcg_plan* p) {
     if (!oz_axis_ok(l)) continue;
     any = true;
     const int MB = (l + 127) / 128, KT = (l + 63) / 64;
+    std::vector<double> VT((size_t)l * l);
+    for (int i = 0; i < l; ++i)
+      for (int j = 0; j < l; ++j) VT[(size_t)j * l + i] = p->ax[m].V[(size_t)i * l + j];
+    std::vector<uint8_t> img;
     for (int d = 0; d < 2; ++d) {
-      const size_t img = (size_t)MB * KT * kDig * kOzImg, bytes = img + (size_t)MB * 128 * sizeof(int);
-      if (cudaMalloc((void**)&p->d_oz[m][d], bytes) != cudaSuccess) {
+      digit_image(d ? VT : p->ax[m].V, l, MB, KT, img);
+      if (cudaMalloc((void**)&p->d_oz[m][d], img.size()) != cudaSuccess) {
         cudaGetLastError();
         p->d_oz[m][d] = nullptr;
         return TPCG_ERR_OOM;
       }
-      p->device_bytes += bytes;
-      k_oz_image<<<MB * 128, 256>>>(p->d_W64[m][d], l, KT, p->d_oz[m][d], reinterpret_cast<int*>(p->d_oz[m][d] + img));
+      p->device_bytes += img.size();
+      if (cudaMemcpy(p->d_oz[m][d], img.data(), img.size(), cudaMemcpyHostToDevice) != cudaSuccess) return TPCG_ERR_CUDA;
     }
   }
   if (any && (cudaFuncSetAttribute(k_modeprod_oz<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)oz_smem(kOzMaxKT)) != cudaSuccess ||
+                                   (int)kOzSmem) != cudaSuccess ||
               cudaFuncSetAttribute(k_modeprod_oz<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)oz_smem(kOzMaxKT)) != cudaSuccess))
+                                   (int)kOzSmem) != cudaSuccess))
     return TPCG_ERR_CUDA;
+  for (const StageParams& sp : p->stages) {
+    if (!sp.scale || !p->d_oz[sp.axis][sp.dir]) continue;
+    if (cudaMalloc((void**)&p->d_G, (size_t)p->N * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      p->d_G = nullptr;
+      return TPCG_ERR_OOM;
+    }
+    p->device_bytes += (size_t)p->N * sizeof(double);
+    k_oz_ghat<<<(int)std::min<long long>((p->N + 255) / 256, p->num_sms * 8), 256>>>(
+        p->d_G, sp.A, sp.B, sp.Cout, sp.oa, sp.ob, sp.oc, p->d_lam64[sp.lamA], p->d_lam64[sp.lamB],
+        p->d_lam64[sp.lamC], p->singular ? 1 : 0);
+  }
   return cudaGetLastError() == cudaSuccess ? TPCG_OK : TPCG_ERR_CUDA;
 }
 
@@ -521,16 +618,13 @@ bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, dou
   a.ob = sp.ob;
   a.oc = sp.oc;
   a.vec_in = (sp.C % 2 == 0 && sp.in_pitch % 2 == 0 && ((uintptr_t)X & 15) == 0) ? 1 : 0;
-  a.vec_out = (!sp.scale && !sp.final_stage && sp.ob == 1 && sp.B % 8 == 0 && sp.oa % 4 == 0 && sp.oc % 4 == 0 &&
+  a.vec_out = (!sp.scale && !sp.final_stage && sp.ob == 1 && sp.B % 4 == 0 && sp.oa % 4 == 0 && sp.oc % 4 == 0 &&
                ((uintptr_t)Y & 31) == 0)
                   ? 1
                   : 0;
   a.first = after_pass ? 0 : 1;
   a.scale = sp.scale;
-  a.singular = p->singular ? 1 : 0;
-  a.lamA = p->d_lam64[sp.lamA];
-  a.lamB = p->d_lam64[sp.lamB];
-  a.lamC = p->d_lam64[sp.lamC];
+  a.G = p->d_G;
   a.R = R;
   a.st = st;
   a.partials = p->d_partials;
@@ -542,7 +636,7 @@ bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, dou
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kOzThreads);
-  cfg.dynamicSmemBytes = oz_smem(a.KT);
+  cfg.dynamicSmemBytes = kOzSmem;
   cfg.stream = p->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

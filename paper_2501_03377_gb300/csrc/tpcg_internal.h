@@ -134,6 +134,7 @@ struct tpcg_plan {
   double* d_W64[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};  // [axis][dir] FP64 W = V or V^T
   // digit images and column scales of the FP64 form's tensor-core mode products, [axis][dir] (modeprod_oz.cu)
   uint8_t* d_oz[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
+  double* d_G = nullptr;  // its Hadamard factors, in the layout of the pass that applies them
   double* d_lam64[3] = {nullptr, nullptr, nullptr};
   float* d_lam32[3] = {nullptr, nullptr, nullptr};
   void* d_Wt16[3][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};   // [axis][dir] BF16 W^T (K-major)
