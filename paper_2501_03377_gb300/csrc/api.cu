@@ -18,11 +18,11 @@ namespace tpcg {
 void launch_apply_laplacian(const tpcg_plan* p, const Geom& g, const double* x, double* w);
 void launch_init_residual(const tpcg_plan* p, const Geom& g, const double* eta, const double* U, bool zero_guess);
 void launch_eta_sum(const tpcg_plan* p, const Geom& g, const double* eta, const double* U0);
-void launch_direction(const tpcg_plan* p, const Geom& g, int k);
-void launch_update(const tpcg_plan* p, const Geom& g, double* U, int k, bool zero_guess_first);
+void launch_direction(const tpcg_plan* p, const Geom& g);
+void launch_update(const tpcg_plan* p, const Geom& g, double* U, bool zero_guess_first);
 void launch_true_residual(const tpcg_plan* p, const Geom& g, const double* eta, const double* U, bool force);
 void launch_form_u(const tpcg_plan* p, const Geom& g, double* U, bool force);
-void launch_center_u(const tpcg_plan* p, const Geom& g, double* U, int iter_lo);
+void launch_center_u(const tpcg_plan* p, const Geom& g, double* U, bool force);
 void launch_zero(const tpcg_plan* p, long long N, double* U);
 void launch_to_lp(const tpcg_plan* p, const Geom& g, const double* r);
 void launch_norm_shift(const tpcg_plan* p, const Geom& g, const double* r);
@@ -282,21 +282,34 @@ int enqueue_state_readback(tpcg_plan* p) {
   return last_cuda_error();
 }
 
-// The launches of `count` iterations starting at j.issued.
+// The launches of `count` iterations starting at j.issued.  A chunk ends with one check of the true residual: the
+// iterations after the one whose recurrence met the tolerance return at once (paused()), so the check sees the
+// iterate it would have seen directly behind that iteration, and neither the checks of the other iterations nor the
+// application of the preconditioner behind a last one are launched (a launch that returns at once still takes 2.3 us:
+// at 64 x 64 x 32 they were 8 of a solve's 35).  An application is due before every iteration but the first, whose
+// Z the set-up formed.  The comparators' kernels run unconditionally: check and application behind every iteration.
 int launch_iterations(SolveJob& j, int count) {
   tpcg_plan* p = j.p;
   const Geom g = make_geom(p);
+  const bool cmp = p->pc_kind != TPCG_PRECOND_PINV;
   for (int c = 0; c < count; ++c) {
-    const int k = j.issued + c;                         // P_k is written to d_P[k & 1], P_{k-1} read from the other
-    launch_direction(p, g, k);                          // direction P, W = L P, alpha
-    launch_update(p, g, j.ups, k, k == 0 && (j.flags & TPCG_ZERO_GUESS));  // U and R updates
-    if (p->defer_u) launch_form_u(p, g, j.ups, false);  // deferred U updates, when a check is due
-    launch_true_residual(p, g, j.eta, j.ups, false);    // stop test
-    const int rc = run_precond(p, p->d_R, p->d_Z, p->d_state);  // Z = M R, rho, beta
-    if (rc) return rc;
+    const int k = j.issued + c;
+    if (!cmp && k > 0) {
+      const int rc = run_precond(p, p->d_R, p->d_Z, p->d_state);  // Z = M R, rho, beta
+      if (rc) return rc;
+    }
+    launch_direction(p, g);                             // direction P, W = L P, alpha
+    launch_update(p, g, j.ups, k == 0 && (j.flags & TPCG_ZERO_GUESS));  // U and R updates
+    if (p->defer_u) launch_form_u(p, g, j.ups, false);  // deferred U updates, when a check is due or the ring is full
+    if (cmp) {
+      launch_true_residual(p, g, j.eta, j.ups, false);  // stop test
+      const int rc = run_precond(p, p->d_R, p->d_Z, p->d_state);
+      if (rc) return rc;
+    }
   }
+  if (!cmp) launch_true_residual(p, g, j.eta, j.ups, false);  // stop test
   // singular operators: centre U on the device if the stop test succeeded inside this chunk
-  if (p->singular) launch_center_u(p, g, j.ups, j.issued);
+  if (p->singular) launch_center_u(p, g, j.ups, false);
   return TPCG_OK;
 }
 
@@ -356,7 +369,7 @@ unsigned graph_flags(const SolveJob& j) {
 // convergence return at once
 int enqueue_iterations(SolveJob& j, int count) {
   tpcg_plan* p = j.p;
-  const int rc = run_graphed(p, GraphKey{1, j.issued, count, graph_flags(j), p->graph_gen},
+  const int rc = run_graphed(p, GraphKey{1, j.issued > 0 ? 1 : 0, count, graph_flags(j), p->graph_gen},
                              [&]() { return launch_iterations(j, count); });
   if (rc) return rc;
   j.issued += count;
@@ -417,6 +430,7 @@ int job_step(SolveJob& j) {
   SolveState* hs = p->h_state;
   if (cudaEventSynchronize(p->ev_state) != cudaSuccess) return last_cuda_error() ? TPCG_ERR_CUDA : TPCG_ERR_CUDA;
   if (j.phase == 1) {
+    j.issued = hs->iter;  // iterations that paused behind a check count for nothing
     if (!hs->done && j.issued <= j.maxit + 1) {
       int rc = enqueue_iterations(j, j.chunk);
       if (rc) return rc;
@@ -438,7 +452,7 @@ int job_step(SolveJob& j) {
           launch_true_residual(p, g, j.eta, j.ups, true);  // report the true residual of the returned iterate
           if (!hs->done) j.status_host = TPCG_ERR_NOT_CONVERGED;
         }
-        if (p->singular) launch_center_u(p, g, j.ups, -1);
+        if (p->singular) launch_center_u(p, g, j.ups, true);
       }
       return enqueue_state_readback(p);
     }

@@ -492,8 +492,8 @@ __global__ void __launch_bounds__(TX* TY) k_residual_fx(Geom g, const double* __
   stencil_sweep_fx<long long, 4>(
       g, f, op, partials, &st->tickets[INIT ? kTkInit : kTkTrue],
       [st, force, N, sr, ku, finite_u](const double(&s)[4]) {
-        const double rr = finite_u ? ldexp(s[0], -2 * sr) : __longlong_as_double(0x7ff8000000000000ll);
-        const double sumR = ldexp(s[1], -sr), sumU = ldexp(s[2], 8 - ku);
+        const double rr = finite_u ? scale_pow2(s[0], -2 * sr) : __longlong_as_double(0x7ff8000000000000ll);
+        const double sumR = scale_pow2(s[1], -sr), sumU = scale_pow2(s[2], 8 - ku);
         if (!INIT) st->checks += 1;
         if (INIT) {
           const double v[3] = {rr, sumR, s[3]};
@@ -535,14 +535,25 @@ __device__ void fin_direction(SolveState* st, const double (&s)[1], const Geom& 
 }
 
 __global__ void __launch_bounds__(TX* TY) k_direction(Geom g, int zchunk, const double* __restrict__ Z,
-                                                      const double* __restrict__ Pold, double* __restrict__ P,
+                                                      double* __restrict__ P0, double* __restrict__ P1,
                                                       double* __restrict__ W, SolveState* st, double* partials) {
-  if (st->done) return;
+  if (paused(st)) return;
+  double* P = (st->iter & 1) ? P1 : P0;  // P_s in buffer s & 1
+  const double* Pold = (st->iter & 1) ? P0 : P1;
   FieldDirection f{Z, Pold, st->mZ, st->beta, st->first};
   OpDirection op{P, W};
   stencil_sweep<1>(g, zchunk, f, op, partials, &st->tickets[kTkDir],
                    [st, g](const double(&s)[1]) { fin_direction(st, s, g); });
 }
+
+// Storage of the directions: P_s is in slot s % slots.  The kernels take s from the state (iterations completed): the
+// host's count runs ahead of it when an iteration pauses (paused()).
+struct DirRing {
+  int* base;
+  unsigned long long stride;  // grid points
+  int slots;
+  __device__ __forceinline__ int* at(int s) const { return base + (unsigned long long)(s % slots) * stride; }
+};
 
 // ------------------------------------------------------------------ direction, mixed forms
 // Z arrives in FP32.  The direction is stored as exact fixed point
@@ -586,10 +597,10 @@ __device__ __forceinline__ void for_each_run(const Geom& g, Run run) {
   }
 }
 
-__global__ void __launch_bounds__(TX* TY) k_direction_int(Geom g, const float* __restrict__ Z,
-                                                          const int* __restrict__ Pold, int* __restrict__ P,
-                                                          SolveState* st, double* partials) {
-  if (st->done) return;
+__global__ void __launch_bounds__(TX* TY) k_direction_int(Geom g, const float* __restrict__ Z, DirRing ring, SolveState* st, double* partials) {
+  if (paused(st)) return;
+  int* __restrict__ P = ring.at(st->iter);
+  const int* __restrict__ Pold = ring.at(st->iter + ring.slots - 1);
   const int kp = st->kp_next;
   const float sc = (kp >= -126 && kp <= 127) ? __int_as_float((kp + 127) << 23) : 0.0f;  // 2^kp
   const float bs = st->bs_next;  // beta_s 2^-kp_{s-1} (0 for the first direction)
@@ -668,8 +679,8 @@ __global__ void __launch_bounds__(TX* TY) k_direction_int(Geom g, const float* _
   const int nblocks = gridDim.x;
   grid_reduce<1>(acc, partials, &st->tickets[kTkDir], nblocks, blockIdx.x, [st, kp, g](const double(&s)[1]) {
     st->kp = kp;
-    st->pmax = ldexp((double)atomicExch(&st->pmax_bits, 0u), -kp);
-    const double v[1] = {ldexp(s[0], -2 * kp)};
+    st->pmax = scale_pow2((double)atomicExch(&st->pmax_bits, 0u), -kp);
+    const double v[1] = {scale_pow2(s[0], -2 * kp)};
     fin_direction(st, v, g);
   });
 }
@@ -677,10 +688,10 @@ __global__ void __launch_bounds__(TX* TY) k_direction_int(Geom g, const float* _
 // The same direction with two adjacent x points per thread (even nx): Z and
 // P_old as 8-byte pairs, P stored as int2; the left neighbour of a pair's
 // first point comes from the previous lane (lane 0: the tile's halo column).
-__global__ void __launch_bounds__(TX* TY) k_direction_pair(Geom g, const float* __restrict__ Z,
-                                                           const int* __restrict__ Pold, int* __restrict__ P,
-                                                           SolveState* st, double* partials) {
-  if (st->done) return;
+__global__ void __launch_bounds__(TX* TY) k_direction_pair(Geom g, const float* __restrict__ Z, DirRing ring, SolveState* st, double* partials) {
+  if (paused(st)) return;
+  int* __restrict__ P = ring.at(st->iter);
+  const int* __restrict__ Pold = ring.at(st->iter + ring.slots - 1);
   const int kp = st->kp_next;
   const float sc = (kp >= -126 && kp <= 127) ? __int_as_float((kp + 127) << 23) : 0.0f;  // 2^kp
   const float bs = st->bs_next;  // beta_s 2^-kp_{s-1} (0 for the first direction)
@@ -769,8 +780,8 @@ __global__ void __launch_bounds__(TX* TY) k_direction_pair(Geom g, const float* 
   if (threadIdx.x + threadIdx.y == 0) atomicMax(&st->pmax_bits, (unsigned)m);
   grid_reduce<1>(acc, partials, &st->tickets[kTkDir], gridDim.x, blockIdx.x, [st, kp, g](const double(&s)[1]) {
     st->kp = kp;
-    st->pmax = ldexp((double)atomicExch(&st->pmax_bits, 0u), -kp);
-    const double v[1] = {ldexp(s[0], -2 * kp)};
+    st->pmax = scale_pow2((double)atomicExch(&st->pmax_bits, 0u), -kp);
+    const double v[1] = {scale_pow2(s[0], -2 * kp)};
     fin_direction(st, v, g);
   });
 }
@@ -780,10 +791,10 @@ __global__ void __launch_bounds__(TX* TY) k_direction_pair(Geom g, const float* 
 // quad's first point comes from the previous lane (lane 0: the tile's halo
 // column).  Loads, address arithmetic and loop control are shared by four
 // points instead of two.
-__global__ void __launch_bounds__(TX* TY) k_direction_quad(Geom g, const float* __restrict__ Z,
-                                                           const int* __restrict__ Pold, int* __restrict__ P,
-                                                           SolveState* st, double* partials) {
-  if (st->done) return;
+__global__ void __launch_bounds__(TX* TY) k_direction_quad(Geom g, const float* __restrict__ Z, DirRing ring, SolveState* st, double* partials) {
+  if (paused(st)) return;
+  int* __restrict__ P = ring.at(st->iter);
+  const int* __restrict__ Pold = ring.at(st->iter + ring.slots - 1);
   const int kp = st->kp_next;
   const float sc = (kp >= -126 && kp <= 127) ? __int_as_float((kp + 127) << 23) : 0.0f;  // 2^kp
   const float bs = st->bs_next;  // beta_s 2^-kp_{s-1} (0 for the first direction)
@@ -890,8 +901,8 @@ __global__ void __launch_bounds__(TX* TY) k_direction_quad(Geom g, const float* 
   if (threadIdx.x + threadIdx.y == 0) atomicMax(&st->pmax_bits, (unsigned)m);
   grid_reduce<1>(acc, partials, &st->tickets[kTkDir], gridDim.x, blockIdx.x, [st, kp, g](const double(&s)[1]) {
     st->kp = kp;
-    st->pmax = ldexp((double)atomicExch(&st->pmax_bits, 0u), -kp);
-    const double v[1] = {ldexp(s[0], -2 * kp)};
+    st->pmax = scale_pow2((double)atomicExch(&st->pmax_bits, 0u), -kp);
+    const double v[1] = {scale_pow2(s[0], -2 * kp)};
     fin_direction(st, v, g);
   });
 }
@@ -906,7 +917,7 @@ __global__ void __launch_bounds__(TX* TY) k_direction_quad(Geom g, const float* 
 // pslot >= 0 (mixed forms): U was not touched; record alpha_s, the exponent of P_s and its ring slot for
 // k_form_u.  pslot < 0 (FP64 form): U was updated; take max|U| for the residual check.
 __device__ void fin_update(SolveState* st, const double (&s)[2], int shift, const Geom& g, int pslot) {
-  const double rr = ldexp(s[0], -2 * shift), sumR = ldexp(s[1], -shift);
+  const double rr = scale_pow2(s[0], -2 * shift), sumR = scale_pow2(s[1], -shift);
   st->rr = rr;
   st->sumR = sumR;
   st->iter += 1;
@@ -934,9 +945,11 @@ __device__ void fin_update(SolveState* st, const double (&s)[2], int shift, cons
 // integer stencil of P_int, in a register-window stream (see k_direction_int).  The loads of plane k+1
 // (P two planes ahead, the y neighbours and R) are issued before plane k is processed.  U += alpha P is
 // not applied: the finalize records it for k_form_u (P_s stays in ring slot pslot until then).
-__global__ void __launch_bounds__(TX* TY, 4) k_update_int(Geom g, const int* __restrict__ P, double* __restrict__ R,
-                                                          LowPrec lp, SolveState* st, double* partials, int pslot) {
-  if (st->done) return;
+__global__ void __launch_bounds__(TX* TY, 4) k_update_int(Geom g, DirRing ring, double* __restrict__ R,
+                                                          LowPrec lp, SolveState* st, double* partials) {
+  if (paused(st)) return;
+  const int pslot = st->iter % ring.slots;
+  const int* __restrict__ P = ring.at(st->iter);
   const double na0 = st->nah[0], na1 = st->nah[1], na2 = st->nah[2];  // -alpha / h^2 per axis
   const int kp = st->kp;
   const int shift = st->lp_shift;
@@ -1026,9 +1039,11 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_int(Geom g, const int* __r
 // as 16-byte double2, P and its y neighbours as int2, the FP16 copy as one
 // packed pair; only the outer x neighbours of a pair come by warp shuffle.
 // A warp covers 64 consecutive x of one row.
-__global__ void __launch_bounds__(TX* TY, 4) k_update_pair(Geom g, const int* __restrict__ P, double* __restrict__ R,
-                                                           LowPrec lp, SolveState* st, double* partials, int pslot) {
-  if (st->done) return;
+__global__ void __launch_bounds__(TX* TY, 4) k_update_pair(Geom g, DirRing ring, double* __restrict__ R,
+                                                           LowPrec lp, SolveState* st, double* partials) {
+  if (paused(st)) return;
+  const int pslot = st->iter % ring.slots;
+  const int* __restrict__ P = ring.at(st->iter);
   const double na0 = st->nah[0], na1 = st->nah[1], na2 = st->nah[2];  // -alpha / h^2 per axis
   const int kp = st->kp;
   const int shift = st->lp_shift;
@@ -1131,9 +1146,10 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_pair(Geom g, const int* __
 // ZG: the first update of a zero initial guess writes U = alpha P.
 template <bool ZG>
 __global__ void __launch_bounds__(TX* TY, 4) k_update_u_int(Geom g, double* __restrict__ U,
-                                                          const int* __restrict__ P, double* __restrict__ R,
+                                                          DirRing ring, double* __restrict__ R,
                                                           LowPrec lp, SolveState* st, double* partials) {
-  if (st->done) return;
+  if (paused(st)) return;
+  const int* __restrict__ P = ring.at(st->iter);
   // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
   U = st->ups;
   const double alpha = st->alpha;
@@ -1236,9 +1252,10 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_int(Geom g, double* __re
 // A warp covers 64 consecutive x of one row.
 template <bool ZG>
 __global__ void __launch_bounds__(TX* TY, 4) k_update_u_pair(Geom g, double* __restrict__ U,
-                                                           const int* __restrict__ P, double* __restrict__ R,
+                                                           DirRing ring, double* __restrict__ R,
                                                            LowPrec lp, SolveState* st, double* partials) {
-  if (st->done) return;
+  if (paused(st)) return;
+  const int* __restrict__ P = ring.at(st->iter);
   // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
   U = st->ups;
   const double alpha = st->alpha;
@@ -1349,11 +1366,12 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_pair(Geom g, double* __r
 }
 
 // FP64 form: P and W = L P are stored by the direction kernel.
-__global__ void __launch_bounds__(256) k_update(Geom g, double* __restrict__ U, const double* __restrict__ P,
-                                                const double* __restrict__ W, double* __restrict__ R, LowPrec lp,
-                                                SolveState* st, double* partials) {
+__global__ void __launch_bounds__(256) k_update(Geom g, double* __restrict__ U, const double* __restrict__ P0,
+                                                const double* __restrict__ P1, const double* __restrict__ W,
+                                                double* __restrict__ R, LowPrec lp, SolveState* st, double* partials) {
   const long long N = g.N;
-  if (st->done) return;
+  if (paused(st)) return;
+  const double* __restrict__ P = (st->iter & 1) ? P1 : P0;
   // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
   U = st->ups;
   const double alpha = st->alpha;
@@ -1404,7 +1422,7 @@ __global__ void __launch_bounds__(256) k_init_zero(long long N, const double* __
   }
   double acc[2] = {e2, f32_to_f64_int(a1)};
   grid_reduce<2>(acc, partials, &st->tickets[kTkInit], gridDim.x, blockIdx.x, [st, N, shift](const double(&s)[2]) {
-    const double v[3] = {s[0], ldexp(s[1], -shift), s[0]};
+    const double v[3] = {s[0], scale_pow2(s[1], -shift), s[0]};
     fin_init(st, v, N);
   });
 }
@@ -1543,7 +1561,7 @@ __global__ void __launch_bounds__(256) k_init_zero2(unsigned npair, long long N,
   }
   double acc[2] = {e2, f32_to_f64_int(a1)};
   grid_reduce<2>(acc, partials, &st->tickets[kTkInit], gridDim.x, blockIdx.x, [st, N, shift](const double(&s)[2]) {
-    const double v[3] = {s[0], ldexp(s[1], -shift), s[0]};
+    const double v[3] = {s[0], scale_pow2(s[1], -shift), s[0]};
     fin_init(st, v, N);
   });
 }
@@ -1593,14 +1611,13 @@ __global__ void __launch_bounds__(256) k_norm_shift(long long N, const double* _
                  [st, N](const double(&s)[1]) { st->lp_shift = lp_shift_for(s[0], N); });
 }
 
-// U -= sum(U)/N: return the zero-mean (minimum-norm) representative.  With
-// iter_lo >= 0 only when the solve converged in an iteration after iter_lo:
-// launched behind each chunk of iterations, it centres U in the chunk where
-// the stop test succeeded (every block takes the same decision: done_iter is
-// set once) and saves the host a round trip.
+// U -= sum(U)/N: return the zero-mean (minimum-norm) representative.  Without
+// `force` only when the stop test has succeeded: launched behind each chunk of
+// iterations, it centres U in the chunk where that happened (the host issues no
+// further one; every block takes the same decision) and saves the host a round trip.
 __global__ void __launch_bounds__(256) k_center_u(long long N, double* __restrict__ U, const SolveState* st,
-                                                  int iter_lo) {
-  if (iter_lo >= 0 && !(st->done == 1 && st->status == TPCG_OK && st->done_iter > iter_lo)) return;
+                                                  int force) {
+  if (!force && !(st->done == 1 && st->status == TPCG_OK && st->done_iter > 0)) return;
   // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
   U = st->ups;
   const double m = st->sumU / (double)N;
@@ -1831,57 +1848,52 @@ void launch_norm_shift(const tpcg_plan* p, const Geom& g, const double* r) {
   LaunchScope ls(p, kKConvert);
   k_norm_shift<<<p->stream_blocks, 256, 0, p->stream>>>(g.N, r, p->d_state, p->d_partials);
 }
-// FP64 form: P_k is written to d_P[k & 1], P_{k-1} read from the other buffer.  Mixed forms: P_k goes to
-// ring slot k % p_slots (with TPCG_OPT_DEFER_U, kept there until k_form_u has applied alpha_k P_k to U).
-void launch_direction(const tpcg_plan* p, const Geom& g, int k) {
+static DirRing dir_ring(const tpcg_plan* p) {
+  return DirRing{(int*)p->d_P[0], (unsigned long long)p->N, p->p_slots};
+}
+// FP64 form: P_s is in d_P[s & 1].  Mixed forms: in ring slot s % p_slots (with TPCG_OPT_DEFER_U, kept there until
+// k_form_u has applied alpha_s P_s to U).
+void launch_direction(const tpcg_plan* p, const Geom& g) {
   LaunchScope ls(p, kKDirection);
   if (p->prec == TPCG_FP64) {
-    k_direction<<<p->st_grid, p->st_block, 0, p->stream>>>(
-        g, p->st_zchunk, (const double*)p->d_Z, (const double*)p->d_P[(k + 1) & 1], (double*)p->d_P[k & 1], p->d_W,
-        p->d_state, p->d_partials);
+    k_direction<<<p->st_grid, p->st_block, 0, p->stream>>>(g, p->st_zchunk, (const double*)p->d_Z, (double*)p->d_P[0],
+                                                            (double*)p->d_P[1], p->d_W, p->d_state, p->d_partials);
     return;
   }
-  const int ns = p->p_slots;
-  const int* Pold = (const int*)p->d_P[(k + ns - 1) % ns];
-  int* Pnew = (int*)p->d_P[k % ns];
+  const DirRing ring = dir_ring(p);
+  const float* Z = (const float*)p->d_Z;
+  const int blocks = p->fx_blocks[kFxDir];
   if (g.nx % 4 == 0)
-    k_direction_quad<<<p->fx_blocks[kFxDir], p->st_block, 0, p->stream>>>(g, (const float*)p->d_Z, Pold, Pnew,
-                                                                           p->d_state, p->d_partials);
+    k_direction_quad<<<blocks, p->st_block, 0, p->stream>>>(g, Z, ring, p->d_state, p->d_partials);
   else if (g.nx % 2 == 0)
-    k_direction_pair<<<p->fx_blocks[kFxDir], p->st_block, 0, p->stream>>>(g, (const float*)p->d_Z, Pold, Pnew,
-                                                                           p->d_state, p->d_partials);
+    k_direction_pair<<<blocks, p->st_block, 0, p->stream>>>(g, Z, ring, p->d_state, p->d_partials);
   else
-    k_direction_int<<<p->fx_blocks[kFxDir], p->st_block, 0, p->stream>>>(g, (const float*)p->d_Z, Pold, Pnew,
-                                                                          p->d_state, p->d_partials);
+    k_direction_int<<<blocks, p->st_block, 0, p->stream>>>(g, Z, ring, p->d_state, p->d_partials);
 }
-void launch_update(const tpcg_plan* p, const Geom& g, double* U, int k, bool zero_guess_first) {
+// zero_guess_first: the first update of a zero initial guess, U = alpha P
+void launch_update(const tpcg_plan* p, const Geom& g, double* U, bool zero_guess_first) {
   LaunchScope ls(p, kKUpdate);
   if (p->prec == TPCG_FP64) {
-    k_update<<<p->stream_blocks, 256, 0, p->stream>>>(g, U, (const double*)p->d_P[k & 1], p->d_W, p->d_R,
-                                                       lowprec(p), p->d_state, p->d_partials);
+    k_update<<<p->stream_blocks, 256, 0, p->stream>>>(g, U, (const double*)p->d_P[0], (const double*)p->d_P[1], p->d_W,
+                                                       p->d_R, lowprec(p), p->d_state, p->d_partials);
     return;
   }
-  const int slot = k % p->p_slots;
-  const int* P = (const int*)p->d_P[slot];
+  const DirRing ring = dir_ring(p);
+  const int blocks = p->fx_blocks[kFxUpd];
+  const LowPrec lp = lowprec(p);
   if (p->defer_u) {  // U += alpha P recorded for k_form_u
     if (g.nx % 2 == 0)
-      k_update_pair<<<p->fx_blocks[kFxUpd], p->st_block, 0, p->stream>>>(g, P, p->d_R, lowprec(p), p->d_state,
-                                                                          p->d_partials, slot);
+      k_update_pair<<<blocks, p->st_block, 0, p->stream>>>(g, ring, p->d_R, lp, p->d_state, p->d_partials);
     else
-      k_update_int<<<p->fx_blocks[kFxUpd], p->st_block, 0, p->stream>>>(g, P, p->d_R, lowprec(p), p->d_state,
-                                                                         p->d_partials, slot);
-  } else if (g.nx % 2 == 0 && aligned16(U) && zero_guess_first) {  // first update of a zero guess: U = alpha P
-    k_update_u_pair<true><<<p->fx_blocks[kFxUpd], p->st_block, 0, p->stream>>>(g, U, P, p->d_R, lowprec(p),
-                                                                                p->d_state, p->d_partials);
+      k_update_int<<<blocks, p->st_block, 0, p->stream>>>(g, ring, p->d_R, lp, p->d_state, p->d_partials);
+  } else if (g.nx % 2 == 0 && aligned16(U) && zero_guess_first) {
+    k_update_u_pair<true><<<blocks, p->st_block, 0, p->stream>>>(g, U, ring, p->d_R, lp, p->d_state, p->d_partials);
   } else if (g.nx % 2 == 0 && aligned16(U)) {
-    k_update_u_pair<false><<<p->fx_blocks[kFxUpd], p->st_block, 0, p->stream>>>(g, U, P, p->d_R, lowprec(p),
-                                                                                 p->d_state, p->d_partials);
+    k_update_u_pair<false><<<blocks, p->st_block, 0, p->stream>>>(g, U, ring, p->d_R, lp, p->d_state, p->d_partials);
   } else if (zero_guess_first) {
-    k_update_u_int<true><<<p->fx_blocks[kFxUpd], p->st_block, 0, p->stream>>>(g, U, P, p->d_R, lowprec(p),
-                                                                               p->d_state, p->d_partials);
+    k_update_u_int<true><<<blocks, p->st_block, 0, p->stream>>>(g, U, ring, p->d_R, lp, p->d_state, p->d_partials);
   } else {
-    k_update_u_int<false><<<p->fx_blocks[kFxUpd], p->st_block, 0, p->stream>>>(g, U, P, p->d_R, lowprec(p),
-                                                                                p->d_state, p->d_partials);
+    k_update_u_int<false><<<blocks, p->st_block, 0, p->stream>>>(g, U, ring, p->d_R, lp, p->d_state, p->d_partials);
   }
 }
 // Mixed forms: apply the recorded updates to U (k_form_u) when a check is due, the ring is about to wrap,
@@ -1900,9 +1912,9 @@ void launch_true_residual(const tpcg_plan* p, const Geom& g, const double* eta, 
   k_residual_fx<false><<<p->fx_blocks[kFxTrue], p->st_block, 0, p->stream>>>(g, eta, U, p->d_R, lowprec(p),
                                                                               p->d_state, p->d_partials, force ? 1 : 0);
 }
-void launch_center_u(const tpcg_plan* p, const Geom& g, double* U, int iter_lo) {
+void launch_center_u(const tpcg_plan* p, const Geom& g, double* U, bool force) {
   LaunchScope ls(p, kKCenter);
-  k_center_u<<<p->stream_blocks, 256, 0, p->stream>>>(g.N, U, p->d_state, iter_lo);
+  k_center_u<<<p->stream_blocks, 256, 0, p->stream>>>(g.N, U, p->d_state, force ? 1 : 0);
 }
 void launch_zero(const tpcg_plan* p, long long N, double* U) {
   LaunchScope ls(p, kKConvert);

@@ -41,7 +41,7 @@ struct ModeArgsF64 {
 
 template <bool FINAL>
 __global__ void __launch_bounds__(256) k_modeprod_f64(ModeArgsF64 a) {
-  if (a.st && a.st->done) return;
+  if (a.st && paused(a.st)) return;
   __shared__ double As[KT][MT + 2];
   __shared__ double Bs[KT][NT];
   const StageParams& p = a.p;

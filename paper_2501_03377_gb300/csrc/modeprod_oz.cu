@@ -160,7 +160,7 @@ __device__ __forceinline__ double scaled_i64(long long v, int e) {
 template <bool FINAL>
 __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
   if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
-  if (a.st && a.st->done) return;  // (uniform over the grid)
+  if (a.st && paused(a.st)) return;  // (uniform over the grid)
   // Programmatic dependent launch: the next pass sets up on SMs this grid has left and waits
   // (griddepcontrol.wait) before it touches this pass's output.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

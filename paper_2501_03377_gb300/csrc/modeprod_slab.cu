@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
     k_frontal_pair(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmA1,
                    const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmO, SlabArgs a) {
   if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
-  if (a.st && a.st->done) return;
+  if (a.st && paused(a.st)) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
     grid_reduce<2>(acc, a.partials, &st->tickets[kTkPrec], gridDim.x, blockIdx.x,
                    [st, N, shR](const double(&s)[2]) {
                      st->zmax = __uint_as_float(atomicExch(&st->zmax_bits, 0u));
-                     const double v[2] = {ldexp(s[0], -shR), s[1]};
+                     const double v[2] = {scale_pow2(s[0], -shR), s[1]};
                      if (!st->timeout) {
                        fin_precond(st, N, v);
                        plan_next_direction(st);
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
     k_tube_pair(const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmW1,
                 const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmO, SlabArgs a) {
   if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
-  if (a.st && a.st->done) return;
+  if (a.st && paused(a.st)) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     k_modeprod_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                   const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmO, TcArgs a) {
   if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
-  if (a.st && a.st->done) return;
+  if (a.st && paused(a.st)) return;
   // Programmatic dependent launch: the next pass may start its prologue (barriers, TMEM, eigenbasis
   // load) on SMs this grid frees; it waits (griddepcontrol.wait) before touching this pass's output.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     grid_reduce<2>(acc, a.partials, &st->tickets[kTkPrec], gridDim.x, blockIdx.x,
                    [st, N, shR](const double(&s)[2]) {
                      st->zmax = __uint_as_float(atomicExch(&st->zmax_bits, 0u));
-                     const double v[2] = {ldexp(s[0], -shR), s[1]};
+                     const double v[2] = {scale_pow2(s[0], -shR), s[1]};
                      if (!st->timeout) {
                        fin_precond(st, N, v);
                        plan_next_direction(st);
@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     k_modeprod_pair(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW1,
                     const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmO, TcArgs a) {
   if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
-  if (a.st && a.st->done) return;
+  if (a.st && paused(a.st)) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -1048,7 +1048,7 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
     k_modeprod_pair_split(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW1,
                           const __grid_constant__ CUtensorMap tmW2, TcArgs a) {
   if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
-  if (a.st && a.st->done) return;
+  if (a.st && paused(a.st)) return;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);

@@ -68,6 +68,10 @@ struct SolveState {
 
 enum Ticket { kTkEta = 0, kTkInit = 1, kTkDir = 2, kTkUpd = 3, kTkTrue = 4, kTkPrec = 5, kTkMisc = 6, kTkForm = 7 };
 
+// Nothing to do for the kernels of the recurrence and the preconditioner: the solve is over, or the recurrence has
+// met the tolerance and the true-residual check at the end of the host's chunk of iterations decides what follows.
+__device__ __forceinline__ bool paused(const SolveState* st) { return st->done || st->need_check; }
+
 // Geometry of a grid and its stencil (eq. lap1d / eq. ourproblem).
 struct Geom {
   int nx, ny, nz;
@@ -112,31 +116,64 @@ struct LaunchScope {
   }
 };
 
-// Block-wide sum of NQ doubles; result valid in thread 0.  Fixed order: the
-// result is bitwise reproducible for a fixed launch configuration.
+// Sum over the warp of NQ doubles (a power of two), quantity q in the lanes of group q (32 / NQ lanes each): the
+// first steps halve the quantities a lane carries instead of the lanes, so NQ = 2 takes five FP64 additions a lane
+// and NQ = 4 six, instead of ten and twenty (a warp's addition occupies the FP64 pipe for 16 clocks).
 template <int NQ>
-__device__ __forceinline__ void block_sum(double (&v)[NQ], double* sh /* NQ*32 doubles */) {
+__device__ __forceinline__ double warp_sum_packed(const double (&v)[NQ], int lane) {
+  static_assert(NQ == 1 || NQ == 2 || NQ == 4, "packed by halves");
+  double x;
+  int o = 16;
+  if constexpr (NQ == 4) {
+    const bool up = (lane & 16) != 0;
+    double a = up ? v[2] : v[0], b = up ? v[3] : v[1];
+    a += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 16);
+    b += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 16);
+    const bool up8 = (lane & 8) != 0;
+    x = up8 ? b : a;
+    x += __shfl_xor_sync(0xffffffffu, up8 ? a : b, 8);
+    o = 4;
+  } else if constexpr (NQ == 2) {
+    const bool up = (lane & 16) != 0;
+    x = up ? v[1] : v[0];
+    x += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 16);
+    o = 8;
+  } else {
+    x = v[0];
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+
+// Block-wide sum of NQ doubles; result valid in warp 0.  Fixed order: the
+// result is bitwise reproducible for a fixed launch configuration.  `any` (uniform over a warp): the warp's values
+// may be non-zero.
+template <int NQ>
+__device__ __forceinline__ void block_sum(double (&v)[NQ], double* sh /* NQ*32 doubles */, bool any = true) {
+  constexpr int kG = 32 / NQ;
   const int lane = threadIdx.x & 31;
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int warp = tid >> 5;
   const int nthreads = blockDim.x * blockDim.y * blockDim.z;
   const int nwarps = (nthreads + 31) >> 5;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    double x = v[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if (lane == 0) sh[q * 32 + warp] = x;
-  }
+  const double x = any ? warp_sum_packed<NQ>(v, lane) : 0.0;
+  if (lane % kG == 0) sh[(lane / kG) * 32 + warp] = x;
   __syncthreads();
   if (warp == 0) {
+    double y;
+    if (nwarps <= kG) {  // the warps' sums of a quantity fit its lane group
+      y = (lane % kG) < nwarps ? sh[(lane / kG) * 32 + lane % kG] : 0.0;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-      double x = (lane < nwarps) ? sh[q * 32 + lane] : 0.0;
+      for (int o = kG / 2; o > 0; o >>= 1)
+        if (o < nwarps) y += __shfl_xor_sync(0xffffffffu, y, o);
+    } else {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      v[q] = x;
+      for (int q = 0; q < NQ; ++q) v[q] = (lane < nwarps) ? sh[q * 32 + lane] : 0.0;
+      y = warp_sum_packed<NQ>(v, lane);
     }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] = __shfl_sync(0xffffffffu, y, q * kG);
   }
   __syncthreads();
 }
@@ -169,7 +206,7 @@ __device__ __forceinline__ void grid_reduce(double (&v)[NQ], double* partials, u
 #pragma unroll
     for (int q = 0; q < NQ; ++q) s[q] += __ldcg(&partials[(size_t)b * NQ + q]);
   }
-  block_sum<NQ>(s, sh);
+  block_sum<NQ>(s, sh, (tid & ~31) < nblocks);
   if (tid == 0) {
     fin(s);
     *ticket = 0u;
@@ -268,12 +305,28 @@ __device__ __forceinline__ uint16_t f64_to_f16_bits(double x, int shift) {
   return (uint16_t)(sign | bits);
 }
 
+// The scalar work of a finalize runs in one thread on a pipe whose division, square root and ldexp take hundreds of
+// clocks each, at the end of every reducing kernel: exponents are taken from the bit pattern instead.
+
+// x * 2^k (one rounding, as ldexp).
+__device__ __forceinline__ double scale_pow2(double x, int k) {
+  return (k > -1000 && k < 1000) ? x * __hiloint2double((1023 + k) << 20, 0) : ldexp(x, k);
+}
+// floor(log2 x) of a finite x > 0.
+__device__ __forceinline__ int ilogb_pos(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e ? e - 1023 : ilogb(x);
+}
+
 // Exponent s with rms * 2^s in [0.5, 1) for the FP16 copy of a vector of
-// squared 2-norm n2 and length N (0 when the vector is zero).
+// squared 2-norm n2 and length N <= 2^31 (0 when the vector is zero).  The quotient n2 / N is formed in FP32.
 __device__ __forceinline__ int lp_shift_for(double n2, long long N) {
   if (!(n2 > 0.0) || !isfinite(n2)) return 0;
-  const double rms = sqrt(n2 / (double)N);
-  int s = -ilogb(rms) - 1;
+  const int e = ilogb_pos(n2);
+  const unsigned long long m = (unsigned long long)__double_as_longlong(scale_pow2(n2, -e));  // [1, 2)
+  const float q = __uint_as_float(0x3f800000u | ((uint32_t)(m >> 29) & 0x7fffffu)) / (float)(unsigned)N;
+  const int eq = e + (int)(__float_as_uint(q) >> 23) - 127;  // floor(log2(n2 / N))
+  const int s = -(eq >> 1) - 1;
   return s < -120 ? -120 : (s > 120 ? 120 : s);
 }
 
@@ -317,7 +370,7 @@ __device__ __forceinline__ double i32_to_f64_scaled(int v, int e) {
 // magic-number rule below, and every 7-point stencil fits in 24 bits.
 __device__ __forceinline__ int fixed_shift_for(double bound) {
   if (!(bound > 0.0) || !isfinite(bound)) return 0;
-  const int k = 19 - ilogb(bound);
+  const int k = 19 - ilogb_pos(bound);
   return k < -900 ? -900 : (k > 900 ? 900 : k);
 }
 
@@ -366,7 +419,7 @@ __device__ __forceinline__ uint16_t f32_to_bf16_bits_rn(float v) {
 // result an FP64 normal number.
 __device__ __forceinline__ int fixed64_shift_for(double umax) {
   if (!(umax > 0.0) || !isfinite(umax)) return 0;
-  const int k = 57 - ilogb(umax);
+  const int k = 57 - ilogb_pos(umax);
   return k < -960 ? -960 : (k > 960 ? 960 : k);
 }
 
@@ -455,18 +508,20 @@ __device__ __forceinline__ double f32_to_f64_int(float f) {
 __device__ __forceinline__ void plan_next_direction(SolveState* st) {
   const double bound = (double)st->zmax + (st->first ? 0.0 : fabs(st->beta) * st->pmax);
   st->kp_next = fixed_shift_for(bound);
-  st->bs_next = st->first ? 0.0f : (float)ldexp(st->beta, -st->kp);
+  st->bs_next = st->first ? 0.0f : (float)scale_pow2(st->beta, -st->kp);
 }
 
 // Scales of the next fixed-point residual check, from max|U| and ||eta_hat||:
-// |eta_hat - L U| <= ||eta_hat|| + 12 max(1/h^2) max|U| entrywise.  Set by
-// the finalize that last changed U (or measured U_0), read by the check.
+// |eta_hat - L U| <= ||eta_hat|| + 12 max(1/h^2) max|U| entrywise, bounded by powers of two (2^-sr only has to keep the
+// check's FP32 sums in range).  Set by the finalize that last changed U (or measured U_0), read by the check.
 __device__ __forceinline__ void plan_residual_check(SolveState* st, const Geom& g) {
-  const double umax = st->umax;
+  const double umax = st->umax, n2 = st->eta_norm2;
   st->ku = fixed64_shift_for(umax);
-  const double ihmax = fmax(g.ih2[0], fmax(g.ih2[1], g.ih2[2]));
-  const double bound = 2.0 * (sqrt(fmax(st->eta_norm2, 0.0)) + 12.0 * ihmax * umax);
-  st->sr = (bound > 0.0 && isfinite(bound)) ? -ilogb(bound) : 0;
+  const int ih = max(__double2hiint(g.ih2[0]), max(__double2hiint(g.ih2[1]), __double2hiint(g.ih2[2]))) >> 20;
+  int eb = -4000;
+  if (n2 > 0.0) eb = (ilogb_pos(n2) >> 1) + 1;                                  // sqrt(n2) < 2^eb
+  if (umax > 0.0) eb = max(eb, ilogb_pos(umax) + 1 + (ih - 1023) + 1 + 4);      // 12 ih umax < 2^..
+  st->sr = (eb > -4000 && isfinite(umax) && isfinite(n2)) ? -(eb + 2) : 0;
 }
 
 // Value of a compensated FP32 sum in FP64.

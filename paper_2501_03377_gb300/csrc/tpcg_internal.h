@@ -91,7 +91,7 @@ struct SolveJob {
   tpcg_info info{};
 };
 // A launch sequence of a solve captured as a CUDA graph: the set-up (what = 0) or a chunk of `count`
-// iterations starting at iteration k0 (what = 1); flags: zero initial guess and the 16-byte alignment of
+// iterations (what = 1), the first (k0 = 0) or a later one (k0 = 1: it begins with the preconditioner); flags: zero initial guess and the 16-byte alignment of
 // the caller's arrays (they choose kernel variants); gen: the plan's option generation.
 struct GraphKey {
   int what, k0, count;
