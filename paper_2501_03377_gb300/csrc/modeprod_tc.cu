@@ -95,6 +95,7 @@ struct TcArgs {
   int rtma;  // last pass: R~ arrives by TMA, else by global loads
   int rhalf;   // R~ ring slots per epilogue half (last pass, rtma)
   int tstore;  // outputs leave through shared memory by TMA stores (tmO), else by direct stores
+  int stg;     // direct stores of unaligned runs: transposed within half warps (odd extents)
   int tperm;   // form 2 output map: dims {B, A, Cout} (1) or {B, Cout, A} (0)
   int aux;     // bytes of shared memory after the stages: R~ ring (last pass) and output staging
   int wstream;  // eigenbasis K tiles streamed with the data tiles (each stage holds both), else resident
@@ -191,7 +192,74 @@ __device__ __forceinline__ void store16(void* out, long long plane, long long o,
   }
 }
 
-template <int FORM, class InT, class OutT, bool FINAL>
+// The bits of one output as a 32-bit word (split form: hi in the low half, lo in the high half) and its store.
+template <class OutT>
+__device__ __forceinline__ uint32_t out_word(float v) {
+  if constexpr (std::is_same<OutT, Bf16Pair>::value) {
+    const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
+    return (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16);
+  } else if constexpr (std::is_same<OutT, __half>::value) {
+    return (uint32_t)__half_as_ushort(__float2half_rn(v));
+  } else if constexpr (sizeof(OutT) == 2) {
+    return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v));
+  } else {
+    return __float_as_uint(v);
+  }
+}
+template <class OutT>
+__device__ __forceinline__ void store_word(void* out, long long plane, long long o, uint32_t w) {
+  if constexpr (std::is_same<OutT, Bf16Pair>::value) {
+    reinterpret_cast<uint16_t*>(out)[o] = (uint16_t)w;
+    reinterpret_cast<uint16_t*>(out)[plane + o] = (uint16_t)(w >> 16);
+  } else if constexpr (sizeof(OutT) == 2) {
+    reinterpret_cast<uint16_t*>(out)[o] = (uint16_t)w;
+  } else {
+    reinterpret_cast<uint32_t*>(out)[o] = w;
+  }
+}
+
+// Transposes the [16 lanes][16] words of each half warp: afterwards word i of a lane is element lane % 16 of lane i of
+// its half.  Used where an extent is not a multiple of 8, so that a thread's 16 outputs are contiguous but not
+// aligned: stored from their thread, element by element, every store instruction touches 32 sectors; transposed,
+// sixteen lanes write one run and it touches two to four.
+__device__ __forceinline__ void half_warp_transpose16(int lane, uint32_t (&w)[16]) {
+  __syncwarp();
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) {
+    const bool up = (lane & d) != 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i & d) continue;
+      const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? w[i] : w[i | d], d);
+      if (up) w[i] = got;
+      else w[i | d] = got;
+    }
+  }
+}
+
+// Sixteen consecutive rows r0.. of output index cb + lane (all lanes of the warp), form 2, stored by runs along the rows.
+template <class OutT>
+__device__ __forceinline__ void store_rows_transposed(const TcArgs& a, int lane, int cb, int r0, const float (&v)[16]) {
+  uint32_t w[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) w[i] = out_word<OutT>(v[i]);
+  half_warp_transpose16(lane, w);
+  const int rr = r0 + (lane & 15);
+  if (rr < a.rows) {
+    const int xa = rr / a.B, xb = rr - xa * a.B;
+    const int cc = cb + (lane & 16);
+    const long long o = (long long)xa * a.oa + (long long)xb * a.ob + (long long)cc * a.oc;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (cc + i < a.Cout) store_word<OutT>(a.out, a.oplane, o + (long long)i * a.oc, w[i]);
+  }
+  __syncwarp();
+}
+
+// ODD: unaligned runs of outputs (TcArgs::stg), stored transposed; an instantiation of its own, since its code costs
+// the aligned one registers (the 256 x 256 x 128 solve took 1 % longer with both in one kernel).
+template <int FORM, class InT, class OutT, bool FINAL, bool ODD>
 __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     k_modeprod_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                   const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmO, TcArgs a) {
@@ -496,7 +564,7 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
           }
         };
         auto process = [&](int c0, const uint32_t (&t)[16], const uint4 (&rcur)[2]) {
-          if (!valid && !a.tstore) return;
+          if (!valid && !a.tstore && !ODD) return;
           float v[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(t[i]);
@@ -519,7 +587,18 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = tf32_rn(v[j]);
           }
-          if (a.tstore) emit(v, c0, row0 + q * 32, 0);  // rows past `rows`, columns past Cout: clipped
+          if (!ODD && a.tstore) emit(v, c0, row0 + q * 32, 0);  // rows past `rows`, columns past Cout: clipped
+          if constexpr (ODD) {  // the rows follow one another (oa = B ob): sixteen lanes write the columns of one row
+            uint32_t w[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) w[i] = out_word<OutT>(v[i]);
+            half_warp_transpose16(lane, w);
+            const int cc = c0 + (lane & 15), rr = row0 + q * 32 + (lane & 16);
+            if (cc < a.Cout)
+#pragma unroll
+              for (int i = 0; i < 16; ++i)
+                if (rr + i < a.rows) store_word<OutT>(a.out, a.oplane, (long long)(rr + i) * a.ob + cc, w[i]);
+          }
           if (!valid) return;
           if (vec && c0 + 16 <= a.Cout) {
             if (!a.tstore) store16<OutT>(a.out, a.oplane, obase + c0, v);
@@ -571,20 +650,59 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
                        (((v[8] + v[9]) + (v[10] + v[11])) + ((v[12] + v[13]) + (v[14] + v[15]))));
             }
           } else {
+            float rv[16];
+            if constexpr (FINAL) {  // R~, its rows padded to a multiple of 8 elements: by 16-byte pieces inside the pitch
+              const long long ro = (long long)r * a.rpitch + c0;
+              if (ODD && c0 + 16 <= a.rpitch) {
+                if constexpr (KS::tf32) {
+                  const float4* rp = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(a.Rt) + ro);
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) {
+                    const float4 x = __ldg(rp + i);
+                    rv[4 * i] = x.x, rv[4 * i + 1] = x.y, rv[4 * i + 2] = x.z, rv[4 * i + 3] = x.w;
+                  }
+                } else {
+                  const uint4* hp = reinterpret_cast<const uint4*>(a.Rt + ro);
+                  const uint4 h0 = __ldg(hp), h1 = __ldg(hp + 1);
+                  const uint32_t hw[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+                  using LpT = typename std::conditional<KS::split, __nv_bfloat16, InT>::type;
+#pragma unroll
+                  for (int i = 0; i < 8; ++i) {
+                    const float2 x = lp2_to_f32<LpT>(hw[i]);
+                    rv[2 * i] = x.x, rv[2 * i + 1] = x.y;
+                  }
+                  if constexpr (KS::split) {
+                    const uint4* lq = reinterpret_cast<const uint4*>(Rlo + ro);
+                    const uint4 l0 = __ldg(lq), l1 = __ldg(lq + 1);
+                    const uint32_t lw[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                      const float2 x = lp2_to_f32<__nv_bfloat16>(lw[i]);
+                      rv[2 * i] += x.x, rv[2 * i + 1] += x.y;
+                    }
+                  }
+                }
+              } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                  rv[j] = 0.0f;
+                  if (c0 + j < a.Cout) {
+                    if constexpr (KS::tf32) rv[j] = __ldg(reinterpret_cast<const float*>(a.Rt) + ro + j);
+                    else if constexpr (KS::split)
+                      rv[j] = lp2_to_f32<__nv_bfloat16>(__ldg(a.Rt + ro + j)).x +
+                              lp2_to_f32<__nv_bfloat16>(__ldg(Rlo + ro + j)).x;
+                    else rv[j] = lp2_to_f32<InT>(__ldg(a.Rt + ro + j)).x;
+                  }
+                }
+              }
+            }
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const int c = c0 + j;
               if (c < a.Cout) {
-                const long long o = obase + (long long)c * a.oc;
-                if (!a.tstore) store_out<OutT>(a.out, a.oplane, o, v[j]);
+                if (!a.tstore && !ODD) store_out<OutT>(a.out, a.oplane, obase + (long long)c * a.oc, v[j]);
                 if (FINAL) {
-                  float rv;
-                  if constexpr (KS::tf32) rv = __ldg(reinterpret_cast<const float*>(a.Rt) + (long long)r * a.rpitch + c);
-                  else if constexpr (KS::split)
-                    rv = lp2_to_f32<__nv_bfloat16>(__ldg(a.Rt + (long long)r * a.rpitch + c)).x +
-                         lp2_to_f32<__nv_bfloat16>(__ldg(Rlo + (long long)r * a.rpitch + c)).x;
-                  else rv = lp2_to_f32<InT>(__ldg(a.Rt + (long long)r * a.rpitch + c)).x;
-                  red0.add(rv * rs * v[j]);
+                  red0.add(rv[j] * rs * v[j]);
                   red1.add(v[j]);
                   zmax = fmaxf(zmax, fabsf(v[j]));
                 }
@@ -642,9 +760,13 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
           for (int i = 0; i < 16; ++i) v[i] = KS::tf32 ? tf32_rn(__uint_as_float(t[i])) : __uint_as_float(t[i]);
           int ia = r0 / a.B;
           int ib = r0 - ia * a.B;
-          if (a.tstore) {  // B % 16 == 0: the 16 rows share one a; output indices past Cout are clipped
+          if (!ODD && a.tstore) {  // B % 16 == 0: the 16 rows share one a; output indices past Cout are clipped
             if (a.tperm) emit(v, ib, ia, cb);
             else emit(v, ib, cb, ia);
+            return;
+          }
+          if constexpr (ODD) {  // sixteen lanes write the rows of one output index
+            store_rows_transposed<OutT>(a, lane, cb, r0, v);
             return;
           }
           if (c >= a.Cout) return;
@@ -1298,10 +1420,15 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
       const int c = q * 32 + lane;
       auto out = [&](int c0, const uint32_t (&t)[16]) {
         const int r0 = row0 + c0;
-        if (r0 >= a.rows || c >= a.Cout) return;
+        if (r0 >= a.rows) return;  // warp-uniform
         float v[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(t[k]);
+        if (a.stg) {
+          store_rows_transposed<Bf16Pair>(a, lane, q * 32, r0, v);
+          return;
+        }
+        if (c >= a.Cout) return;
         int ia = r0 / a.B;
         int ib = r0 - ia * a.B;
         if (a.vec && ib + 16 <= a.B && r0 + 16 <= a.rows) {
@@ -1463,8 +1590,10 @@ int encode_pair(CUtensorMap* map, const void* gaddr, int inner, long long outer,
 
 template <int FORM, class InT, class OutT, bool FINAL>
 int set_smem_attr(size_t smem) {
-  return cudaFuncSetAttribute(k_modeprod_tc<FORM, InT, OutT, FINAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem) == cudaSuccess
+  return (cudaFuncSetAttribute(k_modeprod_tc<FORM, InT, OutT, FINAL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)smem) == cudaSuccess &&
+          cudaFuncSetAttribute(k_modeprod_tc<FORM, InT, OutT, FINAL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)smem) == cudaSuccess)
              ? 0
              : -1;
 }
@@ -1515,7 +1644,8 @@ void launch(const TcStage& s, const TcArgs& a, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_modeprod_tc<FORM, InT, OutT, FINAL>, s.tmX, s.tmW, s.tmR, s.tmO, a);
+  if (a.stg) cudaLaunchKernelEx(&cfg, k_modeprod_tc<FORM, InT, OutT, FINAL, true>, s.tmX, s.tmW, s.tmR, s.tmO, a);
+  else cudaLaunchKernelEx(&cfg, k_modeprod_tc<FORM, InT, OutT, FINAL, false>, s.tmX, s.tmW, s.tmR, s.tmO, a);
 }
 
 template <class InT>
@@ -1695,6 +1825,9 @@ int tc_plan_setup(tpcg_plan* p) {
       a.tstore = 0;
       a.aux = 2 * a.rhalf * kRBytes;
     }
+    // direct stores of runs that no 16-byte store fits (an extent that is not a multiple of 8): at 255 x 201 x 97 in
+    // the split form such a pass took 95 us, element by element from each thread
+    a.stg = (!a.tstore && !a.vec && (st.form == 2 || (sp.oa == (long long)sp.B * sp.ob || sp.A == 1))) ? 1 : 0;
     fixed += (size_t)a.aux;
     a.NS = (int)std::min<size_t>(8, (kMaxSmem - fixed) / sbytes);
     st.smem = fixed + (size_t)a.NS * sbytes;
