@@ -685,14 +685,6 @@ int tpcg_plan_create(int nx, int ny, int nz, const int bc[3], const double h[3],
   // launch configuration, fixed per plan (reproducible reductions)
   if (!rc) {
     p->st_block = dim3(32, 8, 1);
-    const int bx = (nx + 31) / 32, by = (ny + 7) / 8;
-    const int target = p->num_sms * 6;
-    int zsplit = std::max(1, std::min(nz, (target + bx * by - 1) / (bx * by)));
-    int zchunk = (nz + zsplit - 1) / zsplit;
-    zsplit = (nz + zchunk - 1) / zchunk;
-    p->st_grid = dim3(bx, by, zsplit);
-    p->st_zchunk = zchunk;
-    if ((size_t)bx * by * zsplit * 4 > p->partial_slots) rc = TPCG_ERR_UNSUPPORTED;
     if (!rc && setup_fx_grids(p)) rc = TPCG_ERR_CUDA;
     for (int i = 0; i < kFxCount && !rc; ++i)
       if ((size_t)p->fx_blocks[i] * 4 > p->partial_slots) rc = TPCG_ERR_UNSUPPORTED;

@@ -4,14 +4,14 @@
 // and the deterministic reductions that produce alpha, beta and the stop test
 // on the device.
 //
-// Stencil scheme: a block owns a 32 x 8 tile of (x, y) columns and marches
-// along z through a chunk of planes.  Each plane of the field, with a one-point
-// halo in x and y, is staged in a 4-slot shared-memory ring, so the z
-// neighbours come from the ring as well and every field value is loaded (and,
-// for the direction kernel, formed) once per tile.  Boundary conditions enter
-// only through the halo ("ghost") values: periodic wraps, Dirichlet reads 0,
-// Neumann mirrors the boundary value -- which reproduces the corner entries
-// (alpha, beta, gamma) of eq. (lap1d) exactly.
+// Stencil scheme (stencil_sweep_fx): a block walks runs of planes of 32 x 8
+// tiles of (x, y) columns.  Each plane of the field, with a one-point halo in x
+// and y, is staged in a shared-memory ring, so the z neighbours come from the
+// ring as well and every field value is loaded (and, for the direction kernel,
+// formed) once per tile.  Boundary conditions enter only through the halo
+// ("ghost") values: periodic wraps, Dirichlet reads 0, Neumann mirrors the
+// boundary value -- which reproduces the corner entries (alpha, beta, gamma) of
+// eq. (lap1d) exactly.
 #include <cstdio>
 
 #include "tpcg_dev.cuh"
@@ -36,117 +36,6 @@ __device__ __forceinline__ int ghost_index(int g, int n, int bc) {
     return -1;
   }
   return -1;
-}
-
-// ------------------------------------------------------------------ fields
-struct FieldPlain {  // the stencil is applied to x itself
-  const double* __restrict__ x;
-  __device__ __forceinline__ double operator()(long long i) const { return __ldg(x + i); }
-};
-
-struct FieldDirection {  // FP64 form: P = (Z - mean Z) + beta * P_old   (Algorithm 1; Remark orthogonality)
-  const double* __restrict__ z;
-  const double* __restrict__ pold;
-  double mZ, beta;
-  int first;
-  __device__ __forceinline__ double operator()(long long i) const {
-    const double zi = __ldg(z + i) - mZ;
-    return first ? zi : fma(beta, __ldg(pold + i), zi);
-  }
-};
-
-// ------------------------------------------------------------------ stencil driver
-// Calls op(idx, c, w, acc) for every grid point, where c is the field value
-// and w = (L field)(point).  Accumulates NQ sums and finishes with fin().
-template <int NQ, class Field, class Op, class Fin>
-__device__ __forceinline__ void stencil_sweep(const Geom& g, int zchunk, const Field& field, Op& op, double* partials,
-                                              unsigned* ticket, Fin fin) {
-  __shared__ double ring[4][SY][SX];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int tid = ty * TX + tx;
-  const int bx0 = blockIdx.x * TX, by0 = blockIdx.y * TY;
-  const int x = bx0 + tx, y = by0 + ty;
-  const int k0 = blockIdx.z * zchunk;
-  const int k1 = min(g.nz, k0 + zchunk);
-  const bool active = (x < g.nx) && (y < g.ny);
-  const bool has_z = g.nz > 1;
-  const long long plane = (long long)g.nx * g.ny;
-  double acc[NQ > 0 ? NQ : 1];
-#pragma unroll
-  for (int q = 0; q < (NQ > 0 ? NQ : 1); ++q) acc[q] = 0.0;
-
-  auto load_plane = [&](int kk) {
-    const int kz = has_z ? ghost_index(kk, g.nz, g.bc[2]) : kk;
-    double(*dst)[SX] = ring[kk & 3];
-    for (int e = tid; e < SX * SY; e += TX * TY) {
-      const int sx = e % SX, sy = e / SX;
-      const int gx = ghost_index(bx0 + sx - 1, g.nx, g.bc[0]);
-      const int gy = ghost_index(by0 + sy - 1, g.ny, g.bc[1]);
-      double v = 0.0;
-      if (kz >= 0 && gx >= 0 && gy >= 0 && bx0 + sx - 1 <= g.nx && by0 + sy - 1 <= g.ny)
-        v = field((long long)kz * plane + (long long)gy * g.nx + gx);
-      dst[sy][sx] = v;
-    }
-  };
-
-  if (k0 < k1) {
-    if (has_z) load_plane(k0 - 1);
-    load_plane(k0);
-    const double ihx = g.ih2[0], ihy = g.ih2[1], ihz = g.ih2[2];
-    const bool uniform = (ihx == ihy) && (!has_z || ihz == ihx);
-    for (int k = k0; k < k1; ++k) {
-      if (has_z) load_plane(k + 1);
-      __syncthreads();
-      if (active) {
-        const double(*cur)[SX] = ring[k & 3];
-        const double c = cur[ty + 1][tx + 1];
-        double w;
-        if (uniform) {
-          double s = (cur[ty + 1][tx] + cur[ty + 1][tx + 2]) + (cur[ty][tx + 1] + cur[ty + 2][tx + 1]);
-          double diag = 4.0;
-          if (has_z) {
-            s += ring[(k - 1) & 3][ty + 1][tx + 1] + ring[(k + 1) & 3][ty + 1][tx + 1];
-            diag = 6.0;
-          }
-          w = fma(diag, c, -s);
-          if (ihx != 1.0) w *= ihx;
-        } else {
-          const double wx = fma(2.0, c, -(cur[ty + 1][tx] + cur[ty + 1][tx + 2]));
-          const double wy = fma(2.0, c, -(cur[ty][tx + 1] + cur[ty + 2][tx + 1]));
-          w = fma(wx, ihx, wy * ihy);
-          if (has_z) {
-            const double wz = fma(2.0, c, -(ring[(k - 1) & 3][ty + 1][tx + 1] + ring[(k + 1) & 3][ty + 1][tx + 1]));
-            w = fma(wz, ihz, w);
-          }
-        }
-        const long long idx = (long long)k * plane + (long long)y * g.nx + x;
-        op(idx, c, w, acc);
-      }
-    }
-  }
-  if constexpr (NQ > 0) {
-    const int nblocks = gridDim.x * gridDim.y * gridDim.z;
-    const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    grid_reduce<NQ>(acc, partials, ticket, nblocks, bid, fin);
-  }
-}
-
-struct NoFin {
-  template <class T>
-  __device__ void operator()(T&) const {}
-};
-
-// ------------------------------------------------------------------ W = L x
-struct OpApply {
-  double* __restrict__ w;
-  __device__ __forceinline__ void operator()(long long i, double, double wv, double (&)[1]) { w[i] = wv; }
-};
-
-__global__ void __launch_bounds__(TX* TY) k_apply_laplacian(Geom g, int zchunk, const double* __restrict__ x,
-                                                            double* __restrict__ w) {
-  FieldPlain f{x};
-  OpApply op{w};
-  stencil_sweep<0>(g, zchunk, f, op, nullptr, nullptr, NoFin{});
 }
 
 // ------------------------------------------------------------------ low-precision copy of R
@@ -233,9 +122,8 @@ __device__ __forceinline__ void store_lp_pair(const LowPrec& lp, long long i, do
 }
 
 // ------------------------------------------------------------------ fixed-point stencil driver
-// Same 32 x 8 tiles and 4-slot plane ring as stencil_sweep, for fields held as
-// exact integers (IT = int or long long), organised for memory-level
-// parallelism:
+// 32 x 8 tiles and a plane ring, for fields held as exact integers (IT = long
+// long) or as FP64 values (IT = double), organised for memory-level parallelism:
 //  * persistent and balanced: the (tile, plane) pairs are numbered tile-major
 //    and block b takes a contiguous range of T / G or T / G + 1 of them,
 //    walked as one or two runs of consecutive planes of a tile;
@@ -250,9 +138,14 @@ __device__ __forceinline__ void store_lp_pair(const LowPrec& lp, long long i, do
 // its six neighbours with the ghosts applied (zl = zr = c in 2D), so every
 // second difference is exact.  op.flush(acc) turns the op's own per-thread
 // sums into the NQ doubles of the deterministic grid reduction.
+struct NoFin {
+  template <class T>
+  __device__ void operator()(SolveState*, T&) const {}
+};
+
 template <class IT, int NQ, class Field, class Op, class Fin>
 __device__ __forceinline__ void stencil_sweep_fx(const Geom& g, const Field& field, Op& op, double* partials,
-                                                 unsigned* ticket, Fin fin) {
+                                                 SolveState* st, int ticket, Fin fin) {
   constexpr int NT = TX * TY;
   constexpr int PER = (SX * SY + NT - 1) / NT;
   __shared__ IT ring[6][SY][SX];
@@ -347,12 +240,103 @@ __device__ __forceinline__ void stencil_sweep_fx(const Geom& g, const Field& fie
       pre1 = next1;
     }
   }
-  double acc[NQ];
-  op.flush(acc);
-  grid_reduce<NQ>(acc, partials, ticket, gridDim.x, blockIdx.x, fin);
+  if constexpr (NQ > 0) {
+    double acc[NQ];
+    op.flush(acc);
+    __shared__ __align__(16) unsigned scratch[kStateWords];
+    grid_reduce_state<NQ>(acc, partials, st, ticket, gridDim.x, blockIdx.x, scratch, fin);
+  }
 }
 
 struct NoPre {};
+
+// ------------------------------------------------------------------ FP64 fields through the integer units
+// The stencil of an FP64 field (tpcg_apply_laplacian, the FP64 form's W = L P, the Jacobi comparator).  An FP64 addition
+// occupies its pipe as long as 64 instructions occupy the others here, so the seven values of a point are aligned to
+// the largest of their exponents as 59-bit integers (some ten instructions each), summed exactly and rounded to FP64
+// once: the bits shifted out are below 2^-58 of the largest value, less than the rounding of a single FP64 addition.
+// 256 x 256 x 128: six FP64 operations a point took 157 us (0.6 of the pipe).
+
+// x as a multiple of 2^(E - 1081), E the exponent field E20 >> 20 >= that of x, truncated.
+__device__ __forceinline__ long long aligned59(double x, int E20) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x), mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const int d = min((E20 - (hi & 0x7ff00000)) >> 20, 63);
+  unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 6) << 32) | (unsigned long long)(lo << 6);
+  m >>= d;
+  return hi < 0 ? -(long long)m : (long long)m;
+}
+
+struct Weights {  // 1/h^2 per axis
+  double ih0, ih1, ih2;
+  int uniform;
+};
+
+// (L field)(point) from the point's value and its neighbours.  HW: convert with the FP64 pipe's instruction (kernels
+// that leave it idle), else by integer arithmetic.
+template <bool HW>
+__device__ __forceinline__ double stencil_f64(double c, double xl, double xr, double yl, double yr, double zl, double zr,
+                                              const Weights& w) {
+  auto ex = [](double v) { return __double2hiint(v) & 0x7ff00000; };
+  const int E20 = max(max(ex(c), max(ex(xl), ex(xr))), max(max(ex(yl), ex(yr)), max(ex(zl), ex(zr))));
+  if (E20 < (70 << 20) || E20 > (2040 << 20)) {  // next to the ends of the range, or not finite
+    const double dx = fma(2.0, c, -(xl + xr)), dy = fma(2.0, c, -(yl + yr)), dz = fma(2.0, c, -(zl + zr));
+    return fma(dz, w.ih2, fma(dx, w.ih0, dy * w.ih1));
+  }
+  const int e = (E20 >> 20) - 1081;
+  auto to_f64 = [&](long long v) { return HW ? i64_to_f64_scaled_hw(v, e) : i64_to_f64_scaled(v, e); };
+  const long long c2 = 2 * aligned59(c, E20);
+  const long long dx = c2 - aligned59(xl, E20) - aligned59(xr, E20), dy = c2 - aligned59(yl, E20) - aligned59(yr, E20),
+                  dz = c2 - aligned59(zl, E20) - aligned59(zr, E20);
+  if (w.uniform) {
+    const double r = to_f64(dx + dy + dz);
+    return w.ih0 != 1.0 ? r * w.ih0 : r;
+  }
+  return fma(to_f64(dz), w.ih2, fma(to_f64(dx), w.ih0, to_f64(dy) * w.ih1));
+}
+
+__device__ __forceinline__ Weights weights_of(const Geom& g) { return Weights{g.ih2[0], g.ih2[1], g.ih2[2], g.uniform}; }
+
+struct FieldPlain {  // the stencil is applied to x itself
+  using Raw = double;
+  const double* __restrict__ x;
+  __device__ __forceinline__ double load(unsigned i) const { return __ldg(x + i); }
+  __device__ __forceinline__ double convert(double v) const { return v; }
+};
+
+struct FieldDirection {  // FP64 form: P = (Z - mean Z) + beta * P_old   (Algorithm 1; Remark orthogonality)
+  struct Raw {
+    double z, p;
+  };
+  const double* __restrict__ z;
+  const double* __restrict__ pold;
+  double mZ, beta;
+  int first;
+  __device__ __forceinline__ Raw load(unsigned i) const { return Raw{__ldg(z + i), first ? 0.0 : __ldg(pold + i)}; }
+  __device__ __forceinline__ double convert(const Raw& r) const {
+    const double zi = r.z - mZ;
+    return first ? zi : fma(beta, r.p, zi);
+  }
+};
+
+// ------------------------------------------------------------------ W = L x
+struct OpApply {
+  using Pre = NoPre;
+  double* __restrict__ w;
+  Weights wt;
+  __device__ __forceinline__ NoPre load(unsigned) const { return NoPre{}; }
+  __device__ __forceinline__ void operator()(unsigned i, int, int, int, NoPre, double c, double xl, double xr, double yl,
+                                             double yr, double zl, double zr) {
+    w[i] = stencil_f64<true>(c, xl, xr, yl, yr, zl, zr, wt);
+  }
+};
+
+__global__ void __launch_bounds__(TX* TY) k_apply_laplacian(Geom g, const double* __restrict__ x,
+                                                            double* __restrict__ w) {
+  FieldPlain f{x};
+  OpApply op{w, weights_of(g)};
+  stencil_sweep_fx<double, 0>(g, f, op, nullptr, nullptr, 0, NoFin{});
+}
 
 // max |U| is tracked on FP64 bit patterns shifted left by one: dropping the
 // sign bit this way keeps the order of magnitudes and stays an integer
@@ -490,8 +474,8 @@ __global__ void __launch_bounds__(TX* TY) k_residual_fx(Geom g, const double* __
   const long long N = g.N;
   const bool finite_u = isfinite(st->umax);
   stencil_sweep_fx<long long, 4>(
-      g, f, op, partials, &st->tickets[INIT ? kTkInit : kTkTrue],
-      [st, force, N, sr, ku, finite_u](const double(&s)[4]) {
+      g, f, op, partials, st, INIT ? kTkInit : kTkTrue,
+      [force, N, sr, ku, finite_u](SolveState* st, const double(&s)[4]) {
         const double rr = finite_u ? scale_pow2(s[0], -2 * sr) : __longlong_as_double(0x7ff8000000000000ll);
         const double sumR = scale_pow2(s[1], -sr), sumU = scale_pow2(s[2], 8 - ku);
         if (!INIT) st->checks += 1;
@@ -512,13 +496,20 @@ __global__ void __launch_bounds__(TX* TY) k_residual_fx(Geom g, const double* __
 // P_s = Z_s' + beta_s P_{s-1} (Algorithm 1, with Z centred), W = L P, <W, P>
 // and the step length alpha = rho / <W, P>.
 struct OpDirection {
+  using Pre = NoPre;
   double* __restrict__ P;
   double* __restrict__ W;
-  __device__ __forceinline__ void operator()(long long i, double c, double w, double (&acc)[1]) {
+  Weights wt;
+  double wp;
+  __device__ __forceinline__ NoPre load(unsigned) const { return NoPre{}; }
+  __device__ __forceinline__ void operator()(unsigned i, int, int, int, NoPre, double c, double xl, double xr, double yl,
+                                             double yr, double zl, double zr) {
+    const double w = stencil_f64<false>(c, xl, xr, yl, yr, zl, zr, wt);
     P[i] = c;
     W[i] = w;
-    acc[0] = fma(w, c, acc[0]);
+    wp = fma(w, c, wp);
   }
+  __device__ __forceinline__ void flush(double (&acc)[1]) const { acc[0] = wp; }
 };
 
 __device__ void fin_direction(SolveState* st, const double (&s)[1], const Geom& g) {
@@ -534,16 +525,16 @@ __device__ void fin_direction(SolveState* st, const double (&s)[1], const Geom& 
   for (int m = 0; m < 3; ++m) st->nah[m] = -alpha * g.ih2[m];
 }
 
-__global__ void __launch_bounds__(TX* TY) k_direction(Geom g, int zchunk, const double* __restrict__ Z,
+__global__ void __launch_bounds__(TX* TY) k_direction(Geom g, const double* __restrict__ Z,
                                                       double* __restrict__ P0, double* __restrict__ P1,
                                                       double* __restrict__ W, SolveState* st, double* partials) {
   if (paused(st)) return;
   double* P = (st->iter & 1) ? P1 : P0;  // P_s in buffer s & 1
   const double* Pold = (st->iter & 1) ? P0 : P1;
   FieldDirection f{Z, Pold, st->mZ, st->beta, st->first};
-  OpDirection op{P, W};
-  stencil_sweep<1>(g, zchunk, f, op, partials, &st->tickets[kTkDir],
-                   [st, g](const double(&s)[1]) { fin_direction(st, s, g); });
+  OpDirection op{P, W, weights_of(g), 0.0};
+  stencil_sweep_fx<double, 1>(g, f, op, partials, st, kTkDir,
+                   [g](SolveState* st, const double(&s)[1]) { fin_direction(st, s, g); });
 }
 
 // Storage of the directions: P_s is in slot s % slots.  The kernels take s from the state (iterations completed): the
@@ -677,9 +668,12 @@ __global__ void __launch_bounds__(TX* TY) k_direction_int(Geom g, const float* _
   const unsigned long long m = block_max_u64((unsigned long long)pm);
   if (threadIdx.x + threadIdx.y == 0) atomicMax(&st->pmax_bits, (unsigned)m);
   const int nblocks = gridDim.x;
-  grid_reduce<1>(acc, partials, &st->tickets[kTkDir], nblocks, blockIdx.x, [st, kp, g](const double(&s)[1]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<1>(acc, partials, st, kTkDir, nblocks, blockIdx.x, scratch,
+                       [kp, g](SolveState* st, const double(&s)[1]) {
     st->kp = kp;
-    st->pmax = scale_pow2((double)atomicExch(&st->pmax_bits, 0u), -kp);
+    st->pmax = scale_pow2((double)st->pmax_bits, -kp);
+    st->pmax_bits = 0u;
     const double v[1] = {scale_pow2(s[0], -2 * kp)};
     fin_direction(st, v, g);
   });
@@ -778,9 +772,12 @@ __global__ void __launch_bounds__(TX* TY) k_direction_pair(Geom g, const float* 
   double acc[1] = {f32_to_f64_int(e)};
   const unsigned long long m = block_max_u64((unsigned long long)pm);
   if (threadIdx.x + threadIdx.y == 0) atomicMax(&st->pmax_bits, (unsigned)m);
-  grid_reduce<1>(acc, partials, &st->tickets[kTkDir], gridDim.x, blockIdx.x, [st, kp, g](const double(&s)[1]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<1>(acc, partials, st, kTkDir, gridDim.x, blockIdx.x, scratch,
+                       [kp, g](SolveState* st, const double(&s)[1]) {
     st->kp = kp;
-    st->pmax = scale_pow2((double)atomicExch(&st->pmax_bits, 0u), -kp);
+    st->pmax = scale_pow2((double)st->pmax_bits, -kp);
+    st->pmax_bits = 0u;
     const double v[1] = {scale_pow2(s[0], -2 * kp)};
     fin_direction(st, v, g);
   });
@@ -899,9 +896,12 @@ __global__ void __launch_bounds__(TX* TY) k_direction_quad(Geom g, const float* 
   double acc[1] = {f32_to_f64_int(e)};
   const unsigned long long m = block_max_u64((unsigned long long)pm);
   if (threadIdx.x + threadIdx.y == 0) atomicMax(&st->pmax_bits, (unsigned)m);
-  grid_reduce<1>(acc, partials, &st->tickets[kTkDir], gridDim.x, blockIdx.x, [st, kp, g](const double(&s)[1]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<1>(acc, partials, st, kTkDir, gridDim.x, blockIdx.x, scratch,
+                       [kp, g](SolveState* st, const double(&s)[1]) {
     st->kp = kp;
-    st->pmax = scale_pow2((double)atomicExch(&st->pmax_bits, 0u), -kp);
+    st->pmax = scale_pow2((double)st->pmax_bits, -kp);
+    st->pmax_bits = 0u;
     const double v[1] = {scale_pow2(s[0], -2 * kp)};
     fin_direction(st, v, g);
   });
@@ -929,7 +929,8 @@ __device__ void fin_update(SolveState* st, const double (&s)[2], int shift, cons
     st->pend_slot[n] = pslot;
     st->n_pend = n + 1;
   } else {
-    st->umax = __longlong_as_double((long long)atomicExch(&st->umax_bits, 0ull));
+    st->umax = __longlong_as_double((long long)st->umax_bits);
+    st->umax_bits = 0ull;
     plan_residual_check(st, g);
   }
   advance_shift(st, rr, g.N);
@@ -1031,8 +1032,9 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_int(Geom g, DirRing ring, 
     }
   });
   double acc[2] = {f32_to_f64_int(rr), f32_to_f64_int(sR)};
-  grid_reduce<2>(acc, partials, &st->tickets[kTkUpd], gridDim.x, blockIdx.x,
-                 [st, shift, g, pslot](const double(&s)[2]) { fin_update(st, s, shift, g, pslot); });
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkUpd, gridDim.x, blockIdx.x, scratch,
+                       [shift, g, pslot](SolveState* st, const double(&s)[2]) { fin_update(st, s, shift, g, pslot); });
 }
 
 // The same update with two adjacent x points per thread (even nx): R moves
@@ -1136,8 +1138,9 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_pair(Geom g, DirRing ring,
   if (g.uniform) sweep(std::true_type{});
   else sweep(std::false_type{});
   double acc[2] = {f32_to_f64_int(rr), f32_to_f64_int(sR)};
-  grid_reduce<2>(acc, partials, &st->tickets[kTkUpd], gridDim.x, blockIdx.x,
-                 [st, shift, g, pslot](const double(&s)[2]) { fin_update(st, s, shift, g, pslot); });
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkUpd, gridDim.x, blockIdx.x, scratch,
+                       [shift, g, pslot](SolveState* st, const double(&s)[2]) { fin_update(st, s, shift, g, pslot); });
 }
 
 // Mixed forms, U updated in place (the default): U += alpha P and R -= alpha W with W = L P from the
@@ -1242,8 +1245,9 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_int(Geom g, double* __re
   });
   double acc[2] = {f32_to_f64_int(rr), f32_to_f64_int(sR)};
   fold_umax(st, um);
-  grid_reduce<2>(acc, partials, &st->tickets[kTkUpd], gridDim.x, blockIdx.x,
-                 [st, shift, g](const double(&s)[2]) { fin_update(st, s, shift, g, -1); });
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkUpd, gridDim.x, blockIdx.x, scratch,
+                       [shift, g](SolveState* st, const double(&s)[2]) { fin_update(st, s, shift, g, -1); });
 }
 
 // The same in-place update with two adjacent x points per thread (even nx): R and U move
@@ -1361,8 +1365,9 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_pair(Geom g, double* __r
   else sweep(std::false_type{});
   double acc[2] = {f32_to_f64_int(rr), f32_to_f64_int(sR)};
   fold_umax(st, um);
-  grid_reduce<2>(acc, partials, &st->tickets[kTkUpd], gridDim.x, blockIdx.x,
-                 [st, shift, g](const double(&s)[2]) { fin_update(st, s, shift, g, -1); });
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkUpd, gridDim.x, blockIdx.x, scratch,
+                       [shift, g](SolveState* st, const double(&s)[2]) { fin_update(st, s, shift, g, -1); });
 }
 
 // FP64 form: P and W = L P are stored by the direction kernel.
@@ -1395,8 +1400,9 @@ __global__ void __launch_bounds__(256) k_update(Geom g, double* __restrict__ U, 
   }
   fold_umax(st, um);
   double acc[2] = {f32_to_f64_int(a0), f32_to_f64_int(a1)};
-  grid_reduce<2>(acc, partials, &st->tickets[kTkUpd], gridDim.x, blockIdx.x,
-                 [st, shift, g](const double(&s)[2]) { fin_update(st, s, shift, g, -1); });
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkUpd, gridDim.x, blockIdx.x, scratch,
+                       [shift, g](SolveState* st, const double(&s)[2]) { fin_update(st, s, shift, g, -1); });
 }
 
 // ------------------------------------------------------------------ streaming kernels
@@ -1421,7 +1427,9 @@ __global__ void __launch_bounds__(256) k_init_zero(long long N, const double* __
     a1 += r32;
   }
   double acc[2] = {e2, f32_to_f64_int(a1)};
-  grid_reduce<2>(acc, partials, &st->tickets[kTkInit], gridDim.x, blockIdx.x, [st, N, shift](const double(&s)[2]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkInit, gridDim.x, blockIdx.x, scratch,
+                       [N, shift](SolveState* st, const double(&s)[2]) {
     const double v[3] = {s[0], scale_pow2(s[1], -shift), s[0]};
     fin_init(st, v, N);
   });
@@ -1448,13 +1456,16 @@ __global__ void __launch_bounds__(256) k_eta_sum(Geom g, const double* __restric
     }
   }
   fold_umax(st, um);
-  grid_reduce<2>(acc, partials, &st->tickets[kTkEta], gridDim.x, blockIdx.x, [st, N, g](const double(&s)[2]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkEta, gridDim.x, blockIdx.x, scratch,
+                       [N, g](SolveState* st, const double(&s)[2]) {
     const double mean = st->singular ? s[0] / (double)N : 0.0;
     st->mean_eta = mean;
     const double n2 = s[1] - mean * s[0];
     st->eta_norm2 = n2 > 0.0 ? n2 : s[1];  // estimate; the initial residual kernel sets the exact value
     st->lp_shift = lp_shift_for(n2 > 0.0 ? n2 : s[1], N);
-    st->umax = __longlong_as_double((long long)atomicExch(&st->umax_bits, 0ull));
+    st->umax = __longlong_as_double((long long)st->umax_bits);
+    st->umax_bits = 0ull;
     plan_residual_check(st, g);
   });
 }
@@ -1529,10 +1540,13 @@ __global__ void __launch_bounds__(256) k_form_u(Geom g, double* __restrict__ U, 
   }
   fold_umax(st, um);
   double acc[1] = {0.0};
-  grid_reduce<1>(acc, partials, &st->tickets[kTkForm], gridDim.x, blockIdx.x, [st, g](const double(&)[1]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<1>(acc, partials, st, kTkForm, gridDim.x, blockIdx.x, scratch,
+                       [g](SolveState* st, const double(&)[1]) {
     st->n_pend = 0;
     st->u_valid = 1;
-    st->umax = __longlong_as_double((long long)atomicExch(&st->umax_bits, 0ull));
+    st->umax = __longlong_as_double((long long)st->umax_bits);
+    st->umax_bits = 0ull;
     plan_residual_check(st, g);
   });
 }
@@ -1560,7 +1574,9 @@ __global__ void __launch_bounds__(256) k_init_zero2(unsigned npair, long long N,
     a1 += a32 + b32;
   }
   double acc[2] = {e2, f32_to_f64_int(a1)};
-  grid_reduce<2>(acc, partials, &st->tickets[kTkInit], gridDim.x, blockIdx.x, [st, N, shift](const double(&s)[2]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkInit, gridDim.x, blockIdx.x, scratch,
+                       [N, shift](SolveState* st, const double(&s)[2]) {
     const double v[3] = {s[0], scale_pow2(s[1], -shift), s[0]};
     fin_init(st, v, N);
   });
@@ -1588,13 +1604,16 @@ __global__ void __launch_bounds__(256) k_eta_sum2(Geom g, unsigned npair, const 
     }
   }
   fold_umax(st, um);
-  grid_reduce<2>(acc, partials, &st->tickets[kTkEta], gridDim.x, blockIdx.x, [st, N, g](const double(&s)[2]) {
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkEta, gridDim.x, blockIdx.x, scratch,
+                       [N, g](SolveState* st, const double(&s)[2]) {
     const double mean = st->singular ? s[0] / (double)N : 0.0;
     st->mean_eta = mean;
     const double n2 = s[1] - mean * s[0];
     st->eta_norm2 = n2 > 0.0 ? n2 : s[1];  // estimate; the initial residual kernel sets the exact value
     st->lp_shift = lp_shift_for(n2 > 0.0 ? n2 : s[1], N);
-    st->umax = __longlong_as_double((long long)atomicExch(&st->umax_bits, 0ull));
+    st->umax = __longlong_as_double((long long)st->umax_bits);
+    st->umax_bits = 0ull;
     plan_residual_check(st, g);
   });
 }
@@ -1607,8 +1626,9 @@ __global__ void __launch_bounds__(256) k_norm_shift(long long N, const double* _
     const double v = __ldg(r + i);
     acc[0] = fma(v, v, acc[0]);
   }
-  grid_reduce<1>(acc, partials, &st->tickets[kTkMisc], gridDim.x, blockIdx.x,
-                 [st, N](const double(&s)[1]) { st->lp_shift = lp_shift_for(s[0], N); });
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<1>(acc, partials, st, kTkMisc, gridDim.x, blockIdx.x, scratch,
+                       [N](SolveState* st, const double(&s)[1]) { st->lp_shift = lp_shift_for(s[0], N); });
 }
 
 // U -= sum(U)/N: return the zero-mean (minimum-norm) representative.  Without
@@ -1709,21 +1729,25 @@ __global__ void __launch_bounds__(256) k_jacobi_first(Geom g, const double* __re
 }
 
 struct OpJacobi {
+  using Pre = double;  // R at the point
   const double* __restrict__ R;
   double* __restrict__ Xnew;
   JacobiTable t;
   Geom g;
-  __device__ __forceinline__ void operator()(long long i, double c, double w, double (&)[1]) {
-    Xnew[i] = fma(__ldg(R + i) - w, jacobi_invd(t, g, (unsigned)i), c);
+  Weights wt;
+  __device__ __forceinline__ double load(unsigned i) const { return __ldg(R + i); }
+  __device__ __forceinline__ void operator()(unsigned i, int, int, int, double r, double c, double xl, double xr,
+                                             double yl, double yr, double zl, double zr) {
+    Xnew[i] = fma(r - stencil_f64<true>(c, xl, xr, yl, yr, zl, zr, wt), jacobi_invd(t, g, i), c);
   }
 };
 
-__global__ void __launch_bounds__(TX* TY) k_jacobi_sweep(Geom g, int zchunk, const double* __restrict__ Xold,
+__global__ void __launch_bounds__(TX* TY) k_jacobi_sweep(Geom g, const double* __restrict__ Xold,
                                                          double* __restrict__ Xnew, const double* __restrict__ R,
                                                          JacobiTable t) {
   FieldPlain f{Xold};
-  OpJacobi op{R, Xnew, t, g};
-  stencil_sweep<0>(g, zchunk, f, op, nullptr, nullptr, NoFin{});
+  OpJacobi op{R, Xnew, t, g, weights_of(g)};
+  stencil_sweep_fx<double, 0>(g, f, op, nullptr, nullptr, 0, NoFin{});
 }
 
 // rho = <R, Z> and sum(Z) in FP64 (comparators); Z = R first when copy (M = I).
@@ -1738,8 +1762,9 @@ __global__ void __launch_bounds__(256) k_dot_rz(long long N, const double* __res
     acc[1] += z;
   }
   if (!st) return;
-  grid_reduce<2>(acc, partials, &st->tickets[kTkPrec], gridDim.x, blockIdx.x,
-                 [st, N](const double(&s)[2]) { fin_precond(st, N, s); });
+  __shared__ __align__(16) unsigned scratch[kStateWords];
+  grid_reduce_state<2>(acc, partials, st, kTkPrec, gridDim.x, blockIdx.x, scratch,
+                       [N](SolveState* st, const double(&s)[2]) { fin_precond(st, N, s); });
 }
 
 // ------------------------------------------------------------------ electric field
@@ -1787,7 +1812,7 @@ __global__ void __launch_bounds__(256) k_efield(Geom g, const double* __restrict
 // ------------------------------------------------------------------ host launchers
 void launch_apply_laplacian(const tpcg_plan* p, const Geom& g, const double* x, double* w) {
   LaunchScope ls(p, kKApply);
-  k_apply_laplacian<<<p->st_grid, p->st_block, 0, p->stream>>>(g, p->st_zchunk, x, w);
+  k_apply_laplacian<<<p->fx_blocks[kFxApply], p->st_block, 0, p->stream>>>(g, x, w);
 }
 // Persistent grids of the fixed-point sweeps: every SM holds as many blocks as
 // the kernel's resources allow (at most 8), and every block takes at least
@@ -1798,12 +1823,15 @@ int setup_fx_grids(tpcg_plan* p) {
   const long long grain = p->sweep_grain;
   p->stream_blocks = (int)std::max(1LL, std::min<long long>((p->N + 256 * grain - 1) / (256 * grain),
                                                            (long long)p->num_sms * 8));
-  const bool pair = p->nx % 2 == 0;  // direction and update take two x points per thread
-  const bool quad = p->nx % 4 == 0;  // direction takes four
-  const void* fns[kFxCount] = {quad ? (const void*)k_direction_quad
-                                    : (pair ? (const void*)k_direction_pair : (const void*)k_direction_int),
+  const bool f64 = p->prec == TPCG_FP64;
+  const bool pair = !f64 && p->nx % 2 == 0;  // direction and update take two x points per thread
+  const bool quad = !f64 && p->nx % 4 == 0;  // direction takes four
+  const void* fns[kFxCount] = {f64    ? (const void*)k_direction
+                               : quad ? (const void*)k_direction_quad
+                                      : (pair ? (const void*)k_direction_pair : (const void*)k_direction_int),
                                pair ? (const void*)k_update_pair : (const void*)k_update_int,
-                               (const void*)k_residual_fx<false>, (const void*)k_residual_fx<true>};
+                               (const void*)k_residual_fx<false>, (const void*)k_residual_fx<true>,
+                               (const void*)k_apply_laplacian};
   for (int i = 0; i < kFxCount; ++i) {
     const int tw = (i == kFxDir && quad) ? 4 * TX : (((i == kFxUpd || i == kFxDir) && pair) ? 2 * TX : TX);
     const long long T = (long long)((p->nx + tw - 1) / tw) * ((p->ny + TY - 1) / TY) * p->nz;
@@ -1856,8 +1884,9 @@ static DirRing dir_ring(const tpcg_plan* p) {
 void launch_direction(const tpcg_plan* p, const Geom& g) {
   LaunchScope ls(p, kKDirection);
   if (p->prec == TPCG_FP64) {
-    k_direction<<<p->st_grid, p->st_block, 0, p->stream>>>(g, p->st_zchunk, (const double*)p->d_Z, (double*)p->d_P[0],
-                                                            (double*)p->d_P[1], p->d_W, p->d_state, p->d_partials);
+    k_direction<<<p->fx_blocks[kFxDir], p->st_block, 0, p->stream>>>(g, (const double*)p->d_Z, (double*)p->d_P[0],
+                                                                      (double*)p->d_P[1], p->d_W, p->d_state,
+                                                                      p->d_partials);
     return;
   }
   const DirRing ring = dir_ring(p);
@@ -1956,7 +1985,7 @@ void run_precond_cmp(const tpcg_plan* p, const Geom& g, const double* R, double*
     }
     for (int j = 2; j <= p->jac_p; ++j) {
       LaunchScope ls(p, kKModeF64);
-      k_jacobi_sweep<<<p->st_grid, p->st_block, 0, p->stream>>>(g, p->st_zchunk, buf(j - 1), buf(j), R, t);
+      k_jacobi_sweep<<<p->fx_blocks[kFxApply], p->st_block, 0, p->stream>>>(g, buf(j - 1), buf(j), R, t);
     }
   }
   if (st || p->pc_kind == TPCG_PRECOND_NONE) {

@@ -111,8 +111,9 @@ __global__ void __launch_bounds__(256) k_modeprod_f64(ModeArgsF64 a) {
   if constexpr (FINAL) {
     SolveState* st = a.st;
     const long long N = a.N;
-    grid_reduce<2>(red, a.partials, &st->tickets[kTkPrec], gridDim.x * gridDim.y, blockIdx.x + gridDim.x * blockIdx.y,
-                   [st, N](const double(&s)[2]) { fin_precond(st, N, s); });
+    __shared__ __align__(16) unsigned scratch[kStateWords];
+    grid_reduce_state<2>(red, a.partials, st, kTkPrec, gridDim.x * gridDim.y, blockIdx.x + gridDim.x * blockIdx.y,
+                         scratch, [N](SolveState* st, const double(&s)[2]) { fin_precond(st, N, s); });
   }
 }
 

@@ -484,7 +484,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
     double acc[2] = {red0, red1};
     SolveState* st = a.st;
     const long long N = a.N;
-    grid_reduce<2>(acc, a.partials, &st->tickets[kTkPrec], gridDim.x, blockIdx.x, [st, N](const double(&s)[2]) {
+    // (the shared memory of the tiles is free: every copy and MMA has completed)
+    grid_reduce_state<2>(acc, a.partials, st, kTkPrec, gridDim.x, blockIdx.x, reinterpret_cast<unsigned*>(sm),
+                         [N](SolveState* st, const double(&s)[2]) {
       if (!st->timeout) {
         fin_precond(st, N, s);
       } else {

@@ -451,9 +451,11 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
     double acc[2] = {acc_value(red0), acc_value(red1)};
     SolveState* st = a.st;
     const long long N = a.N;
-    grid_reduce<2>(acc, a.partials, &st->tickets[kTkPrec], gridDim.x, blockIdx.x,
-                   [st, N, shR](const double(&s)[2]) {
-                     st->zmax = __uint_as_float(atomicExch(&st->zmax_bits, 0u));
+    // (the shared memory of the tiles is free: every copy and MMA has completed)
+    grid_reduce_state<2>(acc, a.partials, st, kTkPrec, gridDim.x, blockIdx.x, reinterpret_cast<unsigned*>(sm),
+                   [N, shR](SolveState* st, const double(&s)[2]) {
+                     st->zmax = __uint_as_float(st->zmax_bits);
+                     st->zmax_bits = 0u;
                      const double v[2] = {scale_pow2(s[0], -shR), s[1]};
                      if (!st->timeout) {
                        fin_precond(st, N, v);

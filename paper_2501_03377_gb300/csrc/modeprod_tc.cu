@@ -126,6 +126,18 @@ __device__ __forceinline__ void st_global_v8(void* p, const uint32_t (&w)[8]) {
                : "memory");
 }
 
+// 32 bytes from global memory (data that no running kernel writes): in one load where the address allows it.
+__device__ __forceinline__ void ld_global_32(const void* p, uint32_t (&w)[8]) {
+  if (((uintptr_t)p & 31) == 0) {
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "l"(p));
+  } else {
+    const uint4 a = __ldg(reinterpret_cast<const uint4*>(p)), b = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+    w[0] = a.x, w[1] = a.y, w[2] = a.z, w[3] = a.w, w[4] = b.x, w[5] = b.y, w[6] = b.z, w[7] = b.w;
+  }
+}
+
 // hi = bf16(v) at o, lo = bf16(v - hi) one plane further (v - hi is exact in FP32).
 __device__ __forceinline__ void store_pair(void* out, long long plane, long long o, float v) {
   const __nv_bfloat16 hi = __float2bfloat16_rn(v);
@@ -186,6 +198,16 @@ __device__ __forceinline__ void store16(void* out, long long plane, long long o,
     d[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
     d[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
   } else {
+    if ((o & 7) == 0) {  // 32-byte aligned: full sectors
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        uint32_t w[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) w[k] = __float_as_uint(x[8 * i + k]);
+        st_global_v8(reinterpret_cast<float*>(out) + o + 8 * i, w);
+      }
+      return;
+    }
     float4* d = reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + o);
 #pragma unroll
     for (int i = 0; i < 4; ++i) d[i] = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
@@ -563,7 +585,16 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
             rb[1] = __ldg(rp + 1);
           }
         };
-        auto process = [&](int c0, const uint32_t (&t)[16], const uint4 (&rcur)[2]) {
+        // split form: the 16 hi and the 16 lo words of R~ chunk j of this row
+        auto fetch_pair = [&](int j, uint32_t (&hw)[8], uint32_t (&lw)[8]) {
+          if ((ODD ? valid : vec) && j < J && col(j) + 16 <= (ODD ? a.rpitch : a.Cout)) {
+            const long long ro = (long long)r * a.rpitch + col(j);
+            ld_global_32(a.Rt + ro, hw);
+            ld_global_32(Rlo + ro, lw);
+          }
+        };
+        auto process = [&](int c0, const uint32_t (&t)[16], const uint4 (&rcur)[2], const uint32_t (&hw)[8],
+                           const uint32_t (&lw)[8]) {
           if (!valid && !a.tstore && !ODD) return;
           float v[16];
 #pragma unroll
@@ -602,12 +633,7 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
           if (!valid) return;
           if (vec && c0 + 16 <= a.Cout) {
             if (!a.tstore) store16<OutT>(a.out, a.oplane, obase + c0, v);
-            if (FINAL && KS::split) {  // R~ = hi + lo, 16 values of this row from each plane
-              const uint4* hp = reinterpret_cast<const uint4*>(a.Rt + (long long)r * a.rpitch + c0);
-              const uint4* lq = reinterpret_cast<const uint4*>(Rlo + (long long)r * a.rpitch + c0);
-              const uint4 h0 = __ldg(hp), h1 = __ldg(hp + 1), l0 = __ldg(lq), l1 = __ldg(lq + 1);
-              const uint32_t hw[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-              const uint32_t lw[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
+            if (FINAL && KS::split) {  // R~ = hi + lo, 16 values of this row from each plane (fetch_pair)
               float d0 = 0.0f, d1 = 0.0f;
 #pragma unroll
               for (int i = 0; i < 8; ++i) {
@@ -661,25 +687,20 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
                     const float4 x = __ldg(rp + i);
                     rv[4 * i] = x.x, rv[4 * i + 1] = x.y, rv[4 * i + 2] = x.z, rv[4 * i + 3] = x.w;
                   }
+                } else if constexpr (KS::split) {
+#pragma unroll
+                  for (int i = 0; i < 8; ++i) {
+                    const float2 x = lp2_to_f32<__nv_bfloat16>(hw[i]), y = lp2_to_f32<__nv_bfloat16>(lw[i]);
+                    rv[2 * i] = x.x + y.x, rv[2 * i + 1] = x.y + y.y;
+                  }
                 } else {
                   const uint4* hp = reinterpret_cast<const uint4*>(a.Rt + ro);
                   const uint4 h0 = __ldg(hp), h1 = __ldg(hp + 1);
-                  const uint32_t hw[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-                  using LpT = typename std::conditional<KS::split, __nv_bfloat16, InT>::type;
+                  const uint32_t ww[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
 #pragma unroll
                   for (int i = 0; i < 8; ++i) {
-                    const float2 x = lp2_to_f32<LpT>(hw[i]);
+                    const float2 x = lp2_to_f32<InT>(ww[i]);
                     rv[2 * i] = x.x, rv[2 * i + 1] = x.y;
-                  }
-                  if constexpr (KS::split) {
-                    const uint4* lq = reinterpret_cast<const uint4*>(Rlo + ro);
-                    const uint4 l0 = __ldg(lq), l1 = __ldg(lq + 1);
-                    const uint32_t lw[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                      const float2 x = lp2_to_f32<__nv_bfloat16>(lw[i]);
-                      rv[2 * i] += x.x, rv[2 * i + 1] += x.y;
-                    }
                   }
                 }
               } else {
@@ -712,13 +733,32 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
         };
         uint32_t tA[16], tB[16];
         uint4 rA[2], rB[2];
-        if (rtma) {
+        uint32_t rw0[8], rw1[8];
+        if constexpr (FINAL && KS::split) {
+          // R~ of the next chunk is on its way while this one is processed; the accumulator's chunk is loaded when
+          // needed (tens of clocks against the some eight hundred of R~, which, waited for chunk by chunk, made this
+          // pass twice as long as the others: 42 against 22 us at 256 x 256 x 128)
+          uint32_t rw2[8], rw3[8];
+          fetch_pair(0, rw0, rw1);
+          for (int j = 0; j < J; j += 2) {
+            tc_ld16_issue(tacc + (uint32_t)col(j), tA);
+            fetch_pair(j + 1, rw2, rw3);
+            tc_ld16_wait(tA);
+            process(col(j), tA, rA, rw0, rw1);
+            if (j + 1 < J) {
+              tc_ld16_issue(tacc + (uint32_t)col(j + 1), tA);
+              fetch_pair(j + 2, rw0, rw1);
+              tc_ld16_wait(tA);
+              process(col(j + 1), tA, rA, rw2, rw3);
+            }
+          }
+        } else if (rtma) {
           bool ok = true;
           for (int j = 0; ok && j < J; ++j) {
             tc_ld16_issue(tacc + (uint32_t)col(j), tA);
             ok = __all_sync(0xffffffffu, take_r(j, rA));  // warp-uniform: tcgen05.ld is .sync.aligned
             tc_ld16_wait(tA);
-            if (ok) process(col(j), tA, rA);
+            if (ok) process(col(j), tA, rA, rw0, rw1);
           }
         } else {
           if (J > 0) {
@@ -729,12 +769,12 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
           }
           for (int j = 0; j < J; j += 2) {
             if (j + 1 < J) tc_ld16_issue(tacc + (uint32_t)col(j + 1), tB);
-            process(col(j), tA, rA);
+            process(col(j), tA, rA, rw0, rw1);
             fetch_r(j + 2, rA);
             if (j + 1 < J) {
               tc_ld16_wait(tB);
               if (j + 2 < J) tc_ld16_issue(tacc + (uint32_t)col(j + 2), tA);
-              process(col(j + 1), tB, rB);
+              process(col(j + 1), tB, rB, rw0, rw1);
               fetch_r(j + 3, rB);
               if (j + 2 < J) tc_ld16_wait(tA);
             }
@@ -828,9 +868,11 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     double acc[2] = {acc_value(red0), acc_value(red1)};
     SolveState* st = a.st;
     const long long N = a.N;
-    grid_reduce<2>(acc, a.partials, &st->tickets[kTkPrec], gridDim.x, blockIdx.x,
-                   [st, N, shR](const double(&s)[2]) {
-                     st->zmax = __uint_as_float(atomicExch(&st->zmax_bits, 0u));
+    // (the shared memory of the tiles is free: every copy and MMA has completed)
+    grid_reduce_state<2>(acc, a.partials, st, kTkPrec, gridDim.x, blockIdx.x, reinterpret_cast<unsigned*>(sm),
+                   [N, shR](SolveState* st, const double(&s)[2]) {
+                     st->zmax = __uint_as_float(st->zmax_bits);
+                     st->zmax_bits = 0u;
                      const double v[2] = {scale_pow2(s[0], -shR), s[1]};
                      if (!st->timeout) {
                        fin_precond(st, N, v);

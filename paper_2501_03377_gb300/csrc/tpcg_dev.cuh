@@ -178,12 +178,11 @@ __device__ __forceinline__ void block_sum(double (&v)[NQ], double* sh /* NQ*32 d
   __syncthreads();
 }
 
-// Deterministic grid-wide reduction: every block stores its partial sums,
-// the last block to arrive adds all partials in block order and calls
-// fin(sums) from thread 0.  Returns true in the finishing thread.
-template <int NQ, class Fin>
-__device__ __forceinline__ void grid_reduce(double (&v)[NQ], double* partials, unsigned* ticket, int nblocks,
-                                            int block_id, Fin fin) {
+// grid_reduce / grid_reduce_state: begin() in every thread of the last block before the partials are added, fin(sums) in
+// its thread 0, end() in every thread afterwards.
+template <int NQ, class Begin, class Fin, class End>
+__device__ __forceinline__ void grid_reduce_impl(double (&v)[NQ], double* partials, unsigned* ticket, int nblocks,
+                                                 int block_id, Begin begin, Fin fin, End end) {
   __shared__ double sh[NQ * 32];
   __shared__ bool last;
   block_sum<NQ>(v, sh);
@@ -199,6 +198,7 @@ __device__ __forceinline__ void grid_reduce(double (&v)[NQ], double* partials, u
   __syncthreads();
   if (!last) return;
   __threadfence();
+  begin();
   double s[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) s[q] = 0.0;
@@ -206,11 +206,47 @@ __device__ __forceinline__ void grid_reduce(double (&v)[NQ], double* partials, u
 #pragma unroll
     for (int q = 0; q < NQ; ++q) s[q] += __ldcg(&partials[(size_t)b * NQ + q]);
   }
-  block_sum<NQ>(s, sh, (tid & ~31) < nblocks);
-  if (tid == 0) {
+  block_sum<NQ>(s, sh, (tid & ~31) < nblocks);  // (its barriers order begin()'s shared writes before fin)
+  if (tid == 0) fin(s);
+  end();
+}
+
+// Deterministic grid-wide reduction: every block stores its partial sums,
+// the last block to arrive adds all partials in block order and calls
+// fin(sums) from thread 0.
+template <int NQ, class Fin>
+__device__ __forceinline__ void grid_reduce(double (&v)[NQ], double* partials, unsigned* ticket, int nblocks,
+                                            int block_id, Fin fin) {
+  grid_reduce_impl<NQ>(v, partials, ticket, nblocks, block_id, [] {}, [&](const double(&s)[NQ]) {
     fin(s);
     *ticket = 0u;
-  }
+  }, [] {});
+}
+
+constexpr int kStateWords = (int)(sizeof(SolveState) / 4);
+
+// The same for the reductions of a solve: the last block brings the solve's state to shared memory (`scratch`,
+// kStateWords words), fin(state, sums) runs on that copy in thread 0, and the block writes it back.  A finalize reads
+// and writes some twenty words one after another; from global memory that is most of its time.
+template <int NQ, class Fin>
+__device__ __forceinline__ void grid_reduce_state(double (&v)[NQ], double* partials, SolveState* st, int ticket,
+                                                  int nblocks, int block_id, unsigned* scratch, Fin fin) {
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const int nthreads = blockDim.x * blockDim.y * blockDim.z;
+  SolveState* copy = reinterpret_cast<SolveState*>(scratch);
+  grid_reduce_impl<NQ>(
+      v, partials, &st->tickets[ticket], nblocks, block_id,
+      [&] {
+        for (int i = tid; i < kStateWords; i += nthreads) scratch[i] = __ldcg(reinterpret_cast<const unsigned*>(st) + i);
+      },
+      [&](const double(&s)[NQ]) {
+        fin(copy, s);
+        copy->tickets[ticket] = 0u;
+      },
+      [&] {
+        __syncthreads();
+        for (int i = tid; i < kStateWords; i += nthreads) reinterpret_cast<unsigned*>(st)[i] = scratch[i];
+      });
 }
 
 // Finalize of one preconditioner application inside PCG (Algorithm 1):
