@@ -1816,12 +1816,19 @@ void launch_apply_laplacian(const tpcg_plan* p, const Geom& g, const double* x, 
 }
 // Persistent grids of the fixed-point sweeps: every SM holds as many blocks as
 // the kernel's resources allow (at most 8), and every block takes at least
-// sweep_grain (tile, plane) pairs; the grid-stride kernels at most 8 blocks per
+// sweep_grain (tile, plane) pairs (fewer where a default grain leaves SMs idle); the grid-stride kernels at most 8 blocks per
 // SM of at least 256 * sweep_grain points.  A small grid thus leaves SMs to the
 // kernels of other plans.
 int setup_fx_grids(tpcg_plan* p) {
-  const long long grain = p->sweep_grain;
-  p->stream_blocks = (int)std::max(1LL, std::min<long long>((p->N + 256 * grain - 1) / (256 * grain),
+  // The default grain of 4 gives way where it would leave SMs without a block: a small grid's time is the chain of
+  // planes of one block (64 x 64 plane 105 -> 95 us, 64 x 64 x 32 step 230 -> 220 at grain 1-2; 96 x 96 x 48 is 2 % slower
+  // below 4).  A grain that the caller has set is kept.
+  auto grain_of = [&](long long units) {
+    const long long g = p->sweep_grain;
+    return p->sweep_grain_set ? g : std::max(1LL, std::min(g, units / p->num_sms));
+  };
+  const long long sg = grain_of((p->N + 255) / 256);
+  p->stream_blocks = (int)std::max(1LL, std::min<long long>((p->N + 256 * sg - 1) / (256 * sg),
                                                            (long long)p->num_sms * 8));
   const bool f64 = p->prec == TPCG_FP64;
   const bool pair = !f64 && p->nx % 2 == 0;  // direction and update take two x points per thread
@@ -1838,6 +1845,7 @@ int setup_fx_grids(tpcg_plan* p) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[i], TX * TY, 0) != cudaSuccess) return -1;
     per_sm = std::max(1, std::min(per_sm, 8));
+    const long long grain = grain_of(T);
     p->fx_blocks[i] = (int)std::max(1LL, std::min<long long>((T + grain - 1) / grain, (long long)p->num_sms * per_sm));
   }
   return 0;

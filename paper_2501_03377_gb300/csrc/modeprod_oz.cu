@@ -145,12 +145,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
-  return p != 0;
-}
-
 // v * 2^e rounded once to FP64 (|v| < 2^63); outside the normal range by the general scaling.
 __device__ __forceinline__ double scaled_i64(long long v, int e) {
   if (e > -900 && e < 900) return i64_to_f64_scaled_hw(v, e);
@@ -253,7 +247,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
       // clocks each, twice what the tensor pipe needs (71 on average, max(N / 2, 32 + N / 4)).
       const bool lead = elect_one();
       const unsigned long long dW = sw128_desc(sW), dX = sw128_desc(sX);
-      auto wait_all = [&](uint32_t bar, uint32_t par) { return __all_sync(0xffffffffu, wait_bounded(bar, par, ab)) != 0; };
+      auto wait_all = [&](uint32_t bar, uint32_t par) { return wait_bounded_warp(bar, par, ab); };
       bool ok = true;
       uint32_t kts = 0;             // K tiles so far
       uint32_t ws = 0, wpar = 0;    // ring stage of the next image and its parity

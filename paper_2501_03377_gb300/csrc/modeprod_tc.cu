@@ -45,16 +45,21 @@ namespace tpcg {
 namespace {
 using namespace tcx;
 
+// The split form's operand type: x carried as two BF16 planes, hi = bf16(x) and lo = bf16(x - hi).  A stage
+// holds the hi tile and then the lo tile of the data (and of the eigenbasis), and every K step issues three
+// MMAs into one FP32 accumulator: hi.hi + lo.hi + hi.lo (the lo.lo term, 2^-16 relative, is dropped).
+struct Bf16Pair {};
+
 // Warp roles: warp 0 TMA of the operand, warp 1 MMA, then the epilogue warps, one group of four per
 // share of the accumulator's 16-column chunks (a warp may only read its TMEM lane quadrant, warp % 4).
 // The plain passes use sixteen epilogue warps; the last pass of a solve keeps eight, plus one warp
 // that stages R by TMA.
-template <bool FINAL>
+template <bool FINAL, bool SPLIT>
 struct TcWarps {
-  static constexpr int epi = FINAL ? 8 : 16;
+  static constexpr int epi = (FINAL && !SPLIT) ? 8 : 16;
   static constexpr int groups = epi / 4;
-  static constexpr int threads = (2 + epi + (FINAL ? 1 : 0)) * 32;
-  static constexpr int rwarp = FINAL ? 2 + epi : -1;
+  static constexpr int threads = (2 + epi + (FINAL && !SPLIT ? 1 : 0)) * 32;
+  static constexpr int rwarp = (FINAL && !SPLIT) ? 2 + epi : -1;
 };
 constexpr int kRSlots = 16;                // R chunks in flight (last pass): eight slots per epilogue half
 constexpr int kRHalf = kRSlots / 2;
@@ -63,10 +68,6 @@ constexpr int kTileRows = 128;
 constexpr int kKTile = 64;                 // BF16 elements per 128-byte swizzle row
 constexpr int kStageBytes = kTileRows * 128;
 
-// The split form's operand type: x carried as two BF16 planes, hi = bf16(x) and lo = bf16(x - hi).  A stage
-// holds the hi tile and then the lo tile of the data (and of the eigenbasis), and every K step issues three
-// MMAs into one FP32 accumulator: hi.hi + lo.hi + hi.lo (the lo.lo term, 2^-16 relative, is dropped).
-struct Bf16Pair {};
 
 // Elements of InT per 128-byte swizzle row (one K tile) and per MMA K step.
 template <class InT>
@@ -282,7 +283,7 @@ __device__ __forceinline__ void store_rows_transposed(const TcArgs& a, int lane,
 // ODD: unaligned runs of outputs (TcArgs::stg), stored transposed; an instantiation of its own, since its code costs
 // the aligned one registers (the 256 x 256 x 128 solve took 1 % longer with both in one kernel).
 template <int FORM, class InT, class OutT, bool FINAL, bool ODD>
-__global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
+__global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::threads, 1)
     k_modeprod_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                   const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmO, TcArgs a) {
   if (a.first) asm volatile("griddepcontrol.wait;" ::: "memory");  // the kernel before may set `done`
@@ -329,13 +330,13 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull(b), 1);
-      mbar_init(tempty(b), TcWarps<FINAL>::epi * 32);
+      mbar_init(tempty(b), TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::epi * 32);
     }
     mbar_init(vbar, 1);
     mbar_init(drain, 1);
     for (int s = 0; s < kRSlots; ++s) {
       mbar_init(rfull(s), 1);
-      mbar_init(rempty(s), TcWarps<FINAL>::epi * 16);  // the warps of one epilogue half
+      mbar_init(rempty(s), TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::epi * 16);  // the warps of one epilogue half
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -401,27 +402,26 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
+    {
+      // ---------------- MMA issuer (see elect_one)
+      const bool lead = elect_one();
       constexpr uint32_t fmt = KS::tf32 ? 2u : (std::is_same<InT, __half>::value ? 0u : 1u);
       const uint32_t idesc = (FORM == 1) ? idesc_f16kind(128, a.Np, fmt) : idesc_f16kind(128, 128, fmt);
       // Shared-memory descriptors: the address field holds address / 16 in its low 14 bits (shared memory
       // is below 256 KB, so offsets add without a carry out of the field); a 16-element K step is +2.
-      // The issue loop is kept short: one thread issuing small MMAs is otherwise slower than the tensor
-      // pipe executing them.
       const unsigned long long dX0 = sw128_desc(sD), dV0 = sw128_desc(sV);
       const uint32_t vkt = (uint32_t)(a.VR * 128) >> 4;  // one 64-wide K tile of V
       const bool two_mb = (FORM != 1) && a.MB > 1;       // second 128-row block of V (form 2)
-      bool ok = a.wstream ? true : wait_bounded(vbar, 0, ab);
+      bool ok = a.wstream ? true : wait_bounded_warp(vbar, 0, ab);
       int it = 0, tcount = 0;
       for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++tcount) {
         const int b = tcount & 1;
-        if (!(ok = wait_bounded(tempty(b), (uint32_t)(((tcount >> 1) & 1) ^ 1), ab))) break;
+        if (!(ok = wait_bounded_warp(tempty(b), (uint32_t)(((tcount >> 1) & 1) ^ 1), ab))) break;
         tc_fence_after();
         const uint32_t dacc = tmem + (uint32_t)(b * a.acc_cols);
         for (int kt = 0; kt < a.KT; ++kt, ++it) {
           const int s = it % NS;
-          if (!(ok = wait_bounded(full(s), (uint32_t)((it / NS) & 1), ab))) break;
+          if (!(ok = wait_bounded_warp(full(s), (uint32_t)((it / NS) & 1), ab))) break;
           tc_fence_after();
           const unsigned long long xd = dX0 + (uint32_t)s * (sbytes >> 4);
           // a streamed eigenbasis tile follows the data tile(s) of the stage
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
           };
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
-            if (kk < nk) {
+            if (lead && kk < nk) {
               const uint32_t accum = (kt > 0 || kk > 0) ? 1u : 0u;
               if (FORM == 1) {
                 mma(dacc, xd + 2u * kk, vd + 2u * kk, accum);
@@ -461,19 +461,23 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
               }
             }
           }
-          tc_commit(empty(s));
+          if (lead) tc_commit(empty(s));
+          __syncwarp();
         }
         if (!ok) break;
-        tc_commit(tfull(b));
+        if (lead) tc_commit(tfull(b));
+        __syncwarp();
       }
       // all MMAs issued by this thread are complete once `drain` fires
-      tc_commit(drain);
-      const unsigned long long t0 = gtimer();
-      while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+      if (lead) {
+        tc_commit(drain);
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+        }
       }
     }
     __syncwarp();
-  } else if (warp == TcWarps<FINAL>::rwarp) {
+  } else if (warp == TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::rwarp) {
     // ---------------- TMA of R~ (last pass): 16-column chunks of the tile's 128 rows.  Chunk ci belongs to
     // epilogue half ci % 2, which consumes its chunks in order from its own ring of kRHalf slots (a ring
     // shared by both halves would let one half run a phase ahead of a slot and read it early).  Slot s of
@@ -510,7 +514,7 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
     __syncwarp();
   } else if (warp >= 2) {
     // ---------------- epilogue: NG warps per TMEM lane quadrant, each taking every NG-th 16-column chunk
-    constexpr int NG = TcWarps<FINAL>::groups;
+    constexpr int NG = TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::groups;
     const int q = warp & 3;          // TMEM lane quadrant this warp may access
     const int h = (warp - 2) >> 2;   // which share of the column chunks
     // TMA store of one [32][16] box from this warp's two staging buffers (used alternately; a buffer is
@@ -738,19 +742,16 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
           // R~ of the next chunk is on its way while this one is processed; the accumulator's chunk is loaded when
           // needed (tens of clocks against the some eight hundred of R~, which, waited for chunk by chunk, made this
           // pass twice as long as the others: 42 against 22 us at 256 x 256 x 128)
-          uint32_t rw2[8], rw3[8];
           fetch_pair(0, rw0, rw1);
-          for (int j = 0; j < J; j += 2) {
+#pragma unroll 1
+          for (int j = 0; j < J; ++j) {
+            uint32_t rw2[8], rw3[8];
             tc_ld16_issue(tacc + (uint32_t)col(j), tA);
             fetch_pair(j + 1, rw2, rw3);
             tc_ld16_wait(tA);
             process(col(j), tA, rA, rw0, rw1);
-            if (j + 1 < J) {
-              tc_ld16_issue(tacc + (uint32_t)col(j + 1), tA);
-              fetch_pair(j + 2, rw0, rw1);
-              tc_ld16_wait(tA);
-              process(col(j + 1), tA, rA, rw2, rw3);
-            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) rw0[i] = rw2[i], rw1[i] = rw3[i];
           }
         } else if (rtma) {
           bool ok = true;
@@ -855,14 +856,14 @@ __global__ void __launch_bounds__(TcWarps<FINAL>::threads, 1)
   }
   if constexpr (FINAL) {
     // max |Z| of the block -> one atomicMax (order-independent, so deterministic)
-    __shared__ float smax[TcWarps<FINAL>::threads / 32];
+    __shared__ float smax[TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::threads / 32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
     if (lane == 0) smax[warp] = zmax;
     __syncthreads();
     if (threadIdx.x == 0) {
       float m = 0.0f;
-      for (int w = 0; w < TcWarps<FINAL>::threads / 32; ++w) m = fmaxf(m, smax[w]);
+      for (int w = 0; w < TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::threads / 32; ++w) m = fmaxf(m, smax[w]);
       atomicMax(&a.st->zmax_bits, __float_as_uint(m));
     }
     double acc[2] = {acc_value(red0), acc_value(red1)};
@@ -1300,45 +1301,48 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer (BF16 operands; the order of the per-pass split kernel)
+    {
+      // ---------------- MMA issuer (BF16 operands; the order of the per-pass split kernel; see elect_one)
+      const bool lead = elect_one();
       // stage 2: A (W1 read as W2) MN-major, transpose-A bit
       const uint32_t idesc1 = idesc_f16kind(128, a.Np, 1u), idesc2 = idesc_f16kind(128, 128, 1u) | (1u << 15);
       const unsigned long long dX0 = sw128_desc(sD), dW1 = sw128_desc(sW1), dT = sw128_desc(sT);
       // lo planes: one tile after the hi tile of the same K tile (descriptor units of 16 bytes)
       const uint32_t xlo = (uint32_t)kStageBytes >> 4, w1lo = (uint32_t)(a.VR * 128) >> 4,
                      tlo = (uint32_t)kTBytes >> 4;
-      bool ok = wait_bounded(vbar, 0, ab);
+      bool ok = wait_bounded_warp(vbar, 0, ab);
       int it = 0;
       auto stage1 = [&](int i) {  // forward product of tile i into D1[i & 1]
         const int b = i & 1;
-        if (!wait_bounded(d1empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
+        if (!wait_bounded_warp(d1empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
         tc_fence_after();
         const uint32_t dacc = tmem + (uint32_t)(b * 128);
         for (int kt = 0; kt < KT; ++kt, ++it) {
           const int s = it % NS;
-          if (!wait_bounded(full(s), (uint32_t)((it / NS) & 1), ab)) return false;
+          if (!wait_bounded_warp(full(s), (uint32_t)((it / NS) & 1), ab)) return false;
           tc_fence_after();
           const unsigned long long xd = dX0 + (uint32_t)s * (sbytes >> 4);
           const unsigned long long wd = dW1 + (uint32_t)kt * (w1kt >> 4);
           const int nk = min(4, (a.C - kt * kKTile + 15) >> 4);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
-            if (kk < nk) {
+            if (lead && kk < nk) {
               tc_mma(dacc, xd + 2u * kk, wd + 2u * kk, idesc1, (kt > 0 || kk > 0) ? 1u : 0u);
               tc_mma(dacc, xd + xlo + 2u * kk, wd + 2u * kk, idesc1, 1u);
               tc_mma(dacc, xd + 2u * kk, wd + w1lo + 2u * kk, idesc1, 1u);
             }
           }
-          tc_commit(empty(s));
+          if (lead) tc_commit(empty(s));
+          __syncwarp();
         }
-        tc_commit(d1full(b));
+        if (lead) tc_commit(d1full(b));
+        __syncwarp();
         return true;
       };
       auto stage2 = [&](int i) {  // backward product of tile i (T in shared memory) into D2[i & 1]
         const int b = i & 1;
-        if (!wait_bounded(tready(b), (uint32_t)((i >> 1) & 1), ab)) return false;
-        if (!wait_bounded(d2empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
+        if (!wait_bounded_warp(tready(b), (uint32_t)((i >> 1) & 1), ab)) return false;
+        if (!wait_bounded_warp(d2empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
         tc_fence_after();
         const uint32_t dacc = tmem + 256u + (uint32_t)(b * 128);
         for (int kt = 0; kt < KT; ++kt) {
@@ -1346,7 +1350,7 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
           const int nk = min(4, (a.C - kt * kKTile + 15) >> 4);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
-            if (kk < nk) {
+            if (lead && kk < nk) {
               // K step kg: rows 16 kg.. of every W1 tile (two row groups of 1024 bytes each); the M atoms
               // (W1's K tiles) w1kt bytes apart; lo rows VR * 128 bytes after the hi rows
               const uint32_t ka = sW1 + 2048u * (uint32_t)(kt * 4 + kk);
@@ -1358,7 +1362,8 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
             }
           }
         }
-        tc_commit(d2full(b));
+        if (lead) tc_commit(d2full(b));
+        __syncwarp();
         return true;
       };
       if (ok && nmine > 0) ok = stage1(0);
@@ -1366,9 +1371,11 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
         if (i + 1 < nmine && !(ok = stage1(i + 1))) break;
         ok = stage2(i);
       }
-      tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
-      const unsigned long long t0 = gtimer();
-      while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+      if (lead) {
+        tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+        }
       }
     }
     __syncwarp();
@@ -1678,7 +1685,7 @@ template <int FORM, class InT, class OutT, bool FINAL>
 void launch(const TcStage& s, const TcArgs& a, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)s.grid);
-  cfg.blockDim = dim3(TcWarps<FINAL>::threads);
+  cfg.blockDim = dim3(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::value>::threads);
   cfg.dynamicSmemBytes = s.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -1849,8 +1856,8 @@ int tc_plan_setup(tpcg_plan* p) {
     a.oplane = (long long)p->t_plane;
     a.rplane = (long long)p->lp_plane;
     // staging bytes: two [32][16] boxes per epilogue warp (sixteen warps; eight in the last pass of a solve)
-    const size_t stage_plain = a.tstore ? (size_t)TcWarps<false>::epi * 2 * 32 * 16 * esz : 0;
-    const size_t stage_final = (a.tstore && last) ? (size_t)TcWarps<true>::epi * 2 * 32 * 16 * esz : 0;
+    const size_t stage_plain = a.tstore ? (size_t)TcWarps<false, false>::epi * 2 * 32 * 16 * esz : 0;
+    const size_t stage_final = (a.tstore && last) ? (size_t)TcWarps<true, false>::epi * 2 * 32 * 16 * esz : 0;
     // last pass of a solve: R~ (the first pass's input, rows of pitch pitch16[0], a multiple of 8
     // elements) by TMA through the largest ring (up to kRHalf slots per half) that leaves two stages
     a.rpitch = p->pitch16[0];

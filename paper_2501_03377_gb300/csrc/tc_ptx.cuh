@@ -117,6 +117,19 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// One lane of the (converged) warp.  MMA issue loops are walked by the whole warp with this lane issuing: with
+// warp-uniform control flow the descriptors stay in uniform registers, where a loop of one lane moves each of them over
+// for every MMA and issues slower than the tensor pipe executes.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+// wait_bounded by a whole warp, with one answer for all its lanes.
+__device__ __forceinline__ bool wait_bounded_warp(uint32_t bar, uint32_t parity, const Abort& ab) {
+  return __all_sync(0xffffffffu, wait_bounded(bar, parity, ab)) != 0;
+}
+
 // TMEM -> registers, 16 columns of the thread's lane, in split form for
 // software pipelining: issue the load, do other work, then wait.  The wait names the destination registers as in/out
 // operands, so the compiler cannot read them before the load has landed.

@@ -178,6 +178,7 @@ struct tpcg_plan {
 
   // launch configuration (fixed per plan so that reductions are reproducible)
   dim3 st_block;            // stencil kernels
+  bool sweep_grain_set = false;  // the caller chose the grain
   int sweep_grain = 4;  // TPCG_OPT_SWEEP_GRAIN: least (tile, plane) pairs (x 256 points) per sweep block
   int fx_blocks[tpcg::kFxCount] = {1, 1, 1, 1, 1};  // FxKernel -> blocks of the persistent fixed-point sweeps
   // comparator preconditioner of the FP64 form (TPCG_PRECOND_*), Jacobi(p, omega) and its table of
