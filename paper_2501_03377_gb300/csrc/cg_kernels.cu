@@ -12,6 +12,7 @@
 // ("ghost") values: periodic wraps, Dirichlet reads 0, Neumann mirrors the
 // boundary value -- which reproduces the corner entries (alpha, beta, gamma) of
 // eq. (lap1d) exactly.
+#include <cmath>
 #include <cstdio>
 
 #include "tpcg_dev.cuh"
@@ -346,10 +347,11 @@ __global__ void __launch_bounds__(TX* TY) k_apply_laplacian(Geom g, const double
 __device__ __forceinline__ unsigned long long mag_key(double u) {
   return (unsigned long long)__double_as_longlong(u) << 1;
 }
-__device__ __forceinline__ void fold_umax(SolveState* st, unsigned long long um) {
-  const unsigned long long m = block_max_u64(um);
-  if (threadIdx.x + threadIdx.y == 0) atomicMax(&st->umax_bits, m >> 1);
+__device__ __forceinline__ void fold_max(unsigned long long* word, unsigned long long key) {
+  const unsigned long long m = block_max_u64(key);
+  if (threadIdx.x + threadIdx.y == 0) atomicMax(word, m >> 1);
 }
+__device__ __forceinline__ void fold_umax(SolveState* st, unsigned long long um) { fold_max(&st->umax_bits, um); }
 
 // ------------------------------------------------------------------ residual R = eta_hat - L U
 // The initial residual (Algorithm 1) and the check of the true
@@ -369,14 +371,14 @@ struct OpResidualFx {
   double* __restrict__ R;
   LowPrec lp;
   double mean, nih0, nih1, nih2;  // -1/h^2 per axis
-  int shift, sr, ku, uniform;
+  int shift, sr, ku, uniform, sub;  // sub: a mean is removed
   float rr, sR;
   double ee;  // ||eta_hat||^2 in FP64: it scales the tolerance and is reported
   long long su;
   __device__ __forceinline__ void operator()(unsigned i, int, int, int, double eta_i, long long c, long long xl,
                                              long long xr, long long yl, long long yr, long long zl, long long zr) {
     const long long dx = 2 * c - xl - xr, dy = 2 * c - yl - yr, dz = 2 * c - zl - zr;
-    const double e = eta_i - mean;
+    const double e = sub ? eta_i - mean : eta_i;
     double r;
     if (uniform) {
       r = fma(nih0, i64_to_f64_scaled_hw(dx + dy + dz, -ku), e);
@@ -470,7 +472,7 @@ __global__ void __launch_bounds__(TX* TY) k_residual_fx(Geom g, const double* __
   const int ku = st->ku, sr = st->sr;
   FieldFixed64 f{U, ku};
   OpResidualFx<INIT> op{eta, R, lp, st->mean_eta, g.nih2[0], g.nih2[1], g.nih2[2], st->lp_shift, sr, ku, g.uniform,
-                        0.0f, 0.0f, 0.0, 0};
+                        st->singular, 0.0f, 0.0f, 0.0, 0};
   const long long N = g.N;
   const bool finite_u = isfinite(st->umax);
   stencil_sweep_fx<long long, 4>(
@@ -1371,9 +1373,10 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_pair(Geom g, double* __r
 }
 
 // FP64 form: P and W = L P are stored by the direction kernel.
+template <bool PAIR>
 __global__ void __launch_bounds__(256) k_update(Geom g, double* __restrict__ U, const double* __restrict__ P0,
                                                 const double* __restrict__ P1, const double* __restrict__ W,
-                                                double* __restrict__ R, LowPrec lp, SolveState* st, double* partials) {
+                                                double* __restrict__ R, SolveState* st, double* partials) {
   const long long N = g.N;
   if (paused(st)) return;
   const double* __restrict__ P = (st->iter & 1) ? P1 : P0;
@@ -1385,18 +1388,33 @@ __global__ void __launch_bounds__(256) k_update(Geom g, double* __restrict__ U, 
   const int shift = st->lp_shift;
   float a0 = 0.0f, a1 = 0.0f;
   unsigned long long um = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const double p = __ldg(P + i);
-    const double u = zg ? alpha * p : fma(alpha, p, U[i]);
-    U[i] = u;
+  auto point = [&](double p, double w, double& u, double& r) {
+    u = zg ? alpha * p : fma(alpha, p, u);
     const unsigned long long ub = mag_key(u);
     um = ub > um ? ub : um;
-    const double r = fma(nalpha, __ldg(W + i), R[i]);
-    R[i] = r;
+    r = fma(nalpha, w, r);
     const float r32 = f64_to_f32_odd(r, shift);
-    store_lp(lp, i, r, r32);
     a0 = fmaf(r32, r32, a0);
     a1 += r32;
+  };
+  if constexpr (PAIR) {  // two adjacent points per thread (N even, U 16-byte aligned)
+    const unsigned npair = (unsigned)(N / 2), stride = gridDim.x * blockDim.x;
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < npair; t += stride) {
+      const double2 p = __ldg(reinterpret_cast<const double2*>(P) + t), w = __ldg(reinterpret_cast<const double2*>(W) + t);
+      double2 u = zg ? make_double2(0.0, 0.0) : reinterpret_cast<const double2*>(U)[t];
+      double2 r = reinterpret_cast<const double2*>(R)[t];
+      point(p.x, w.x, u.x, r.x);
+      point(p.y, w.y, u.y, r.y);
+      reinterpret_cast<double2*>(U)[t] = u;
+      reinterpret_cast<double2*>(R)[t] = r;
+    }
+  } else {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+      double u = zg ? 0.0 : U[i], r = R[i];
+      point(__ldg(P + i), __ldg(W + i), u, r);
+      U[i] = u;
+      R[i] = r;
+    }
   }
   fold_umax(st, um);
   double acc[2] = {f32_to_f64_int(a0), f32_to_f64_int(a1)};
@@ -1408,7 +1426,10 @@ __global__ void __launch_bounds__(256) k_update(Geom g, double* __restrict__ U, 
 // ------------------------------------------------------------------ streaming kernels
 // R = eta_hat (zero initial guess: U_0 = 0 in Algorithm 1); ||eta_hat||^2 in
 // FP64 (it scales the tolerance and is reported), sum(R) in FP32 from
-// R * 2^lp_shift.
+// R * 2^lp_shift.  SUB: a mean is removed (singular operators).  PAIR: two
+// adjacent points per thread, 16-byte accesses.  One or two FP64 operations per
+// point bound it (27 us each at 256 x 256 x 128).
+template <bool SUB, bool PAIR>
 __global__ void __launch_bounds__(256) k_init_zero(long long N, const double* __restrict__ eta,
                                                    double* __restrict__ R, LowPrec lp, SolveState* st,
                                                    double* partials) {
@@ -1418,13 +1439,26 @@ __global__ void __launch_bounds__(256) k_init_zero(long long N, const double* __
   const int shift = st->lp_shift;
   double e2 = 0.0;
   float a1 = 0.0f;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const double r = __ldg(eta + i) - mean;
-    R[i] = r;
-    const float r32 = f64_to_f32_odd(r, shift);
-    store_lp(lp, i, r, r32);
-    e2 = fma(r, r, e2);
-    a1 += r32;
+  if constexpr (PAIR) {
+    const unsigned npair = (unsigned)(N / 2), stride = gridDim.x * blockDim.x;
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < npair; t += stride) {
+      const double2 e = __ldg(reinterpret_cast<const double2*>(eta) + t);
+      const double r0 = SUB ? e.x - mean : e.x, r1 = SUB ? e.y - mean : e.y;
+      reinterpret_cast<double2*>(R)[t] = make_double2(r0, r1);
+      const float a32 = f64_to_f32_odd(r0, shift), b32 = f64_to_f32_odd(r1, shift);
+      store_lp_pair(lp, 2ll * t, r0, r1, a32, b32);
+      e2 = fma(r0, r0, fma(r1, r1, e2));
+      a1 += a32 + b32;
+    }
+  } else {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+      const double e = __ldg(eta + i), r = SUB ? e - mean : e;
+      R[i] = r;
+      const float r32 = f64_to_f32_odd(r, shift);
+      store_lp(lp, i, r, r32);
+      e2 = fma(r, r, e2);
+      a1 += r32;
+    }
   }
   double acc[2] = {e2, f32_to_f64_int(a1)};
   __shared__ __align__(16) unsigned scratch[kStateWords];
@@ -1435,35 +1469,69 @@ __global__ void __launch_bounds__(256) k_init_zero(long long N, const double* __
   });
 }
 
-// sum(eta) and sum(eta^2): the mean removed by eq. (centering) when the
-// operator is singular, and the exponent of the first low-precision copy;
-// with a given initial guess also max|U_0| for the fixed-point residual.
+// The mean removed by eq. (centering) when the operator is singular (SUM) and the exponent of the first low-precision
+// copy, from the 2-norm where the copy's range needs it (SQ: the FP16 form), else from max|eta|, an integer operation:
+// the other forms' copies and FP32 sums are the same for any power of two that keeps them in range.  The sums take an
+// FP64 operation per point each (both: 43 us at 256 x 256 x 128, of which the memory needs 10).  With a given initial
+// guess also max|U_0| for the fixed-point residual.  PAIR: two adjacent points per thread.
+template <bool SUM, bool SQ, bool PAIR>
 __global__ void __launch_bounds__(256) k_eta_sum(Geom g, const double* __restrict__ eta,
                                                  const double* __restrict__ U0, SolveState* st, double* partials) {
   // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
   eta = st->eta;
   if (U0) U0 = st->ups;  // (NULL: zero initial guess)
   const long long N = g.N;
-  double acc[2] = {0.0, 0.0};
-  unsigned long long um = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const double e = __ldg(eta + i);
-    acc[0] += e;
-    acc[1] = fma(e, e, acc[1]);
-    if (U0) {
-      const unsigned long long ub = mag_key(__ldg(U0 + i));
-      um = ub > um ? ub : um;
+  double s1 = 0.0, s2 = 0.0;
+  unsigned long long um = 0, em = 0;
+  auto max_key = [](unsigned long long m, double v) {
+    const unsigned long long k = mag_key(v);
+    return k > m ? k : m;
+  };
+  auto take = [&](double e) {
+    if constexpr (SUM) s1 += e;
+    if constexpr (SQ) s2 = fma(e, e, s2);
+    else em = max_key(em, e);
+  };
+  if constexpr (PAIR) {
+    const unsigned npair = (unsigned)(N / 2), stride = gridDim.x * blockDim.x;
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < npair; t += stride) {
+      const double2 e = __ldg(reinterpret_cast<const double2*>(eta) + t);
+      take(e.x);
+      take(e.y);
+      if (U0) {
+        const double2 u = __ldg(reinterpret_cast<const double2*>(U0) + t);
+        um = max_key(max_key(um, u.x), u.y);
+      }
+    }
+  } else {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+      take(__ldg(eta + i));
+      if (U0) um = max_key(um, __ldg(U0 + i));
     }
   }
-  fold_umax(st, um);
+  if (U0) fold_max(&st->umax_bits, um);
+  if constexpr (!SQ) fold_max(&st->emax_bits, em);
+  constexpr int NQ = (SUM && SQ) ? 2 : 1;
+  double acc[NQ];
+  acc[0] = SUM ? s1 : s2;
+  if constexpr (NQ == 2) acc[1] = s2;
   __shared__ __align__(16) unsigned scratch[kStateWords];
-  grid_reduce_state<2>(acc, partials, st, kTkEta, gridDim.x, blockIdx.x, scratch,
-                       [N, g](SolveState* st, const double(&s)[2]) {
-    const double mean = st->singular ? s[0] / (double)N : 0.0;
+  grid_reduce_state<NQ>(acc, partials, st, kTkEta, gridDim.x, blockIdx.x, scratch,
+                        [N, g](SolveState* st, const double(&s)[NQ]) {
+    const double mean = SUM ? s[0] / (double)N : 0.0;
     st->mean_eta = mean;
-    const double n2 = s[1] - mean * s[0];
-    st->eta_norm2 = n2 > 0.0 ? n2 : s[1];  // estimate; the initial residual kernel sets the exact value
-    st->lp_shift = lp_shift_for(n2 > 0.0 ? n2 : s[1], N);
+    // eta_norm2: an estimate or bound; the initial residual kernel sets the exact value
+    if constexpr (SQ) {
+      const double sq = s[NQ - 1], n2 = SUM ? sq - mean * s[0] : sq;
+      st->eta_norm2 = n2 > 0.0 ? n2 : sq;
+      st->lp_shift = lp_shift_for(n2 > 0.0 ? n2 : sq, N);
+    } else {  // |eta - mean| <= 2 max|eta|
+      const double emax = __longlong_as_double((long long)st->emax_bits);
+      st->emax_bits = 0ull;
+      st->eta_norm2 = fmin(4.0 * (double)N * emax * emax, 8.0e307);
+      const int k = (emax > 0.0 && isfinite(emax)) ? -ilogb_pos(emax) - 2 : 0;
+      st->lp_shift = k < -120 ? -120 : (k > 120 ? 120 : k);
+    }
     st->umax = __longlong_as_double((long long)st->umax_bits);
     st->umax_bits = 0ull;
     plan_residual_check(st, g);
@@ -1551,73 +1619,6 @@ __global__ void __launch_bounds__(256) k_form_u(Geom g, double* __restrict__ U, 
   });
 }
 
-// k_init_zero and k_eta_sum with two adjacent points per thread (N even and
-// below 2^32; nx even when there is a low-precision copy, so a pair never
-// straddles a padded row): 16-byte loads and stores and 32-bit indices.
-__global__ void __launch_bounds__(256) k_init_zero2(unsigned npair, long long N, const double* __restrict__ eta,
-                                                    double* __restrict__ R, LowPrec lp, SolveState* st,
-                                                    double* partials) {
-  // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
-  eta = st->eta;
-  const double mean = st->mean_eta;
-  const int shift = st->lp_shift;
-  double e2 = 0.0;
-  float a1 = 0.0f;
-  const unsigned stride = gridDim.x * blockDim.x;
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < npair; t += stride) {
-    const double2 e = __ldg(reinterpret_cast<const double2*>(eta) + t);
-    const double r0 = e.x - mean, r1 = e.y - mean;
-    reinterpret_cast<double2*>(R)[t] = make_double2(r0, r1);
-    const float a32 = f64_to_f32_odd(r0, shift), b32 = f64_to_f32_odd(r1, shift);
-    store_lp_pair(lp, 2ll * t, r0, r1, a32, b32);
-    e2 = fma(r0, r0, fma(r1, r1, e2));
-    a1 += a32 + b32;
-  }
-  double acc[2] = {e2, f32_to_f64_int(a1)};
-  __shared__ __align__(16) unsigned scratch[kStateWords];
-  grid_reduce_state<2>(acc, partials, st, kTkInit, gridDim.x, blockIdx.x, scratch,
-                       [N, shift](SolveState* st, const double(&s)[2]) {
-    const double v[3] = {s[0], scale_pow2(s[1], -shift), s[0]};
-    fin_init(st, v, N);
-  });
-}
-
-__global__ void __launch_bounds__(256) k_eta_sum2(Geom g, unsigned npair, const double* __restrict__ eta,
-                                                  const double* __restrict__ U0, SolveState* st, double* partials) {
-  // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
-  eta = st->eta;
-  if (U0) U0 = st->ups;  // (NULL: zero initial guess)
-  const long long N = g.N;
-  double acc[2] = {0.0, 0.0};
-  unsigned long long um = 0;
-  const unsigned stride = gridDim.x * blockDim.x;
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < npair; t += stride) {
-    const double2 e = __ldg(reinterpret_cast<const double2*>(eta) + t);
-    acc[0] += e.x;
-    acc[0] += e.y;
-    acc[1] = fma(e.y, e.y, fma(e.x, e.x, acc[1]));
-    if (U0) {
-      const double2 u = __ldg(reinterpret_cast<const double2*>(U0) + t);
-      const unsigned long long a = mag_key(u.x), b = mag_key(u.y);
-      const unsigned long long ub = a > b ? a : b;
-      um = ub > um ? ub : um;
-    }
-  }
-  fold_umax(st, um);
-  __shared__ __align__(16) unsigned scratch[kStateWords];
-  grid_reduce_state<2>(acc, partials, st, kTkEta, gridDim.x, blockIdx.x, scratch,
-                       [N, g](SolveState* st, const double(&s)[2]) {
-    const double mean = st->singular ? s[0] / (double)N : 0.0;
-    st->mean_eta = mean;
-    const double n2 = s[1] - mean * s[0];
-    st->eta_norm2 = n2 > 0.0 ? n2 : s[1];  // estimate; the initial residual kernel sets the exact value
-    st->lp_shift = lp_shift_for(n2 > 0.0 ? n2 : s[1], N);
-    st->umax = __longlong_as_double((long long)st->umax_bits);
-    st->umax_bits = 0ull;
-    plan_residual_check(st, g);
-  });
-}
-
 // ||r||^2 -> exponent of the low-precision copy (tpcg_precond_apply).
 __global__ void __launch_bounds__(256) k_norm_shift(long long N, const double* __restrict__ r, SolveState* st,
                                                     double* partials) {
@@ -1635,12 +1636,23 @@ __global__ void __launch_bounds__(256) k_norm_shift(long long N, const double* _
 // `force` only when the stop test has succeeded: launched behind each chunk of
 // iterations, it centres U in the chunk where that happened (the host issues no
 // further one; every block takes the same decision) and saves the host a round trip.
+template <bool PAIR>
 __global__ void __launch_bounds__(256) k_center_u(long long N, double* __restrict__ U, const SolveState* st,
                                                   int force) {
   if (!force && !(st->done == 1 && st->status == TPCG_OK && st->done_iter > 0)) return;
   // the solve's buffers come from the state (a captured launch sequence serves every solve of the plan)
   U = st->ups;
   const double m = st->sumU / (double)N;
+  if constexpr (PAIR) {
+    const unsigned npair = (unsigned)(N / 2), stride = gridDim.x * blockDim.x;
+    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < npair; t += stride) {
+      double2 u = reinterpret_cast<const double2*>(U)[t];
+      u.x -= m;
+      u.y -= m;
+      reinterpret_cast<double2*>(U)[t] = u;
+    }
+    return;
+  }
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
     U[i] -= m;
 }
@@ -1779,34 +1791,70 @@ struct FaceData {
   double inv2h[3];  // 1 / (2 h)
 };
 
-__global__ void __launch_bounds__(256) k_efield(Geom g, const double* __restrict__ U, FaceData fd,
-                                                double* __restrict__ ex, double* __restrict__ ey,
-                                                double* __restrict__ ez) {
-  const unsigned plane = (unsigned)g.nx * (unsigned)g.ny;  // N <= 2^31: 32-bit index arithmetic
-  const int naxes = g.nz > 1 ? 3 : 2;
-  for (long long ii = blockIdx.x * (long long)blockDim.x + threadIdx.x; ii < g.N;
-       ii += (long long)gridDim.x * blockDim.x) {
-    const unsigned i = (unsigned)ii;
-    const int k = (int)(i / plane);
-    const unsigned rem = i - (unsigned)k * plane;
-    const int y = (int)(rem / (unsigned)g.nx), x = (int)(rem - (unsigned)y * (unsigned)g.nx);
-    const int pos[3] = {x, y, k}, len[3] = {g.nx, g.ny, g.nz};
-    const unsigned stride[3] = {1u, (unsigned)g.nx, plane};
-    const double u0 = __ldg(U + i);
-    for (int m = 0; m < naxes; ++m) {
-      const int bc = g.bc[m];
-      const bool startD = bc == kBcD || bc == kBcDN, endD = bc == kBcD || bc == kBcND;
-      double lo, hi;
-      if (pos[m] > 0) lo = __ldg(U + i - stride[m]);
-      else if (bc == kBcP) lo = __ldg(U + i + (unsigned)(len[m] - 1) * stride[m]);
-      else lo = startD ? fd.v[2 * m] : fma(fd.h[m], fd.v[2 * m], u0);
-      if (pos[m] < len[m] - 1) hi = __ldg(U + i + stride[m]);
-      else if (bc == kBcP) hi = __ldg(U + i - (unsigned)(len[m] - 1) * stride[m]);
-      else hi = endD ? fd.v[2 * m + 1] : fma(fd.h[m], fd.v[2 * m + 1], u0);
-      double* out = m == 0 ? ex : (m == 1 ? ey : ez);
-      out[i] = (lo - hi) * fd.inv2h[m];
-    }
+// (lo - hi) * 2^e2 when the factor is a power of two (one FP64 operation, the scaling on the exponent field), else
+// (lo - hi) * f.
+struct FieldScale {
+  double f;
+  int e2;   // exponent of a power of two
+  int pow2;
+};
+__device__ __forceinline__ double scaled_diff(double lo, double hi, const FieldScale& s) {
+  const double d = lo - hi;
+  if (s.pow2) {
+    const int h = __double2hiint(d), e = (h >> 20) & 0x7ff, n = e + s.e2;
+    if (e != 0 && e != 0x7ff && n > 0 && n < 0x7ff) return __hiloint2double(h + (s.e2 << 20), __double2loint(d));
+    if (d == 0.0) return d;
   }
+  return d * s.f;
+}
+
+// A thread owns the column (x, y) of a 32 x 8 tile and marches in z with the z neighbours in registers (see
+// k_direction_int); the x and y neighbours come from the cache.  Six FP64 operations a point (a difference and a product
+// per axis) bound the plain form: 115 us at 256 x 256 x 128, where the memory needs 39.  With a power of two for
+// 1 / (2 h) the product is an integer operation.
+__global__ void __launch_bounds__(TX* TY) k_efield(Geom g, const double* __restrict__ U, FaceData fd, FieldScale sx,
+                                                   FieldScale sy, FieldScale sz, double* __restrict__ ex,
+                                                   double* __restrict__ ey, double* __restrict__ ez) {
+  const unsigned nx = (unsigned)g.nx, plane = nx * (unsigned)g.ny;  // N <= 2^31: 32-bit index arithmetic
+  const bool has_z = g.nz > 1;
+  // ghost value of axis m at its start (lo) or end: face data of Sec. 3.4.2
+  auto ghost = [&](int m, bool end, double u0) {
+    const int bc = g.bc[m];
+    const bool dir = bc == kBcD || bc == (end ? kBcND : kBcDN);
+    const double v = fd.v[2 * m + (end ? 1 : 0)];
+    return dir ? v : fma(fd.h[m], v, u0);
+  };
+  for_each_run(g, [&](int bx0, int by0, int k0, int k1) {
+    const int x = bx0 + (int)threadIdx.x, y = by0 + (int)threadIdx.y;
+    if (x >= g.nx || y >= g.ny) return;
+    const unsigned col = (unsigned)y * nx + (unsigned)x;
+    const bool px = g.bc[0] == kBcP, py = g.bc[1] == kBcP, pz = g.bc[2] == kBcP;
+    // neighbours inside the grid (periodic faces wrapped); a face of another kind takes its ghost value
+    const bool fxl = x == 0 && !px, fxr = x == g.nx - 1 && !px, fyl = y == 0 && !py, fyr = y == g.ny - 1 && !py;
+    const unsigned cxl = x > 0 ? col - 1 : (px ? col + nx - 1 : col), cxr = x < g.nx - 1 ? col + 1 : (px ? col + 1 - nx : col);
+    const unsigned cyl = y > 0 ? col - nx : (py ? col + plane - nx : col),
+                   cyr = y < g.ny - 1 ? col + nx : (py ? col + nx - plane : col);
+    double c = __ldg(U + (unsigned)k0 * plane + col);
+    double zl = c;
+    if (has_z) zl = k0 > 0 ? __ldg(U + (unsigned)(k0 - 1) * plane + col)
+                           : (pz ? __ldg(U + (unsigned)(g.nz - 1) * plane + col) : ghost(2, false, c));
+#pragma unroll 2
+    for (int k = k0; k < k1; ++k) {
+      const unsigned base = (unsigned)k * plane, i = base + col;
+      double zr = c;
+      if (has_z) zr = k + 1 < g.nz ? __ldg(U + i + plane) : (pz ? __ldg(U + col) : ghost(2, true, c));
+      double xl = __ldg(U + base + cxl), xr = __ldg(U + base + cxr), yl = __ldg(U + base + cyl), yr = __ldg(U + base + cyr);
+      if (fxl) xl = ghost(0, false, c);
+      if (fxr) xr = ghost(0, true, c);
+      if (fyl) yl = ghost(1, false, c);
+      if (fyr) yr = ghost(1, true, c);
+      ex[i] = scaled_diff(xl, xr, sx);
+      ey[i] = scaled_diff(yl, yr, sy);
+      if (has_z) ez[i] = scaled_diff(zl, zr, sz);
+      zl = c;
+      c = zr;
+    }
+  });
 }
 
 // ------------------------------------------------------------------ host launchers
@@ -1838,7 +1886,7 @@ int setup_fx_grids(tpcg_plan* p) {
                                       : (pair ? (const void*)k_direction_pair : (const void*)k_direction_int),
                                pair ? (const void*)k_update_pair : (const void*)k_update_int,
                                (const void*)k_residual_fx<false>, (const void*)k_residual_fx<true>,
-                               (const void*)k_apply_laplacian};
+                               (const void*)k_apply_laplacian, (const void*)k_efield};
   for (int i = 0; i < kFxCount; ++i) {
     const int tw = (i == kFxDir && quad) ? 4 * TX : (((i == kFxUpd || i == kFxDir) && pair) ? 2 * TX : TX);
     const long long T = (long long)((p->nx + tw - 1) / tw) * ((p->ny + TY - 1) / TY) * p->nz;
@@ -1862,23 +1910,35 @@ static bool aligned16(const void* a) { return ((uintptr_t)a & 15) == 0; }
 static bool pairs_ok(const tpcg_plan* p, const Geom& g, const void* a, const void* b) {
   return g.N % 2 == 0 && g.N < (1ll << 32) && (p->d_Rlp == nullptr || g.nx % 2 == 0) && aligned16(a) && aligned16(b);
 }
+template <bool SUB, bool PAIR>
+static void init_zero(const tpcg_plan* p, const Geom& g, const double* eta) {
+  k_init_zero<SUB, PAIR><<<p->stream_blocks, 256, 0, p->stream>>>(g.N, eta, p->d_R, lowprec(p), p->d_state, p->d_partials);
+}
 void launch_init_residual(const tpcg_plan* p, const Geom& g, const double* eta, const double* U, bool zero_guess) {
   LaunchScope ls(p, kKInit);
-  if (zero_guess && pairs_ok(p, g, eta, nullptr))
-    k_init_zero2<<<p->stream_blocks, 256, 0, p->stream>>>((unsigned)(g.N / 2), g.N, eta, p->d_R, lowprec(p),
-                                                          p->d_state, p->d_partials);
-  else if (zero_guess)
-    k_init_zero<<<p->stream_blocks, 256, 0, p->stream>>>(g.N, eta, p->d_R, lowprec(p), p->d_state, p->d_partials);
-  else
+  if (!zero_guess) {
     k_residual_fx<true><<<p->fx_blocks[kFxInit], p->st_block, 0, p->stream>>>(g, eta, U, p->d_R, lowprec(p),
                                                                                p->d_state, p->d_partials, 0);
+  } else if (pairs_ok(p, g, eta, nullptr)) {
+    if (p->singular) init_zero<true, true>(p, g, eta);
+    else init_zero<false, true>(p, g, eta);
+  } else {
+    if (p->singular) init_zero<true, false>(p, g, eta);
+    else init_zero<false, false>(p, g, eta);
+  }
+}
+template <bool SUM, bool SQ>
+static void eta_sum(const tpcg_plan* p, const Geom& g, const double* eta, const double* U0) {
+  if (pairs_ok(p, g, eta, U0))
+    k_eta_sum<SUM, SQ, true><<<p->stream_blocks, 256, 0, p->stream>>>(g, eta, U0, p->d_state, p->d_partials);
+  else
+    k_eta_sum<SUM, SQ, false><<<p->stream_blocks, 256, 0, p->stream>>>(g, eta, U0, p->d_state, p->d_partials);
 }
 void launch_eta_sum(const tpcg_plan* p, const Geom& g, const double* eta, const double* U0) {
   LaunchScope ls(p, kKEtaSum);
-  if (pairs_ok(p, g, eta, U0))
-    k_eta_sum2<<<p->stream_blocks, 256, 0, p->stream>>>(g, (unsigned)(g.N / 2), eta, U0, p->d_state, p->d_partials);
-  else
-    k_eta_sum<<<p->stream_blocks, 256, 0, p->stream>>>(g, eta, U0, p->d_state, p->d_partials);
+  const bool sq = p->lp_kind == 2;
+  if (p->singular) sq ? eta_sum<true, true>(p, g, eta, U0) : eta_sum<true, false>(p, g, eta, U0);
+  else sq ? eta_sum<false, true>(p, g, eta, U0) : eta_sum<false, false>(p, g, eta, U0);
 }
 void launch_norm_shift(const tpcg_plan* p, const Geom& g, const double* r) {
   LaunchScope ls(p, kKConvert);
@@ -1911,8 +1971,11 @@ void launch_direction(const tpcg_plan* p, const Geom& g) {
 void launch_update(const tpcg_plan* p, const Geom& g, double* U, bool zero_guess_first) {
   LaunchScope ls(p, kKUpdate);
   if (p->prec == TPCG_FP64) {
-    k_update<<<p->stream_blocks, 256, 0, p->stream>>>(g, U, (const double*)p->d_P[0], (const double*)p->d_P[1], p->d_W,
-                                                       p->d_R, lowprec(p), p->d_state, p->d_partials);
+    const double *P0 = (const double*)p->d_P[0], *P1 = (const double*)p->d_P[1];
+    if (pairs_ok(p, g, U, nullptr))
+      k_update<true><<<p->stream_blocks, 256, 0, p->stream>>>(g, U, P0, P1, p->d_W, p->d_R, p->d_state, p->d_partials);
+    else
+      k_update<false><<<p->stream_blocks, 256, 0, p->stream>>>(g, U, P0, P1, p->d_W, p->d_R, p->d_state, p->d_partials);
     return;
   }
   const DirRing ring = dir_ring(p);
@@ -1951,7 +2014,10 @@ void launch_true_residual(const tpcg_plan* p, const Geom& g, const double* eta, 
 }
 void launch_center_u(const tpcg_plan* p, const Geom& g, double* U, bool force) {
   LaunchScope ls(p, kKCenter);
-  k_center_u<<<p->stream_blocks, 256, 0, p->stream>>>(g.N, U, p->d_state, force ? 1 : 0);
+  if (g.N % 2 == 0 && g.N < (1ll << 32) && aligned16(U))
+    k_center_u<true><<<p->stream_blocks, 256, 0, p->stream>>>(g.N, U, p->d_state, force ? 1 : 0);
+  else
+    k_center_u<false><<<p->stream_blocks, 256, 0, p->stream>>>(g.N, U, p->d_state, force ? 1 : 0);
 }
 void launch_zero(const tpcg_plan* p, long long N, double* U) {
   LaunchScope ls(p, kKConvert);
@@ -1978,7 +2044,14 @@ void launch_efield(const tpcg_plan* p, const Geom& g, const double* U, const dou
     fd.h[m] = p->h[m];
     fd.inv2h[m] = 0.5 / p->h[m];
   }
-  k_efield<<<p->stream_blocks, 256, 0, p->stream>>>(g, U, fd, ex, ey, ez);
+  FieldScale sc[3];
+  for (int m = 0; m < 3; ++m) {
+    int e = 0;
+    sc[m].f = fd.inv2h[m];
+    sc[m].pow2 = std::frexp(fd.inv2h[m], &e) == 0.5 ? 1 : 0;
+    sc[m].e2 = e - 1;
+  }
+  k_efield<<<p->fx_blocks[kFxField], p->st_block, 0, p->stream>>>(g, U, fd, sc[0], sc[1], sc[2], ex, ey, ez);
 }
 // Comparator preconditioner of the FP64 form: Z = M(R), then (with st) rho, sum(Z) and the finalize.
 void run_precond_cmp(const tpcg_plan* p, const Geom& g, const double* R, double* Z, SolveState* st) {

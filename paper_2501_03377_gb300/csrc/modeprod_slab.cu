@@ -262,19 +262,20 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
+    {
+      // ---------------- MMA issuer (see elect_one)
+      const bool lead = elect_one();
       constexpr uint32_t fmt = std::is_same<InT, __half>::value ? 0u : 1u;
       const uint32_t idesc1 = idesc_f16kind(128, a.N1, fmt), idesc2 = idesc_f16kind(128, a.N2, fmt);
       int it1 = 0, it2 = 0;
       bool ok = true;
       for (int i = 0; ok && i < nmine; ++i) {
-        if (i > 0 && !(ok = wait_bounded(d2empty, (uint32_t)((i - 1) & 1), ab))) break;
+        if (i > 0 && !(ok = wait_bounded_warp(d2empty, (uint32_t)((i - 1) & 1), ab))) break;
         tc_fence_after();
         // step 1: D1[b] = W1 block b . X^T over the K tiles of n
         for (int kt = 0; ok && kt < a.KT1; ++kt, ++it1) {
           const int s = it1 % NS1;
-          if (!(ok = wait_bounded(full1(s), (uint32_t)((it1 / NS1) & 1), ab))) break;
+          if (!(ok = wait_bounded_warp(full1(s), (uint32_t)((it1 / NS1) & 1), ab))) break;
           tc_fence_after();
           const uint32_t st = sR1 + (uint32_t)s * stage1;
           const unsigned long long xd = sw128_desc(st + (uint32_t)MB1 * kBlk);
@@ -283,37 +284,42 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
             const unsigned long long ad = sw128_desc(st + (uint32_t)b * kBlk);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              if (kk < nk)
+              if (lead && kk < nk)
                 tc_mma(tmem + (uint32_t)(b * a.N1), ad + 2u * kk, xd + 2u * kk, idesc1, (kt > 0 || kk > 0) ? 1u : 0u);
           }
-          tc_commit(empty1(s));
+          if (lead) tc_commit(empty1(s));
+          __syncwarp();
         }
         if (!ok) break;
-        tc_commit(d1full);
+        if (lead) tc_commit(d1full);
+        __syncwarp();
         // step 2: D2[b] = W2 block b . T^T over the K tiles of q, T in shared memory
-        if (!(ok = wait_bounded(tready, (uint32_t)(i & 1), ab))) break;
+        if (!(ok = wait_bounded_warp(tready, (uint32_t)(i & 1), ab))) break;
         tc_fence_after();
         for (int b = 0; ok && b < MB2; ++b) {
           for (int kt = 0; ok && kt < a.KT2; ++kt, ++it2) {
             const int s = it2 % NS2;
-            if (!(ok = wait_bounded(full2(s), (uint32_t)((it2 / NS2) & 1), ab))) break;
+            if (!(ok = wait_bounded_warp(full2(s), (uint32_t)((it2 / NS2) & 1), ab))) break;
             tc_fence_after();
             const unsigned long long ad = sw128_desc(sR2 + (uint32_t)s * kBlk);
             const unsigned long long td = sw128_desc(sT + (uint32_t)kt * (uint32_t)MB1 * kBlk);
             const int nk = min(4, (a.q - kt * 64 + 15) >> 4);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              if (kk < nk)
+              if (lead && kk < nk)
                 tc_mma(tmem + (uint32_t)(b * a.N2), ad + 2u * kk, td + 2u * kk, idesc2, (kt > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(empty2(s));
+            if (lead) tc_commit(empty2(s));
+            __syncwarp();
           }
-          if (ok) tc_commit(d2full0 + 8u * (uint32_t)b);
+          if (ok && lead) tc_commit(d2full0 + 8u * (uint32_t)b);
         }
-        if (ok) tc_commit(tfree);
+        if (ok && lead) tc_commit(tfree);
       }
-      tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
-      const unsigned long long t0 = gtimer();
-      while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+      if (lead) {
+        tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+        }
       }
     }
     __syncwarp();
@@ -586,44 +592,47 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
+    {
+      // ---------------- MMA issuer (see elect_one)
+      const bool lead = elect_one();
       constexpr uint32_t fmt = std::is_same<InT, __half>::value ? 0u : 1u;
       const uint32_t idesc = idesc_f16kind_bmn(128, kTubeCols, fmt);
-      bool ok = wait_bounded(vbar, 0, ab);
+      bool ok = wait_bounded_warp(vbar, 0, ab);
       int it = 0;
       // stage 1 of tile i: D = W1 . F (data MN-major: K step of 16 rows = +2048 bytes; atoms KS rows apart)
       auto stage1 = [&](int i) {
         const int b = i & 1;
-        if (!wait_bounded(d1empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
+        if (!wait_bounded_warp(d1empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
         tc_fence_after();
         const uint32_t dacc = tmem + (PAIR ? (uint32_t)(b * 128) : (uint32_t)(b * 256));
         for (int ks = 0; ks < a.KTs; ++ks, ++it) {
           const int s = it % NS;
-          if (!wait_bounded(full(s), (uint32_t)((it / NS) & 1), ab)) return false;
+          if (!wait_bounded_warp(full(s), (uint32_t)((it / NS) & 1), ab)) return false;
           tc_fence_after();
           const uint32_t sd = sD + (uint32_t)s * kStage;
           const int nk = min(a.KS >> 4, (a.t - ks * a.KS + 15) >> 4);
           for (int mb = 0; mb < MBz; ++mb) {
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-              if (kk < nk) {
+              if (lead && kk < nk) {
                 const int kg = ks * (a.KS >> 4) + kk;  // K step of 16 rows; the eigenbasis K tiles hold 4 of them
                 const unsigned long long wd = sw128_desc(sW1 + (uint32_t)((kg >> 2) * MBz + mb) * kBlk) + 2u * (kg & 3);
                 tc_mma(dacc + (uint32_t)(mb * 128), wd, mn128_desc(sd + 2048u * kk, kStage / 2, 1024), idesc,
                        (ks > 0 || kk > 0) ? 1u : 0u);
               }
           }
-          tc_commit(empty(s));
+          if (lead) tc_commit(empty(s));
+          __syncwarp();
         }
-        tc_commit(d1full(b));
+        if (lead) tc_commit(d1full(b));
+        __syncwarp();
         return true;
       };
       // stage 2 of tile i (PAIR): D2 = W2 . T, T MN-major in shared memory (atoms 16 KB apart)
       auto stage2 = [&](int i) {
         const int b = i & 1;
-        if (!wait_bounded(tready(b), (uint32_t)((i >> 1) & 1), ab)) return false;
-        if (!wait_bounded(d2empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
+        if (!wait_bounded_warp(tready(b), (uint32_t)((i >> 1) & 1), ab)) return false;
+        if (!wait_bounded_warp(d2empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
         tc_fence_after();
         const uint32_t dacc = tmem + 256u + (uint32_t)(b * 128);
         const uint32_t tb = sT + (uint32_t)b * 2u * kAtomT;
@@ -632,11 +641,12 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
           const int nk = min(4, (a.t - kt * 64 + 15) >> 4);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            if (kk < nk)
+            if (lead && kk < nk)
               tc_mma(dacc, wd + 2u * kk, mn128_desc(tb + (uint32_t)kt * 8192u + 2048u * kk, kAtomT, 1024), idesc,
                      (kt > 0 || kk > 0) ? 1u : 0u);
         }
-        tc_commit(d2full(b));
+        if (lead) tc_commit(d2full(b));
+        __syncwarp();
         return true;
       };
       if (PAIR) {
@@ -648,9 +658,11 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
       } else {
         for (int i = 0; ok && i < nmine; ++i) ok = stage1(i);
       }
-      tc_commit(drain);
-      const unsigned long long t0 = gtimer();
-      while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+      if (lead) {
+        tc_commit(drain);
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+        }
       }
     }
     __syncwarp();

@@ -540,6 +540,17 @@ __global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::va
     int tcount = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++tcount) {
       const int b = tcount & 1;
+      uint32_t rw0[8], rw1[8];  // split form, last pass: R~ of the chunk at hand
+      // the 16 hi and the 16 lo words of R~ of this thread's row from column c0 on
+      auto fetch_pair = [&](int c0, uint32_t (&hw)[8], uint32_t (&lw)[8]) {
+        const int r = tile * kTileRows + q * 32 + lane;
+        if (r < a.rows && (ODD || a.vec) && c0 + 16 <= (ODD ? a.rpitch : a.Cout)) {
+          const long long ro = (long long)r * a.rpitch + c0;
+          ld_global_32(a.Rt + ro, hw);
+          ld_global_32(Rlo + ro, lw);
+        }
+      };
+      if constexpr (FINAL && KS::split) fetch_pair(h * 16, rw0, rw1);  // on its way before the accumulator is ready
       if (!wait_bounded(tfull(b), (uint32_t)((tcount >> 1) & 1), ab)) break;
       tc_fence_after();
       const uint32_t tacc = tmem + (uint32_t)(b * a.acc_cols) + ((uint32_t)(q * 32) << 16);
@@ -587,14 +598,6 @@ __global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::va
             const uint4* rp = reinterpret_cast<const uint4*>(a.Rt + (long long)r * a.rpitch + col(j));
             rb[0] = __ldg(rp);
             rb[1] = __ldg(rp + 1);
-          }
-        };
-        // split form: the 16 hi and the 16 lo words of R~ chunk j of this row
-        auto fetch_pair = [&](int j, uint32_t (&hw)[8], uint32_t (&lw)[8]) {
-          if ((ODD ? valid : vec) && j < J && col(j) + 16 <= (ODD ? a.rpitch : a.Cout)) {
-            const long long ro = (long long)r * a.rpitch + col(j);
-            ld_global_32(a.Rt + ro, hw);
-            ld_global_32(Rlo + ro, lw);
           }
         };
         auto process = [&](int c0, const uint32_t (&t)[16], const uint4 (&rcur)[2], const uint32_t (&hw)[8],
@@ -737,17 +740,15 @@ __global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::va
         };
         uint32_t tA[16], tB[16];
         uint4 rA[2], rB[2];
-        uint32_t rw0[8], rw1[8];
         if constexpr (FINAL && KS::split) {
           // R~ of the next chunk is on its way while this one is processed; the accumulator's chunk is loaded when
           // needed (tens of clocks against the some eight hundred of R~, which, waited for chunk by chunk, made this
           // pass twice as long as the others: 42 against 22 us at 256 x 256 x 128)
-          fetch_pair(0, rw0, rw1);
 #pragma unroll 1
           for (int j = 0; j < J; ++j) {
             uint32_t rw2[8], rw3[8];
             tc_ld16_issue(tacc + (uint32_t)col(j), tA);
-            fetch_pair(j + 1, rw2, rw3);
+            fetch_pair(col(j + 1), rw2, rw3);
             tc_ld16_wait(tA);
             process(col(j), tA, rA, rw0, rw1);
 #pragma unroll
@@ -1004,39 +1005,42 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer
+    {
+      // ---------------- MMA issuer (see elect_one)
+      const bool lead = elect_one();
       constexpr uint32_t fmt = std::is_same<InT, __half>::value ? 0u : 1u;
       const uint32_t idesc1 = idesc_f16kind(128, a.Np, fmt), idesc2 = idesc_f16kind(128, 128, fmt);
       const unsigned long long dX0 = sw128_desc(sD), dW1 = sw128_desc(sW1), dW2 = sw128_desc(sW2), dT = sw128_desc(sT);
       const uint32_t w1kt = (uint32_t)(a.VR * 128) >> 4, w2kt = (uint32_t)(128 * 128) >> 4,
                      tkt = (uint32_t)kTBytes >> 4;
-      bool ok = wait_bounded(vbar, 0, ab);
+      bool ok = wait_bounded_warp(vbar, 0, ab);
       int it = 0;
       auto stage1 = [&](int i) {  // forward product of tile i into D1[i & 1]
         const int b = i & 1;
-        if (!wait_bounded(d1empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
+        if (!wait_bounded_warp(d1empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
         tc_fence_after();
         const uint32_t dacc = tmem + (uint32_t)(b * 128);
         for (int kt = 0; kt < KT; ++kt, ++it) {
           const int s = it % NS;
-          if (!wait_bounded(full(s), (uint32_t)((it / NS) & 1), ab)) return false;
+          if (!wait_bounded_warp(full(s), (uint32_t)((it / NS) & 1), ab)) return false;
           tc_fence_after();
           const unsigned long long xd = dX0 + (uint32_t)s * (uint32_t)(kStageBytes >> 4);
           const unsigned long long wd = dW1 + (uint32_t)kt * w1kt;
           const int nk = min(4, (a.C - kt * kKTile + 15) >> 4);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            if (kk < nk) tc_mma(dacc, xd + 2u * kk, wd + 2u * kk, idesc1, (kt > 0 || kk > 0) ? 1u : 0u);
-          tc_commit(empty(s));
+            if (lead && kk < nk) tc_mma(dacc, xd + 2u * kk, wd + 2u * kk, idesc1, (kt > 0 || kk > 0) ? 1u : 0u);
+          if (lead) tc_commit(empty(s));
+          __syncwarp();
         }
-        tc_commit(d1full(b));
+        if (lead) tc_commit(d1full(b));
+        __syncwarp();
         return true;
       };
       auto stage2 = [&](int i) {  // backward product of tile i (T in shared memory) into D2[i & 1]
         const int b = i & 1;
-        if (!wait_bounded(tready(b), (uint32_t)((i >> 1) & 1), ab)) return false;
-        if (!wait_bounded(d2empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
+        if (!wait_bounded_warp(tready(b), (uint32_t)((i >> 1) & 1), ab)) return false;
+        if (!wait_bounded_warp(d2empty(b), (uint32_t)(((i >> 1) & 1) ^ 1), ab)) return false;
         tc_fence_after();
         const uint32_t dacc = tmem + 256u + (uint32_t)(b * 128);
         for (int kt = 0; kt < KT; ++kt) {
@@ -1044,9 +1048,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
           const int nk = min(4, (a.C - kt * kKTile + 15) >> 4);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            if (kk < nk) tc_mma(dacc, wd + 2u * kk, td + 2u * kk, idesc2, (kt > 0 || kk > 0) ? 1u : 0u);
+            if (lead && kk < nk) tc_mma(dacc, wd + 2u * kk, td + 2u * kk, idesc2, (kt > 0 || kk > 0) ? 1u : 0u);
         }
-        tc_commit(d2full(b));
+        if (lead) tc_commit(d2full(b));
+        __syncwarp();
         return true;
       };
       if (ok && nmine > 0) ok = stage1(0);
@@ -1054,9 +1059,11 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         if (i + 1 < nmine && !(ok = stage1(i + 1))) break;
         ok = stage2(i);
       }
-      tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
-      const unsigned long long t0 = gtimer();
-      while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+      if (lead) {
+        tc_commit(drain);  // every MMA this thread issued is complete once `drain` fires
+        const unsigned long long t0 = gtimer();
+        while (!mbar_try_wait(drain, 0) && gtimer() - t0 < kWaitLimitNs) {
+        }
       }
     }
     __syncwarp();

@@ -52,6 +52,7 @@ struct SolveState {
   unsigned pmax_bits;  // max |P_int| accumulator of the direction kernel (atomicMax)
   double pmax;         // max |P_s| of the current direction
   unsigned long long umax_bits;  // max |U| accumulator (FP64 bits of |U|; atomicMax)
+  unsigned long long emax_bits;  // max |eta| accumulator of the solve's first kernel (as umax_bits)
   double umax;         // max |U| of the current iterate
   int ku;              // fixed-point exponent of U for the residual check (from umax)
   int sr;              // 2^-sr bounds every |eta_hat - L U| entry (scale of the check's FP32 sums)

@@ -53,7 +53,7 @@ struct SolveState;  // device-side scalars (tpcg_dev.cuh)
 
 // Kernel kinds for the launch counter and the optional event profiler.
 // Persistent fixed-point sweeps (grid size per kernel, from its occupancy).
-enum FxKernel { kFxDir = 0, kFxUpd, kFxTrue, kFxInit, kFxApply, kFxCount };
+enum FxKernel { kFxDir = 0, kFxUpd, kFxTrue, kFxInit, kFxApply, kFxField, kFxCount };
 
 enum KernelKind {
   kKEtaSum = 0, kKInit, kKDirection, kKUpdate, kKTrueRes, kKCenter, kKApply, kKModeF64, kKModeTC, kKConvert, kKFormU,
@@ -180,7 +180,7 @@ struct tpcg_plan {
   dim3 st_block;            // stencil kernels
   bool sweep_grain_set = false;  // the caller chose the grain
   int sweep_grain = 4;  // TPCG_OPT_SWEEP_GRAIN: least (tile, plane) pairs (x 256 points) per sweep block
-  int fx_blocks[tpcg::kFxCount] = {1, 1, 1, 1, 1};  // FxKernel -> blocks of the persistent fixed-point sweeps
+  int fx_blocks[tpcg::kFxCount] = {1, 1, 1, 1, 1, 1};  // FxKernel -> blocks of the persistent fixed-point sweeps
   // comparator preconditioner of the FP64 form (TPCG_PRECOND_*), Jacobi(p, omega) and its table of
   // 1 / (omega d) indexed by the boundary class (start, interior, end) of x + 3 y + 9 z
   int pc_kind = 0;
