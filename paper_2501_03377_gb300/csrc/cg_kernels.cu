@@ -477,7 +477,7 @@ __device__ void fin_true(SolveState* st, const double (&s)[3], long long N) {
 // Otherwise the stop-test check; `force` evaluates the residual of the
 // returned iterate for the report only.
 template <bool INIT>
-__global__ void __launch_bounds__(TX* TY) k_residual_fx(Geom g, const double* __restrict__ eta,
+__global__ void __launch_bounds__(TX* TY, 4) k_residual_fx(Geom g, const double* __restrict__ eta,
                                                         const double* __restrict__ U, double* __restrict__ R,
                                                         LowPrec lp, SolveState* st, double* partials, int force) {
   if (!INIT && !force && (st->done || !st->need_check)) return;
@@ -1038,11 +1038,11 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_int(Geom g, DirRing ring, 
         const int dx = 2 * c - xl - xr, dy = 2 * c - cur.yl - cur.yr, dz = 2 * c - zlv - zrv;
         double r = cur.r;
         if (g.uniform) {
-          r = fma(na0, i32_to_f64_scaled(dx + dy + dz, -kp), r);
+          r = fma(na0, i24_to_f64_scaled(dx + dy + dz, -kp), r);
         } else {
-          r = fma(na0, i32_to_f64_scaled(dx, -kp), r);
-          r = fma(na1, i32_to_f64_scaled(dy, -kp), r);
-          if (dz) r = fma(na2, i32_to_f64_scaled(dz, -kp), r);
+          r = fma(na0, i24_to_f64_scaled(dx, -kp), r);
+          r = fma(na1, i24_to_f64_scaled(dy, -kp), r);
+          if (dz) r = fma(na2, i24_to_f64_scaled(dz, -kp), r);
         }
         const unsigned i = (unsigned)k * plane + col;
         R[i] = r;
@@ -1137,15 +1137,15 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_pair(Geom g, DirRing ring,
         const int dz0 = 2 * c.x - zlv.x - zrv.x, dz1 = 2 * c.y - zlv.y - zrv.y;
         double r0 = cur.r.x, r1 = cur.r.y;
         if constexpr (kUni) {
-          r0 = fma(na0, i32_to_f64_scaled(dx0 + dy0 + dz0, -kp), r0);
-          r1 = fma(na0, i32_to_f64_scaled(dx1 + dy1 + dz1, -kp), r1);
+          r0 = fma(na0, i24_to_f64_scaled(dx0 + dy0 + dz0, -kp), r0);
+          r1 = fma(na0, i24_to_f64_scaled(dx1 + dy1 + dz1, -kp), r1);
         } else {
-          r0 = fma(na0, i32_to_f64_scaled(dx0, -kp), r0);
-          r0 = fma(na1, i32_to_f64_scaled(dy0, -kp), r0);
-          if (dz0) r0 = fma(na2, i32_to_f64_scaled(dz0, -kp), r0);
-          r1 = fma(na0, i32_to_f64_scaled(dx1, -kp), r1);
-          r1 = fma(na1, i32_to_f64_scaled(dy1, -kp), r1);
-          if (dz1) r1 = fma(na2, i32_to_f64_scaled(dz1, -kp), r1);
+          r0 = fma(na0, i24_to_f64_scaled(dx0, -kp), r0);
+          r0 = fma(na1, i24_to_f64_scaled(dy0, -kp), r0);
+          if (dz0) r0 = fma(na2, i24_to_f64_scaled(dz0, -kp), r0);
+          r1 = fma(na0, i24_to_f64_scaled(dx1, -kp), r1);
+          r1 = fma(na1, i24_to_f64_scaled(dy1, -kp), r1);
+          if (dz1) r1 = fma(na2, i24_to_f64_scaled(dz1, -kp), r1);
         }
         const unsigned i = (unsigned)k * plane + col;
         *reinterpret_cast<double2*>(R + i) = make_double2(r0, r1);
@@ -1245,11 +1245,11 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_int(Geom g, double* __re
         const int dx = 2 * c - xl - xr, dy = 2 * c - cur.yl - cur.yr, dz = 2 * c - zlv - zrv;
         double r = cur.r;
         if (g.uniform) {
-          r = fma(na0, i32_to_f64_scaled(dx + dy + dz, -kp), r);
+          r = fma(na0, i24_to_f64_scaled(dx + dy + dz, -kp), r);
         } else {
-          r = fma(na0, i32_to_f64_scaled(dx, -kp), r);
-          r = fma(na1, i32_to_f64_scaled(dy, -kp), r);
-          if (dz) r = fma(na2, i32_to_f64_scaled(dz, -kp), r);
+          r = fma(na0, i24_to_f64_scaled(dx, -kp), r);
+          r = fma(na1, i24_to_f64_scaled(dy, -kp), r);
+          if (dz) r = fma(na2, i24_to_f64_scaled(dz, -kp), r);
         }
         const unsigned i = (unsigned)k * plane + col;
         R[i] = r;
@@ -1257,7 +1257,7 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_int(Geom g, double* __re
         store_lp(lp, i, r, r32);
         rr = fmaf(r32, r32, rr);
         sR += r32;
-        const double pv = i32_to_f64_scaled(c, -kp);
+        const double pv = i24_to_f64_scaled(c, -kp);
         const double u = ZG ? alpha * pv : fma(alpha, pv, cur.u);
         U[i] = u;
         const unsigned long long ub = mag_key(u);
@@ -1356,15 +1356,15 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_pair(Geom g, double* __r
         const int dz0 = 2 * c.x - zlv.x - zrv.x, dz1 = 2 * c.y - zlv.y - zrv.y;
         double r0 = cur.r.x, r1 = cur.r.y;
         if constexpr (kUni) {
-          r0 = fma(na0, i32_to_f64_scaled(dx0 + dy0 + dz0, -kp), r0);
-          r1 = fma(na0, i32_to_f64_scaled(dx1 + dy1 + dz1, -kp), r1);
+          r0 = fma(na0, i24_to_f64_scaled(dx0 + dy0 + dz0, -kp), r0);
+          r1 = fma(na0, i24_to_f64_scaled(dx1 + dy1 + dz1, -kp), r1);
         } else {
-          r0 = fma(na0, i32_to_f64_scaled(dx0, -kp), r0);
-          r0 = fma(na1, i32_to_f64_scaled(dy0, -kp), r0);
-          if (dz0) r0 = fma(na2, i32_to_f64_scaled(dz0, -kp), r0);
-          r1 = fma(na0, i32_to_f64_scaled(dx1, -kp), r1);
-          r1 = fma(na1, i32_to_f64_scaled(dy1, -kp), r1);
-          if (dz1) r1 = fma(na2, i32_to_f64_scaled(dz1, -kp), r1);
+          r0 = fma(na0, i24_to_f64_scaled(dx0, -kp), r0);
+          r0 = fma(na1, i24_to_f64_scaled(dy0, -kp), r0);
+          if (dz0) r0 = fma(na2, i24_to_f64_scaled(dz0, -kp), r0);
+          r1 = fma(na0, i24_to_f64_scaled(dx1, -kp), r1);
+          r1 = fma(na1, i24_to_f64_scaled(dy1, -kp), r1);
+          if (dz1) r1 = fma(na2, i24_to_f64_scaled(dz1, -kp), r1);
         }
         const unsigned i = (unsigned)k * plane + col;
         *reinterpret_cast<double2*>(R + i) = make_double2(r0, r1);
@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(TX* TY, 4) k_update_u_pair(Geom g, double* __r
         store_lp_pair(lp, i, r0, r1, a32, b32);
         rr = fmaf(a32, a32, fmaf(b32, b32, rr));
         sR += a32 + b32;
-        const double p0 = i32_to_f64_scaled(c.x, -kp), p1 = i32_to_f64_scaled(c.y, -kp);
+        const double p0 = i24_to_f64_scaled(c.x, -kp), p1 = i24_to_f64_scaled(c.y, -kp);
         const double u0 = ZG ? alpha * p0 : fma(alpha, p0, cur.u.x);
         const double u1 = ZG ? alpha * p1 : fma(alpha, p1, cur.u.y);
         *reinterpret_cast<double2*>(U + i) = make_double2(u0, u1);

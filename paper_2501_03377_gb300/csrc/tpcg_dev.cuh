@@ -401,6 +401,13 @@ __device__ __forceinline__ double i32_to_f64_scaled(int v, int e) {
   return __longlong_as_double((long long)bits);
 }
 
+// The same for |v| <= 2^24 through FP32 (exact) and a shift of its fields, some seven instructions instead of fourteen.
+__device__ __forceinline__ double i24_to_f64_scaled(int v, int e) {
+  const uint32_t b = __float_as_uint(__int2float_rn(v));
+  const uint32_t hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((uint32_t)(896 + e) << 20));
+  return v ? __hiloint2double((int)hi, (int)(b << 29)) : 0.0;
+}
+
 // Exponent k with bound * 2^k < 2^20 for the fixed-point direction
 // (bound >= max|P|); 0 when the bound is zero.  With |P_int| <= 2^20 every
 // difference of two values is below 2^22 and converts to FP32 exactly by the
