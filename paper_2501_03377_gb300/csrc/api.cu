@@ -372,6 +372,7 @@ int enqueue_iterations(SolveJob& j, int count) {
   const int rc = run_graphed(p, GraphKey{1, j.issued > 0 ? 1 : 0, count, graph_flags(j), p->graph_gen},
                              [&]() { return launch_iterations(j, count); });
   if (rc) return rc;
+  j.base = j.issued;
   j.issued += count;
   return TPCG_OK;
 }
@@ -431,7 +432,9 @@ int job_step(SolveJob& j) {
   if (cudaEventSynchronize(p->ev_state) != cudaSuccess) return last_cuda_error() ? TPCG_ERR_CUDA : TPCG_ERR_CUDA;
   if (j.phase == 1) {
     j.issued = hs->iter;  // iterations that paused behind a check count for nothing
-    if (!hs->done && j.issued <= j.maxit + 1) {
+    // A chunk completes at least one iteration or ends the solve; a wait that gave up ends it too (the limit of
+    // every wait of the iterations left would pass before the same error).
+    if (!hs->done && !hs->timeout && j.issued > j.base && j.issued <= j.maxit + 1) {
       int rc = enqueue_iterations(j, j.chunk);
       if (rc) return rc;
       return enqueue_state_readback(p);

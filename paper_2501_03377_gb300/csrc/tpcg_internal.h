@@ -85,6 +85,7 @@ struct SolveJob {
   int maxit = 100;
   unsigned flags = 0;
   int issued = 0, chunk = 0;
+  int base = 0;   // iterations completed when the last chunk was issued
   int phase = 0;  // 0 not started, 1 iterating, 2 finishing, 3 finished
   int done_host = 0, status_host = 0;
   int status = 0;
