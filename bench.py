@@ -539,9 +539,9 @@ NCU_TRAFFIC_PER_LAUNCH = {
     },
     "bf16x3": {
         # the five launches of one application (one per mode product, the z pair around G fused): 33.7-33.9 MB
-        # read each (the hi and lo planes of the input), under 0.9 MB written (the outputs stay in L2 until the
-        # next launch reads them)
-        "modeprod_tc": 172.24e6 / 5,
+        # read each (the hi and lo planes of the input; the last also those of R~), under 0.3 MB written (the
+        # outputs stay in L2 until the next launch reads them)
+        "modeprod_tc": 203.0e6 / 5,
     },
 }
 
@@ -551,13 +551,16 @@ def kernel_work(kind, plan_prec, N, dims, iters_total, applies_total, solves, ch
     the work).
 
     Bytes are the data each kernel must move once per grid point (halo re-reads and
-    reduction scratch excluded); flops are the FP64 operations of the FP64 form."""
+    reduction scratch excluded); flops are those of the FP64 form's mode products."""
     n, q, t = dims
     mixed = plan_prec != "fp64"
     # bytes per point of a tensor-core operand (and of the copy of R): FP16/BF16 2, TF32 4, split BF16 pair 4
     lpb = {"fp16": 2, "bf16": 2, "tf32": 4, "bf16x3": 4}.get(plan_prec, 0)
     if kind == "modeprod_f64":
-        return applies_total * 4.0 * N * (n + q + t + 0.25) / 1e12, "TFLOP", "alu", applies_total * (6 if t > 1 else 4)
+        npass = 6 if t > 1 else 4
+        if max(n, q, t) <= 256:  # 28 exact FP16 digit products per FP64 product, on the tensor cores
+            return applies_total * 28 * 4.0 * N * (n + q + t) / 1e12, "TFLOP", "tensor", applies_total * npass
+        return applies_total * 4.0 * N * (n + q + t + 0.25) / 1e12, "TFLOP", "alu", applies_total * npass
     if kind == "modeprod_tc":
         # the per-point figure of the scope table for one application of the mixed preconditioner: about
         # 30 B (2560 flop / ~30 B at 256x256x128), whatever the launch sequence fuses
@@ -576,8 +579,8 @@ def kernel_work(kind, plan_prec, N, dims, iters_total, applies_total, solves, ch
     if kind == "direction":
         if mixed:  # Z (FP32) + P_old (int32) in, P (int32) out
             return iters_total * 12.0 * N / 1e9, "GB", "hbm", iters_total
-        # FP64 form: FP64 flops per point: P = (Z - m) + beta P_old (3), 7-point stencil (7), <W, P> (2)
-        return iters_total * 12.0 * N / 1e12, "TFLOP", "alu", iters_total
+        # FP64 form: Z and P_old (8+8) in, P and W (8+8) out (the stencil's sums are integer)
+        return iters_total * 32.0 * N / 1e9, "GB", "hbm", iters_total
     if kind == "update":
         # the instrumented plan updates U in place: mixed P (4) + R (8+8) + U (8+8) + tensor-core copy of R
         # (lpb); FP64 form: P and W (8+8) + R + U
@@ -890,7 +893,7 @@ def run_ours(args, rank, world, torch):
             if fprec != prec:
                 forms[f"{fprec}_form"] = form_record(fprec)
 
-    # the plain FP64 form for comparison (fewer steps: it is ~100x slower)
+    # the FP64 form for comparison (fewer steps)
     fp64_cmp = None
     if prec != "fp64" and not args.no_fp64_compare:
         p64 = Plan(nx, ny, nz, w0["bcs"], prec="fp64")
