@@ -547,6 +547,9 @@ int tpcg_plan_create(int nx, int ny, int nz, const int bc[3], const double h[3],
   if (cudaGetDevice(&p->device) != cudaSuccess) { delete p; return TPCG_ERR_CUDA; }
   cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device);
   if (p->num_sms <= 0) p->num_sms = 1;
+  int sm_shared = 0;
+  cudaDeviceGetAttribute(&sm_shared, cudaDevAttrMaxSharedMemoryPerMultiprocessor, p->device);
+  if ((size_t)sm_shared > kSmSharedBytes) { delete p; return TPCG_ERR_UNSUPPORTED; }  // sole_smem
 
   // Algorithm 5: eigenpairs per axis (closed forms, checked)
   const int lens[3] = {nx, ny, nz};

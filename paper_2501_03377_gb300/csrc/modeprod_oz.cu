@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(256) k_oz_ghat(double* __restrict__ G, int A, 
 
 constexpr size_t kOzSmem = 1024 + (size_t)kOzStages * kOzImg + (size_t)kOzSlots * kOzSlot +
                            8 * (2 * kOzStages + 2 * kOzSlots + kOzExpBufs + 5) + 4 * kOzExpBufs * kOzRows + 16;
-static_assert(kOzSmem <= (size_t)kMaxSmem, "shared memory of k_modeprod_oz");
+static_assert(kOzSmem <= (size_t)kMaxSmem && kOzSmem == sole_smem(kOzSmem), "shared memory of k_modeprod_oz");
 
 }  // namespace
 

@@ -920,7 +920,7 @@ int slab_plan_setup(tpcg_plan* p) {
             a.NS2 = ns2;
             a.reg1 = reg1;
             a.stg = stg;
-            L.smem = total;
+            L.smem = sole_smem(total);
             found = true;
           }
         }
@@ -966,7 +966,7 @@ int slab_plan_setup(tpcg_plan* p) {
     const size_t kStage = (size_t)a.KS * 256;
     if (fixed + 2 * kStage > (size_t)kMaxSmem) return TPCG_ERR_UNSUPPORTED;
     a.NS = (int)std::min<size_t>(6, (kMaxSmem - fixed) / kStage);
-    L.smem = fixed + (size_t)a.NS * kStage;
+    L.smem = sole_smem(fixed + (size_t)a.NS * kStage);
     const cuuint64_t dF[2] = {(cuuint64_t)C, (cuuint64_t)t}, sF[1] = {(cuuint64_t)C * 2};
     const cuuint32_t bF[2] = {64, (cuuint32_t)a.KS};
     const int lp2 = p->pitch16[2];

@@ -1886,7 +1886,7 @@ int tc_plan_setup(tpcg_plan* p) {
     a.stg = (!a.tstore && !a.vec && (st.form == 2 || (sp.oa == (long long)sp.B * sp.ob || sp.A == 1))) ? 1 : 0;
     fixed += (size_t)a.aux;
     a.NS = (int)std::min<size_t>(8, (kMaxSmem - fixed) / sbytes);
-    st.smem = fixed + (size_t)a.NS * sbytes;
+    st.smem = sole_smem(fixed + (size_t)a.NS * sbytes);
     const int ntiles = (a.rows + kTileRows - 1) / kTileRows;
     st.ntiles = ntiles;
     st.grid = tc_grid(p, ntiles);
@@ -1941,7 +1941,7 @@ int tc_plan_setup(tpcg_plan* p) {
       const size_t fixed = 1024 + (size_t)a.KT * 2 * a.VR * 128 + 2 * (size_t)a.KT * 2 * kTBytes + 512;
       if (fixed + 2 * (size_t)kStageBytes > (size_t)kMaxSmem) return TPCG_ERR_UNSUPPORTED;
       a.NS = (int)std::min<size_t>(8, (kMaxSmem - fixed) / (2 * (size_t)kStageBytes));
-      st.smem = fixed + (size_t)a.NS * 2 * kStageBytes;
+      st.smem = sole_smem(fixed + (size_t)a.NS * 2 * kStageBytes);
       return TPCG_OK;
     }
     if (f.form != 1 || b.form != 2 || !b.args.tstore || b.args.MB != 1 || b.args.B % 16 != 0)
@@ -1966,7 +1966,7 @@ int tc_plan_setup(tpcg_plan* p) {
                          (size_t)kPairEpi * 2 * 32 * 16 * 2 + 512;
     if (fixed + 2 * (size_t)kStageBytes > (size_t)kMaxSmem) return TPCG_ERR_UNSUPPORTED;
     a.NS = (int)std::min<size_t>(8, (kMaxSmem - fixed) / kStageBytes);
-    st.smem = fixed + (size_t)a.NS * kStageBytes;
+    st.smem = sole_smem(fixed + (size_t)a.NS * kStageBytes);
     return TPCG_OK;
   };
   const int bad = tp->tf32    ? set_tf32_smem_attrs()

@@ -49,6 +49,13 @@ struct StageParams {
   int out_C;             // contiguous extent of that view
 };
 
+// Dynamic shared memory of a launch that allocates TMEM: at least half of an SM's 228 KB, so that no two such CTAs
+// share an SM (each takes another 1 KB of the system's).  tcgen05.alloc waits without a limit, and a CTA launched
+// early (programmatic dependent launch) keeps its columns until the grid before it has completed: beside a CTA of that
+// grid, or of another stream's, which waits for the same columns, neither would end.
+constexpr size_t kSmSharedBytes = 228 * 1024;
+constexpr size_t sole_smem(size_t need) { return need > kSmSharedBytes / 2 ? need : kSmSharedBytes / 2; }
+
 struct SolveState;  // device-side scalars (tpcg_dev.cuh)
 
 // Kernel kinds for the launch counter and the optional event profiler.
