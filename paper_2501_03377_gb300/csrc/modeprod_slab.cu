@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
                       full1(s));
       }
     }
-    if (!ok && lane == 0) {  // every issued load completes before the CTA may exit
+    if (lane == 0) {  // every issued load completes (bounded) before the CTA may exit, whoever gave up
       for (int j = (it1 > NS1 ? it1 - NS1 : 0); j < it1; ++j) {
         const unsigned long long t0 = gtimer();
         while (!mbar_try_wait(full1(j % NS1), (uint32_t)((j / NS1) & 1)) && gtimer() - t0 < kWaitLimitNs) {
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
             mbar_expect_tx(full2(s), kBlk);
             tma_load_2d(sR2 + (uint32_t)s * kBlk, &tmA2, kt * 64, b * 128, full2(s));
           }
-      if (!ok) {
+      {
         for (int j = (it2 > NS2 ? it2 - NS2 : 0); j < it2; ++j) {
           const unsigned long long t0 = gtimer();
           while (!mbar_try_wait(full2(j % NS2), (uint32_t)((j / NS2) & 1)) && gtimer() - t0 < kWaitLimitNs) {
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
                       ks * a.KS, full(s));
       }
     }
-    if (!ok && lane == 0) {  // every issued load completes before the CTA may exit
+    if (lane == 0) {  // every issued load completes (bounded) before the CTA may exit, whoever gave up
       for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
         const unsigned long long t0 = gtimer();
         while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {

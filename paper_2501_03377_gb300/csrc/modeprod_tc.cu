@@ -388,8 +388,9 @@ __global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::va
           }
         }
       }
-      // drain: every issued load has completed before the CTA may exit
-      if (*abort_flag) {
+      // drain: every issued load has completed (bounded) before the CTA may exit, also where another warp gives up
+      // after the last one was issued
+      {
         for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
           const unsigned long long t0 = gtimer();
           while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {
@@ -501,7 +502,7 @@ __global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::va
           issued[hh] = k + 1;
         }
       }
-      if (!ok) {  // every issued load completes before the CTA may exit
+      {  // every issued load completes before the CTA may exit
         for (int hh = 0; hh < 2; ++hh)
           for (int k = (issued[hh] > a.rhalf ? issued[hh] - a.rhalf : 0); k < issued[hh]; ++k) {
             const unsigned long long t0 = gtimer();
@@ -992,7 +993,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
           tma_load_2d(sD + (uint32_t)s * kStageBytes, &tmX, kt * kKTile, tile * kTileRows, full(s));
         }
       }
-      if (*abort_flag) {  // every issued load completes before the CTA may exit
+      {  // every issued load completes before the CTA may exit (see k_modeprod_tc)
         for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
           const unsigned long long t0 = gtimer();
           while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {
@@ -1295,7 +1296,7 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
           tma_load_3d(sD + (uint32_t)s * sbytes, &tmX, kt * kKTile, tile * kTileRows, 0, full(s));
         }
       }
-      if (*abort_flag) {  // every issued load completes before the CTA may exit
+      {  // every issued load completes before the CTA may exit (see k_modeprod_tc)
         for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
           const unsigned long long t0 = gtimer();
           while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {
