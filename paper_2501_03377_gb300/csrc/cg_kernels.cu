@@ -281,8 +281,10 @@ __device__ __forceinline__ double stencil_f64(double c, double xl, double xr, do
   auto ex = [](double v) { return __double2hiint(v) & 0x7ff00000; };
   const int E20 = max(max(ex(c), max(ex(xl), ex(xr))), max(max(ex(yl), ex(yr)), max(ex(zl), ex(zr))));
   if (E20 < (70 << 20) || E20 > (2040 << 20)) {  // next to the ends of the range, or not finite
-    const double dx = fma(2.0, c, -(xl + xr)), dy = fma(2.0, c, -(yl + yr)), dz = fma(2.0, c, -(zl + zr));
-    return fma(dz, w.ih2, fma(dx, w.ih0, dy * w.ih1));
+    const double dx = fma(2.0, c, -(xl + xr)), dy = fma(2.0, c, -(yl + yr));
+    const double r = fma(dx, w.ih0, dy * w.ih1);
+    if (w.ih2 == 0.0) return r;  // no z axis (its zl = zr = c would make a NaN of an infinity)
+    return fma(fma(2.0, c, -(zl + zr)), w.ih2, r);
   }
   const int e = (E20 >> 20) - 1081;
   auto to_f64 = [&](long long v) { return HW ? i64_to_f64_scaled_hw(v, e) : i64_to_f64_scaled(v, e); };
