@@ -12,6 +12,7 @@
 // ("ghost") values: periodic wraps, Dirichlet reads 0, Neumann mirrors the
 // boundary value -- which reproduces the corner entries (alpha, beta, gamma) of
 // eq. (lap1d) exactly.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 
@@ -255,8 +256,12 @@ struct NoPre {};
 // The stencil of an FP64 field (tpcg_apply_laplacian, the FP64 form's W = L P, the Jacobi comparator).  An FP64 addition
 // occupies its pipe as long as 64 instructions occupy the others here, so the seven values of a point are aligned to
 // the largest of their exponents as 59-bit integers (some ten instructions each), summed exactly and rounded to FP64
-// once: the bits shifted out are below 2^-58 of the largest value, less than the rounding of a single FP64 addition.
-// 256 x 256 x 128: six FP64 operations a point took 157 us (0.6 of the pipe).
+// once: the bits shifted out are below 2^-58 of the largest value M, 12 of them together 2^-54.4 M / h^2.  With unequal
+// spacings an axis' four cost at most 2^-56 M / h^2 by its own h: below the roundings of the axis that M lies on (2^-53 of
+// M by that axis' 1/h^2, twice) only while the weights are alike.  Where they differ by more than a factor of four each
+// axis is aligned to its own three values (nine alignments instead of seven).
+// 256 x 256 x 128: six FP64 operations a point took 157 us (0.6 of the pipe); one alignment for all 77 us
+// (111 with unequal spacings), one per axis 111.
 
 // x as a multiple of 2^(E - 1081), E the exponent field E20 >> 20 >= that of x, truncated.
 __device__ __forceinline__ long long aligned59(double x, int E20) {
@@ -274,8 +279,9 @@ struct Weights {  // 1/h^2 per axis
 };
 
 // (L field)(point) from the point's value and its neighbours.  HW: convert with the FP64 pipe's instruction (kernels
-// that leave it idle), else by integer arithmetic.
-template <bool HW>
+// that leave it idle), else by integer arithmetic.  APART: weights that differ by more than a factor of four (a kernel of
+// its own: both forms in one cost the direction a block per SM).
+template <bool HW, bool APART>
 __device__ __forceinline__ double stencil_f64(double c, double xl, double xr, double yl, double yr, double zl, double zr,
                                               const Weights& w) {
   auto ex = [](double v) { return __double2hiint(v) & 0x7ff00000; };
@@ -286,19 +292,30 @@ __device__ __forceinline__ double stencil_f64(double c, double xl, double xr, do
     if (w.ih2 == 0.0) return r;  // no z axis (its zl = zr = c would make a NaN of an infinity)
     return fma(fma(2.0, c, -(zl + zr)), w.ih2, r);
   }
+  auto to_f64 = [](long long v, int e) { return HW ? i64_to_f64_scaled_hw(v, e) : i64_to_f64_scaled(v, e); };
+  if constexpr (APART) {
+    auto axis = [&](double l, double r) {
+      const int E = max(max(ex(c), max(ex(l), ex(r))), 70 << 20);
+      return to_f64(2 * aligned59(c, E) - aligned59(l, E) - aligned59(r, E), (E >> 20) - 1081);
+    };
+    return fma(axis(zl, zr), w.ih2, fma(axis(xl, xr), w.ih0, axis(yl, yr) * w.ih1));
+  }
   const int e = (E20 >> 20) - 1081;
-  auto to_f64 = [&](long long v) { return HW ? i64_to_f64_scaled_hw(v, e) : i64_to_f64_scaled(v, e); };
   const long long c2 = 2 * aligned59(c, E20);
   const long long dx = c2 - aligned59(xl, E20) - aligned59(xr, E20), dy = c2 - aligned59(yl, E20) - aligned59(yr, E20),
                   dz = c2 - aligned59(zl, E20) - aligned59(zr, E20);
   if (w.uniform) {
-    const double r = to_f64(dx + dy + dz);
+    const double r = to_f64(dx + dy + dz, e);
     return w.ih0 != 1.0 ? r * w.ih0 : r;
   }
-  return fma(to_f64(dz), w.ih2, fma(to_f64(dx), w.ih0, to_f64(dy) * w.ih1));
+  return fma(to_f64(dz, e), w.ih2, fma(to_f64(dx, e), w.ih0, to_f64(dy, e) * w.ih1));
 }
 
 __device__ __forceinline__ Weights weights_of(const Geom& g) { return Weights{g.ih2[0], g.ih2[1], g.ih2[2], g.uniform}; }
+static bool weights_apart(const tpcg_plan* p) {
+  const double z = p->nz > 1 ? p->h[2] : p->h[0];
+  return std::max({p->h[0], p->h[1], z}) > 2.0 * std::min({p->h[0], p->h[1], z});
+}
 
 struct FieldPlain {  // the stencil is applied to x itself
   using Raw = double;
@@ -323,6 +340,7 @@ struct FieldDirection {  // FP64 form: P = (Z - mean Z) + beta * P_old   (Algori
 };
 
 // ------------------------------------------------------------------ W = L x
+template <bool APART>
 struct OpApply {
   using Pre = NoPre;
   double* __restrict__ w;
@@ -330,14 +348,15 @@ struct OpApply {
   __device__ __forceinline__ NoPre load(unsigned) const { return NoPre{}; }
   __device__ __forceinline__ void operator()(unsigned i, int, int, int, NoPre, double c, double xl, double xr, double yl,
                                              double yr, double zl, double zr) {
-    w[i] = stencil_f64<true>(c, xl, xr, yl, yr, zl, zr, wt);
+    w[i] = stencil_f64<true, APART>(c, xl, xr, yl, yr, zl, zr, wt);
   }
 };
 
+template <bool APART>
 __global__ void __launch_bounds__(TX* TY) k_apply_laplacian(Geom g, const double* __restrict__ x,
                                                             double* __restrict__ w) {
   FieldPlain f{x};
-  OpApply op{w, weights_of(g)};
+  OpApply<APART> op{w, weights_of(g)};
   stencil_sweep_fx<double, 0>(g, f, op, nullptr, nullptr, 0, NoFin{});
 }
 
@@ -522,6 +541,7 @@ __global__ void __launch_bounds__(TX* TY, 4) k_residual_fx(Geom g, const double*
 // ------------------------------------------------------------------ direction + W = L P (FP64 form)
 // P_s = Z_s' + beta_s P_{s-1} (Algorithm 1, with Z centred), W = L P, <W, P>
 // and the step length alpha = rho / <W, P>.
+template <bool APART>
 struct OpDirection {
   using Pre = NoPre;
   double* __restrict__ P;
@@ -531,7 +551,7 @@ struct OpDirection {
   __device__ __forceinline__ NoPre load(unsigned) const { return NoPre{}; }
   __device__ __forceinline__ void operator()(unsigned i, int, int, int, NoPre, double c, double xl, double xr, double yl,
                                              double yr, double zl, double zr) {
-    const double w = stencil_f64<false>(c, xl, xr, yl, yr, zl, zr, wt);
+    const double w = stencil_f64<false, APART>(c, xl, xr, yl, yr, zl, zr, wt);
     P[i] = c;
     W[i] = w;
     wp = fma(w, c, wp);
@@ -552,6 +572,7 @@ __device__ void fin_direction(SolveState* st, const double (&s)[1], const Geom& 
   for (int m = 0; m < 3; ++m) st->nah[m] = -alpha * g.ih2[m];
 }
 
+template <bool APART>
 __global__ void __launch_bounds__(TX* TY) k_direction(Geom g, const double* __restrict__ Z,
                                                       double* __restrict__ P0, double* __restrict__ P1,
                                                       double* __restrict__ W, SolveState* st, double* partials) {
@@ -559,7 +580,7 @@ __global__ void __launch_bounds__(TX* TY) k_direction(Geom g, const double* __re
   double* P = (st->iter & 1) ? P1 : P0;  // P_s in buffer s & 1
   const double* Pold = (st->iter & 1) ? P0 : P1;
   FieldDirection f{Z, Pold, st->mZ, st->beta, st->first};
-  OpDirection op{P, W, weights_of(g), 0.0};
+  OpDirection<APART> op{P, W, weights_of(g), 0.0};
   stencil_sweep_fx<double, 1>(g, f, op, partials, st, kTkDir,
                    [g](SolveState* st, const double(&s)[1]) { fin_direction(st, s, g); });
 }
@@ -1765,6 +1786,7 @@ __global__ void __launch_bounds__(256) k_jacobi_first(Geom g, const double* __re
     X[i] = __ldg(R + i) * jacobi_invd(t, g, (unsigned)i);
 }
 
+template <bool APART>
 struct OpJacobi {
   using Pre = double;  // R at the point
   const double* __restrict__ R;
@@ -1775,15 +1797,16 @@ struct OpJacobi {
   __device__ __forceinline__ double load(unsigned i) const { return __ldg(R + i); }
   __device__ __forceinline__ void operator()(unsigned i, int, int, int, double r, double c, double xl, double xr,
                                              double yl, double yr, double zl, double zr) {
-    Xnew[i] = fma(r - stencil_f64<true>(c, xl, xr, yl, yr, zl, zr, wt), jacobi_invd(t, g, i), c);
+    Xnew[i] = fma(r - stencil_f64<true, APART>(c, xl, xr, yl, yr, zl, zr, wt), jacobi_invd(t, g, i), c);
   }
 };
 
+template <bool APART>
 __global__ void __launch_bounds__(TX* TY) k_jacobi_sweep(Geom g, const double* __restrict__ Xold,
                                                          double* __restrict__ Xnew, const double* __restrict__ R,
                                                          JacobiTable t) {
   FieldPlain f{Xold};
-  OpJacobi op{R, Xnew, t, g, weights_of(g)};
+  OpJacobi<APART> op{R, Xnew, t, g, weights_of(g)};
   stencil_sweep_fx<double, 0>(g, f, op, nullptr, nullptr, 0, NoFin{});
 }
 
@@ -1885,7 +1908,8 @@ __global__ void __launch_bounds__(TX* TY) k_efield(Geom g, const double* __restr
 // ------------------------------------------------------------------ host launchers
 void launch_apply_laplacian(const tpcg_plan* p, const Geom& g, const double* x, double* w) {
   LaunchScope ls(p, kKApply);
-  k_apply_laplacian<<<p->fx_blocks[kFxApply], p->st_block, 0, p->stream>>>(g, x, w);
+  const auto k = weights_apart(p) ? k_apply_laplacian<true> : k_apply_laplacian<false>;
+  k<<<p->fx_blocks[kFxApply], p->st_block, 0, p->stream>>>(g, x, w);
 }
 // Persistent grids of the fixed-point sweeps: every SM holds as many blocks as
 // the kernel's resources allow (at most 8), and every block takes at least
@@ -1906,12 +1930,14 @@ int setup_fx_grids(tpcg_plan* p) {
   const bool f64 = p->prec == TPCG_FP64;
   const bool pair = !f64 && p->nx % 2 == 0;  // direction and update take two x points per thread
   const bool quad = !f64 && p->nx % 4 == 0;  // direction takes four
-  const void* fns[kFxCount] = {f64    ? (const void*)k_direction
+  const bool apart = weights_apart(p);
+  const void* fns[kFxCount] = {f64    ? (apart ? (const void*)k_direction<true> : (const void*)k_direction<false>)
                                : quad ? (const void*)k_direction_quad
                                       : (pair ? (const void*)k_direction_pair : (const void*)k_direction_int),
                                pair ? (const void*)k_update_pair : (const void*)k_update_int,
                                (const void*)k_residual_fx<false>, (const void*)k_residual_fx<true>,
-                               (const void*)k_apply_laplacian, (const void*)k_efield};
+                               apart ? (const void*)k_apply_laplacian<true> : (const void*)k_apply_laplacian<false>,
+                               (const void*)k_efield};
   for (int i = 0; i < kFxCount; ++i) {
     const int tw = (i == kFxDir && quad) ? 4 * TX : (((i == kFxUpd || i == kFxDir) && pair) ? 2 * TX : TX);
     const long long T = (long long)((p->nx + tw - 1) / tw) * ((p->ny + TY - 1) / TY) * p->nz;
@@ -1980,9 +2006,9 @@ static DirRing dir_ring(const tpcg_plan* p) {
 void launch_direction(const tpcg_plan* p, const Geom& g) {
   LaunchScope ls(p, kKDirection);
   if (p->prec == TPCG_FP64) {
-    k_direction<<<p->fx_blocks[kFxDir], p->st_block, 0, p->stream>>>(g, (const double*)p->d_Z, (double*)p->d_P[0],
-                                                                      (double*)p->d_P[1], p->d_W, p->d_state,
-                                                                      p->d_partials);
+    const auto k = weights_apart(p) ? k_direction<true> : k_direction<false>;
+    k<<<p->fx_blocks[kFxDir], p->st_block, 0, p->stream>>>(g, (const double*)p->d_Z, (double*)p->d_P[0],
+                                                            (double*)p->d_P[1], p->d_W, p->d_state, p->d_partials);
     return;
   }
   const DirRing ring = dir_ring(p);
@@ -2094,7 +2120,8 @@ void run_precond_cmp(const tpcg_plan* p, const Geom& g, const double* R, double*
     }
     for (int j = 2; j <= p->jac_p; ++j) {
       LaunchScope ls(p, kKModeF64);
-      k_jacobi_sweep<<<p->fx_blocks[kFxApply], p->st_block, 0, p->stream>>>(g, buf(j - 1), buf(j), R, t);
+      const auto k = weights_apart(p) ? k_jacobi_sweep<true> : k_jacobi_sweep<false>;
+      k<<<p->fx_blocks[kFxApply], p->st_block, 0, p->stream>>>(g, buf(j - 1), buf(j), R, t);
     }
   }
   if (st || p->pc_kind == TPCG_PRECOND_NONE) {

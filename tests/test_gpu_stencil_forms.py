@@ -44,3 +44,46 @@ def test_infinity_stays_an_infinity(shape, h, bad):
             ref[k + d, 3, 4] = -bad
     assert np.array_equal(apply_gpu(pl, x), ref)
     pl.close()
+
+
+def neighbours(x, axis):
+    """Start and end neighbours of every point along an array axis, Dirichlet ghosts."""
+    z = np.zeros_like(np.take(x, [0], axis))
+    e = np.concatenate([z, x, z], axis)
+    return np.take(e, range(x.shape[axis]), axis), np.take(e, range(2, x.shape[axis] + 2), axis)
+
+
+@pytest.mark.parametrize("shape", [(33, 9, 7), (20, 34, 3), (40, 24, 1)])
+@pytest.mark.parametrize("h", [(1.0, 1.0, 2.0), (1.0, 0.49, 1.0), (2.0**-8, 1.0, 16.0), (1.0, 0.01, 3.0), (0.1, 1.0, 10.0),
+                               (50.0, 1.0, 0.02)])
+def test_unequal_spacings_large_values_on_a_weak_axis(shape, h):
+    """Every second plane, row or column 2^12 to 2^40 times larger than the others: where the axis across them has the
+    small weight, the other axes' differences must keep their own accuracy.
+
+    Bound as for any sum of the seven terms in FP64: 4 x 2^-52 of the sum of their magnitudes (a conversion, a product and
+    the sums of the axes), per point, against extended precision.
+    """
+    from paper_2501_03377_gb300 import Plan
+
+    nx, ny, nz = shape
+    pl = Plan(nx, ny, nz, ("D", "D", "D"), h)
+    rng = np.random.default_rng(51)
+    base = rng.standard_normal((nz, ny, nx))
+    for axis in range(3):
+        if base.shape[axis] == 1:
+            continue
+        odd = np.indices(base.shape)[axis] % 2 == 1
+        for k in (12, 26, 40):
+            x = np.where(odd, np.ldexp(base, k), base)
+            w = apply_gpu(pl, x)
+            X = x.astype(np.longdouble)
+            ref, mag = np.zeros_like(X), np.zeros_like(X)
+            for m in range(3):
+                if X.shape[2 - m] == 1:
+                    continue
+                lo, hi = neighbours(X, 2 - m)
+                ref += (2 * X - lo - hi) / np.longdouble(h[m]) ** 2
+                mag += (2 * np.abs(X) + np.abs(lo) + np.abs(hi)) / np.longdouble(h[m]) ** 2
+            worst = (np.abs(w - ref) / mag).max()
+            assert worst <= 4 * 2.0**-52, (axis, k, float(worst * 2.0**52))
+    pl.close()
