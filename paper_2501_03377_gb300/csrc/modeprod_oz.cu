@@ -492,12 +492,16 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
   }
 }
 
+// Bytes of one direction's digit images of an axis and its column scales, which follow them.
+size_t oz_digits(int l) { return (size_t)((l + 127) / 128) * ((l + 63) / 64) * kDig * kOzImg; }
+size_t oz_image_bytes(int l) { return oz_digits(l) + (size_t)((l + 127) / 128) * 128 * sizeof(int); }
+
 // The digit images of an eigenbasis matrix W (l x l, row-major, contraction index first) and the power-of-two
 // scale of each column: column c' as seven base-256 digits at every k, 64-wide K tiles of 128 columns under the
 // 128-byte swizzle; zero past l.
-void digit_image(const std::vector<double>& W, int l, int MB, int KT, std::vector<uint8_t>& out) {
-  const size_t img = (size_t)MB * KT * kDig * kOzImg;
-  out.assign(img + (size_t)MB * 128 * sizeof(int), 0);
+void digit_image(const std::vector<double>& W, int l, int KT, std::vector<uint8_t>& out) {
+  const size_t img = oz_digits(l);
+  out.assign(oz_image_bytes(l), 0);
   uint16_t f16[257];  // FP16 of -128 .. 128
   for (int d = -128; d <= 128; ++d) {
     const int v = d < 0 ? -d : d;
@@ -549,6 +553,14 @@ static_assert(kOzSmem <= (size_t)kMaxSmem && kOzSmem == sole_smem(kOzSmem), "sha
 // Axes whose products run on the digits (others: k_modeprod_f64).
 bool oz_axis_ok(int l) { return l > 1 && l <= 64 * kOzMaxKT; }
 
+// What oz_plan_setup allocates: the images of both directions of an axis, and G where the pass that applies it runs here.
+size_t oz_device_bytes(int nx, int ny, int nz) {
+  size_t b = 0;
+  for (int l : {nx, ny, nz})
+    if (oz_axis_ok(l)) b += 2 * oz_image_bytes(l);
+  return b + (oz_axis_ok(nz > 1 ? nz : ny) ? (size_t)nx * ny * nz * sizeof(double) : 0);
+}
+
 int oz_plan_setup(tpcg_plan* p) {
   const int lens[3] = {p->nx, p->ny, p->nz};
   bool any = false;
@@ -556,13 +568,13 @@ int oz_plan_setup(tpcg_plan* p) {
     const int l = lens[m];
     if (!oz_axis_ok(l)) continue;
     any = true;
-    const int MB = (l + 127) / 128, KT = (l + 63) / 64;
+    const int KT = (l + 63) / 64;
     std::vector<double> VT((size_t)l * l);
     for (int i = 0; i < l; ++i)
       for (int j = 0; j < l; ++j) VT[(size_t)j * l + i] = p->ax[m].V[(size_t)i * l + j];
     std::vector<uint8_t> img;
     for (int d = 0; d < 2; ++d) {
-      digit_image(d ? VT : p->ax[m].V, l, MB, KT, img);
+      digit_image(d ? VT : p->ax[m].V, l, KT, img);
       if (cudaMalloc((void**)&p->d_oz[m][d], img.size()) != cudaSuccess) {
         cudaGetLastError();
         p->d_oz[m][d] = nullptr;

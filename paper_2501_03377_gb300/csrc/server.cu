@@ -23,6 +23,10 @@
 #include "tpcg_dev.cuh"
 
 namespace tpcg {
+
+size_t oz_device_bytes(int nx, int ny, int nz);
+bool oz_axis_ok(int l);
+
 namespace {
 
 using Clock = std::chrono::steady_clock;
@@ -96,6 +100,7 @@ struct tpcg_server {
   int device = 0;
   size_t budget = 0;
   int max_slots = 0;
+  int num_sms = 1;
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
   bool shutdown = false;
@@ -141,18 +146,28 @@ void pinned_put(tpcg_server* s, size_t bytes, void* p) {
 
 // Device bytes a plan of this key will hold, plus the slot's eta/ups buffers
 // (upper estimate matching tpcg_plan_create's allocations).
-size_t estimate_slot_bytes(const PlanKey& k) {
+size_t estimate_slot_bytes(const PlanKey& k, int num_sms) {
   const size_t N = (size_t)k.nx * k.ny * k.nz;
   const bool fp64 = (k.prec == TPCG_FP64);
   // bytes of a tensor-core operand (TF32: FP32 containers; split: hi and lo BF16 planes)
   const size_t lpb = (k.prec == TPCG_MIXED_TF32 || k.prec == TPCG_MIXED_BF16X3) ? 4 : 2;
   size_t b = N * 8 + (fp64 ? N * 8 * 3 : N * 4 * 2);  // R; P[2] and W (FP64) or P[2] in int32
   b += N * (fp64 ? 8 : 4);                   // Z
-  b += fp64 ? 0 : N * lpb + (size_t)k.ny * k.nz * 8 * lpb;  // low-precision copy of R (padded rows)
-  b += 2 * N * (fp64 ? 8 : lpb) + 2 * (size_t)(k.nx + k.ny + k.nz) * 64;  // mode-product intermediates
-  const size_t l2 = (size_t)k.nx * k.nx + (size_t)k.ny * k.ny + (size_t)k.nz * k.nz;
-  b += l2 * (16 + (fp64 ? 0 : 4 * lpb));     // eigenbases
-  b += (1 << 20) + 16384 * 4 * 8;            // state, partial sums, slack
+  if (fp64) {
+    // digit images and G; the matrices of the axes without images; eigenvalues
+    b += oz_device_bytes(k.nx, k.ny, k.nz);
+    for (int l : {k.nx, k.ny, k.nz}) b += (oz_axis_ok(l) ? 0 : (size_t)l * l * 16) + (size_t)l * 12 + 128;
+    // partial sums: a slot of four doubles per block of the largest reducing launch; the state
+    const size_t tiles = (size_t)((k.nx + 31) / 32) * ((k.ny + 7) / 8) * k.nz + (size_t)num_sms * 8;
+    const size_t last = (((size_t)k.ny * k.nz + 63) / 64) * ((k.nx + 63) / 64);
+    b += std::max<size_t>(16384, std::max(tiles, last)) * 4 * 8 + sizeof(SolveState) + 64;
+  } else {
+    b += N * lpb + (size_t)k.ny * k.nz * 8 * lpb;  // low-precision copy of R (padded rows)
+    b += 2 * N * lpb + 2 * (size_t)(k.nx + k.ny + k.nz) * 64;  // mode-product intermediates
+    const size_t l2 = (size_t)k.nx * k.nx + (size_t)k.ny * k.ny + (size_t)k.nz * k.nz;
+    b += l2 * (16 + 4 * lpb);                // eigenbases; room for the partial sums of large grids
+    b += (1 << 20) + 16384 * 4 * 8;          // state, partial sums, slack
+  }
   b += N * 8 * 2;                            // slot's eta / ups buffers
   return b;
 }
@@ -247,7 +262,7 @@ bool try_admit(tpcg_server* s, Request* r, bool* reject) {
     if (sit == s->sessions.end() || sit->second.N != r->N) ses_need = (size_t)r->N * 8;
     else ses = &sit->second;
   }
-  const size_t slot_need = (slot == s->slots.end()) ? estimate_slot_bytes(r->key) : 0;
+  const size_t slot_need = (slot == s->slots.end()) ? estimate_slot_bytes(r->key, s->num_sms) : 0;
   if (slot != s->slots.end()) slot->req = r;  // reserved: not an eviction candidate
   auto unreserve = [&]() {
     if (slot != s->slots.end()) slot->req = nullptr;
@@ -464,6 +479,7 @@ int tpcg_server_create(size_t hbm_budget, int max_slots, tpcg_server** out) {
     delete s;
     return TPCG_ERR_CUDA;
   }
+  cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, s->device);
   if (hbm_budget == 0) {
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {

@@ -140,3 +140,28 @@ def test_server_borrowed_rhs_equal_copied():
     srv.close()
     assert all(st == 0 for st, _, _ in out)
     assert np.array_equal(out[0][1], out[1][1]) and np.array_equal(out[0][1], out[2][1])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "bf16", "fp16", "tf32", "bf16x3"])
+@pytest.mark.parametrize("shape", [(129, 129, 1), (193, 193, 1), (129, 129, 3), (3, 200, 200), (256, 3, 256), (256, 256, 128), (256, 256, 256),
+                                   (3, 3, 3), (257, 9, 300)])
+def test_server_admits_only_what_fits(shape, prec):
+    """A budget one byte below what the plan and its buffers hold refuses the request; in the FP64 form, whose estimate
+    counts the allocations one by one, 16 KB more than they hold takes it."""
+    from paper_2501_03377_gb300 import Plan, Server, binding
+
+    nx, ny, nz = shape
+    bcs = ("P", "D", "N")
+    if prec != "fp64" and max(shape) > 256:
+        pytest.skip("tensor-core forms take axes of at most 256 points")
+    pl = Plan(nx, ny, nz, bcs, prec=prec)
+    held = pl.device_bytes() + 16 * nx * ny * nz
+    pl.close()
+    eta = synth.random_field(nx, ny, nz, seed=61)
+    cases = [(held - 1, binding.TPCG_ERR_ADMISSION)] + ([(held + (16 << 10), 0)] if prec == "fp64" else [])
+    for budget, want in cases:
+        srv = Server(hbm_budget=budget, max_slots=1)
+        st, _, _ = srv.wait(srv.submit(eta, bcs, prec=prec), 60.0)
+        assert st == want
+        assert srv.stats()["device_bytes"] <= budget
+        srv.close()
