@@ -295,7 +295,10 @@ int tpcg_solve_batched(tpcg_plan* const* plans, int nsolves, const int* nrhs, co
 /* z = M(r): one application of the plan's preconditioner (Algorithm 7 in the
  * plan's precision form, or the comparator chosen by tpcg_plan_set_precond),
  * without centring.  r, z: device pointers of nz*ny*nx doubles (may not
- * alias).  Enqueues only.                                                    */
+ * alias).  Enqueues only: where a bounded wait gives up inside the application
+ * (a GPU held by others for seconds) z stays incomplete, and the plan's next
+ * call of this function that finds it so returns TPCG_ERR_TIMEOUT and enqueues
+ * nothing.                                                                   */
 int tpcg_precond_apply(tpcg_plan* plan, const double* r, double* z);
 
 /* ---- comparator preconditioners (Sec. 4.3.1; Experiment 2, Sec. 5) ------ */

@@ -182,7 +182,6 @@ void free_plan(tpcg_plan* p) {
   if (p->s_out) cudaStreamDestroy(p->s_out);
   cudaFree(p->d_state);
   cudaFree(p->d_partials);
-  cudaFree(p->d_err);
   if (p->h_state) cudaFreeHost(p->h_state);
   if (p->ev_state) cudaEventDestroy(p->ev_state);
   for (cudaEvent_t e : p->prof.pool) cudaEventDestroy(e);
@@ -264,6 +263,14 @@ int run_precond(const tpcg_plan* p, const double* R, void* Z, SolveState* st) {
     return TPCG_OK;
   }
   return run_precond_tc(p, (float*)Z, st);
+}
+
+// Whether a wait of an earlier application outside a solve gave up, once.
+bool take_give_up(tpcg_plan* p) {
+  volatile int* word = p->h_err;
+  if (!*word) return false;
+  *word = 0;
+  return true;
 }
 
 int last_cuda_error() {
@@ -681,12 +688,12 @@ int tpcg_plan_create(int nx, int ny, int nz, const int bc[3], const double h[3],
     p->partial_slots = (size_t)std::max(16384LL, most) * 4;
   }
   if (!rc) rc = dalloc(p, &p->d_partials, p->partial_slots);
-  if (!rc) rc = dalloc(p, &p->d_err, 4);
-  if (!rc && cudaMallocHost((void**)&p->h_state, sizeof(SolveState)) != cudaSuccess) rc = TPCG_ERR_OOM;
+  if (!rc && cudaMallocHost((void**)&p->h_state, sizeof(SolveState) + sizeof(int)) != cudaSuccess) rc = TPCG_ERR_OOM;
   if (!rc && cudaEventCreateWithFlags(&p->ev_state, cudaEventDisableTiming) != cudaSuccess) rc = TPCG_ERR_CUDA;
   if (!rc) {
     cudaMemset(p->d_state, 0, sizeof(SolveState));
-    cudaMemset(p->d_err, 0, 16);
+    p->h_err = reinterpret_cast<int*>(p->h_state + 1);
+    *p->h_err = 0;
   }
   // launch configuration, fixed per plan (reproducible reductions)
   if (!rc) {
@@ -975,6 +982,7 @@ int tpcg_plan_set_option(tpcg_plan* plan, int option, int value) {
 
 int tpcg_precond_apply(tpcg_plan* plan, const double* r, double* z) {
   if (!plan || !r || !z || r == z) return TPCG_ERR_INVALID_ARG;
+  if (take_give_up(plan)) return TPCG_ERR_TIMEOUT;  // an earlier application's
   DeviceGuard dg(plan->device);
   int rc;
   if (plan->prec == TPCG_FP64) {
@@ -1128,6 +1136,7 @@ int tpcg_plan_autotune(tpcg_plan* plan, const char* cache_path, int applies, tpc
     }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (!rc && take_give_up(plan)) rc = TPCG_ERR_TIMEOUT;
   plan->tc_slab = rc ? slab0 : best_s;
   plan->tc_fuse = rc ? fuse0 : best_f;
   graph_reset(plan);

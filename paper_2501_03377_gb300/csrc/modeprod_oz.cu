@@ -638,7 +638,7 @@ bool run_pass_oz(const tpcg_plan* p, const StageParams& sp, const double* X, dou
   a.st = st;
   a.partials = p->d_partials;
   a.N = p->N;
-  a.err = p->d_err;
+  a.err = p->h_err;
   const int ntiles = (a.rows + kOzRows - 1) / kOzRows;
   const int grid = std::min(ntiles, p->num_sms);
   a.iters = (ntiles + grid - 1) / grid;

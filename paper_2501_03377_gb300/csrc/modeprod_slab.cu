@@ -881,7 +881,7 @@ int slab_plan_setup(tpcg_plan* p) {
   base.Rt = reinterpret_cast<const uint16_t*>(p->d_Rlp);
   base.rpitch = p->pitch16[0];
   base.N = p->N;
-  base.err = p->d_err;
+  base.err = p->h_err;
   const size_t C = (size_t)q * n;  // columns of a z row of the intermediates ([t][q'][n'], no padding)
   if (p->t_elems < C * (size_t)t) {
     delete sp;

@@ -1837,7 +1837,7 @@ int tc_plan_setup(tpcg_plan* p) {
     a.lamB = p->d_lam32[sp.lamB];
     a.lamC = p->d_lam32[sp.lamC];
     a.N = p->N;
-    a.err = p->d_err;
+    a.err = p->h_err;
     a.last = sp.final_stage;
     a.sG = sG;
     a.gscale = std::ldexp(1.0f, -sG);

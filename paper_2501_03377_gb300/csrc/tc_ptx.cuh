@@ -43,7 +43,7 @@ __device__ __forceinline__ unsigned long long gtimer() {
 
 struct Abort {
   volatile int* flag;  // shared
-  int* err;            // global error word
+  int* err;            // the plan's error word (pinned host memory), for launches without a state
   SolveState* st;
 };
 
@@ -56,8 +56,8 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, cons
     if (*ab.flag) return false;
     if (gtimer() - t0 > kWaitLimitNs) {
       *ab.flag = 1;
-      if (ab.err) atomicExch(ab.err, 1);
       if (ab.st) ab.st->timeout = 1;
+      else if (ab.err) *reinterpret_cast<volatile int*>(ab.err) = 1;
       return false;
     }
   }

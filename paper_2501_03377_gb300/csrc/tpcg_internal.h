@@ -175,7 +175,9 @@ struct tpcg_plan {
   cudaEvent_t ev_state = nullptr;        // recorded after each read-back of the device state
   double* d_partials = nullptr;
   size_t partial_slots = 0;
-  int* d_err = nullptr;   // device error word of bounded waits
+  // pinned, behind h_state: set by a bounded wait that gave up in an application outside a solve (which has no device
+  // state to say so in); taken by the plan's next application
+  int* h_err = nullptr;
 
   std::vector<tpcg::StageParams> stages;
   void* tc_state = nullptr;   // tensor-core pass descriptors (tensor maps, launch shapes)

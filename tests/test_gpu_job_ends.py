@@ -1,0 +1,58 @@
+"""Ends that only a held-up GPU reaches, presented to the host code by hooks (no wait runs out here)."""
+import ctypes
+import subprocess
+
+import pytest
+
+from inputs import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def hooks(tmp_path_factory):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import os
+
+    from paper_2501_03377_gb300 import build
+
+    lib = build.build()
+    out = str(tmp_path_factory.mktemp("hooks") / "hooks.so")
+    src = os.path.join(os.path.dirname(__file__), "_job_hooks.cu")
+    subprocess.run([build._nvcc(), *build.ARCH, *build.COMMON, "-shared", src,
+                    "-o", out, lib, "-Xlinker", "-rpath=" + os.path.dirname(lib)], check=True)
+    return ctypes.CDLL(out)
+
+
+def plan_and_fields(prec):
+    from paper_2501_03377_gb300 import Plan
+
+    bcs = ("P", "D", "N")
+    pl = Plan(40, 24, 12, bcs, prec=prec)
+    eta = torch.from_numpy(synth.random_field(40, 24, 12, seed=71)).cuda()
+    return pl, eta, torch.zeros_like(eta)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "bf16x3"])
+def test_application_that_gave_up_is_reported_once(hooks, prec):
+    from paper_2501_03377_gb300 import binding
+
+    pl, r, z = plan_and_fields(prec)
+    apply = lambda: binding.tpcg_precond_apply(pl.handle, r.data_ptr(), z.data_ptr())  # noqa: E731
+    assert apply() == 0
+    torch.cuda.synchronize()
+    ref = z.clone()
+    hooks.hook_give_up(pl.handle)
+    z.zero_()
+    assert apply() == binding.TPCG_ERR_TIMEOUT
+    torch.cuda.synchronize()
+    assert not bool(z.any())  # nothing was enqueued
+    st, info = pl.solve(r, z.clone(), tol=1e-10, maxit=50, zero_guess=True)
+    assert st == 0
+    assert apply() == 0
+    torch.cuda.synchronize()
+    assert torch.equal(z, ref)
+    pl.close()
