@@ -929,12 +929,9 @@ int tpcg_plan_set_option(tpcg_plan* plan, int option, int value) {
     if (value < 1 || value > 64) return TPCG_ERR_INVALID_ARG;
     DeviceGuard dg(plan->device);
     const int old = plan->sweep_grain;
-    const bool old_set = plan->sweep_grain_set;
     plan->sweep_grain = value;
-    plan->sweep_grain_set = true;
     if (setup_fx_grids(plan)) {
       plan->sweep_grain = old;
-      plan->sweep_grain_set = old_set;
       setup_fx_grids(plan);
       return TPCG_ERR_CUDA;
     }

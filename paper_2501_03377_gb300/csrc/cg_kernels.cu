@@ -1919,10 +1919,11 @@ void launch_apply_laplacian(const tpcg_plan* p, const Geom& g, const double* x, 
 int setup_fx_grids(tpcg_plan* p) {
   // The default grain of 4 gives way where it would leave SMs without a block: a small grid's time is the chain of
   // planes of one block (64 x 64 plane 105 -> 95 us, 64 x 64 x 32 step 230 -> 220 at grain 1-2; 96 x 96 x 48 is 2 % slower
-  // below 4).  A grain that the caller has set is kept.
+  // below 4).  Any other grain is kept.
+  const bool deflt = p->sweep_grain == kDefaultGrain;
   auto grain_of = [&](long long units) {
     const long long g = p->sweep_grain;
-    return p->sweep_grain_set ? g : std::max(1LL, std::min(g, units / p->num_sms));
+    return deflt ? std::max(1LL, std::min(g, units / p->num_sms)) : g;
   };
   const long long sg = grain_of((p->N + 255) / 256);
   p->stream_blocks = (int)std::max(1LL, std::min<long long>((p->N + 256 * sg - 1) / (256 * sg),
@@ -1946,7 +1947,7 @@ int setup_fx_grids(tpcg_plan* p) {
     per_sm = std::max(1, std::min(per_sm, 8));
     // the Laplacian and the field end without a reduction, whose cost per block a grain limits: down to one plane a
     // block (both together at 101 x 80 x 33 24.6 -> 20.6 us, at 48 x 40 x 100 16.4 -> 13.5; large grids the same)
-    const bool free_blocks = !p->sweep_grain_set && (i == kFxApply || i == kFxField);
+    const bool free_blocks = deflt && (i == kFxApply || i == kFxField);
     const long long grain = free_blocks ? 1 : grain_of(T);
     p->fx_blocks[i] = (int)std::max(1LL, std::min<long long>((T + grain - 1) / grain, (long long)p->num_sms * per_sm));
   }

@@ -60,6 +60,7 @@ struct SolveState;  // device-side scalars (tpcg_dev.cuh)
 
 // Kernel kinds for the launch counter and the optional event profiler.
 // Persistent fixed-point sweeps (grid size per kernel, from its occupancy).
+constexpr int kDefaultGrain = 4;  // TPCG_OPT_SWEEP_GRAIN: a rule of its own, see setup_fx_grids
 enum FxKernel { kFxDir = 0, kFxUpd, kFxTrue, kFxInit, kFxApply, kFxField, kFxCount };
 
 enum KernelKind {
@@ -188,8 +189,7 @@ struct tpcg_plan {
 
   // launch configuration (fixed per plan so that reductions are reproducible)
   dim3 st_block;            // stencil kernels
-  bool sweep_grain_set = false;  // the caller chose the grain
-  int sweep_grain = 4;  // TPCG_OPT_SWEEP_GRAIN: least (tile, plane) pairs (x 256 points) per sweep block
+  int sweep_grain = tpcg::kDefaultGrain;  // TPCG_OPT_SWEEP_GRAIN: least (tile, plane) pairs (x 256 points) per sweep block
   int fx_blocks[tpcg::kFxCount] = {1, 1, 1, 1, 1, 1};  // FxKernel -> blocks of the persistent fixed-point sweeps
   // comparator preconditioner of the FP64 form (TPCG_PRECOND_*), Jacobi(p, omega) and its table of
   // 1 / (omega d) indexed by the boundary class (start, interior, end) of x + 3 y + 9 z
