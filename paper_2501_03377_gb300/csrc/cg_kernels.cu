@@ -619,10 +619,10 @@ struct DirRing {
 // (tile, plane) pairs, walked as runs of consecutive planes of one tile.
 // Ghosts: ghost_index() maps a neighbour across a boundary to the wrapped
 // index (P), the point itself (N: mirror) or -1 (D: the value 0).
-template <int TW = TX, class Run>
-__device__ __forceinline__ void for_each_run(const Geom& g, Run run) {
-  const unsigned bxn = (unsigned)(g.nx + TW - 1) / TW, byn = (unsigned)(g.ny + TY - 1) / TY;
-  const unsigned T = bxn * byn * (unsigned)g.nz;
+// for_each_span: the block's runs of planes [k0, k1) of `tiles` columns of tiles.
+template <class Run>
+__device__ __forceinline__ void for_each_span(const Geom& g, unsigned tiles, Run run) {
+  const unsigned T = tiles * (unsigned)g.nz;
   const unsigned G = gridDim.x, q = T / G, rm = T - q * G;
   const unsigned t_begin = blockIdx.x * q + min(blockIdx.x, rm);
   const unsigned t_end = t_begin + q + (blockIdx.x < rm ? 1u : 0u);
@@ -631,9 +631,16 @@ __device__ __forceinline__ void for_each_run(const Geom& g, Run run) {
     const int k0 = (int)(t - tile * (unsigned)g.nz);
     const int k1 = (int)min((unsigned)g.nz, (unsigned)k0 + (t_end - t));
     t += (unsigned)(k1 - k0);
+    run(tile, k0, k1);
+  }
+}
+template <int TW = TX, class Run>
+__device__ __forceinline__ void for_each_run(const Geom& g, Run run) {
+  const unsigned bxn = (unsigned)(g.nx + TW - 1) / TW, byn = (unsigned)(g.ny + TY - 1) / TY;
+  for_each_span(g, bxn * byn, [&](unsigned tile, int k0, int k1) {
     const unsigned tyi = tile / bxn;
     run((int)(tile - tyi * bxn) * TW, (int)tyi * TY, k0, k1);
-  }
+  });
 }
 
 __global__ void __launch_bounds__(TX* TY) k_direction_int(Geom g, const float* __restrict__ Z, DirRing ring, SolveState* st, double* partials) {
@@ -1856,10 +1863,12 @@ __device__ __forceinline__ double scaled_diff(double lo, double hi, const FieldS
   return d * s.f;
 }
 
-// A thread owns the column (x, y) of a 32 x 8 tile and marches in z with the z neighbours in registers (see
-// k_direction_int); the x and y neighbours come from the cache.  Six FP64 operations a point (a difference and a product
-// per axis) bound the plain form: 115 us at 256 x 256 x 128, where the memory needs 39.  With a power of two for
-// 1 / (2 h) the product is an integer operation.
+// A thread owns a column (x, y) and marches in z with the z neighbours in registers (see k_direction_int); the x and y
+// neighbours come from the cache.  A block takes 256 consecutive columns of the plane: 32 x 8 tiles left most of their
+// threads without a column on narrow or odd planes (8 x 512 x 512 87 us against 25, 3 x 700 x 700 159 against 19,
+// 130 x 130 x 130 33 against 26) and gain nothing on the others (256 x 256 x 128 88 against 87).  Six FP64 operations a
+// point (a difference and a product per axis) bound the plain form: 115 us at 256 x 256 x 128, where the memory needs 39.
+// With a power of two for 1 / (2 h) the product is an integer operation.
 __global__ void __launch_bounds__(TX* TY) k_efield(Geom g, const double* __restrict__ U, FaceData fd, FieldScale sx,
                                                    FieldScale sy, FieldScale sz, double* __restrict__ ex,
                                                    double* __restrict__ ey, double* __restrict__ ez) {
@@ -1872,10 +1881,10 @@ __global__ void __launch_bounds__(TX* TY) k_efield(Geom g, const double* __restr
     const double v = fd.v[2 * m + (end ? 1 : 0)];
     return dir ? v : fma(fd.h[m], v, u0);
   };
-  for_each_run(g, [&](int bx0, int by0, int k0, int k1) {
-    const int x = bx0 + (int)threadIdx.x, y = by0 + (int)threadIdx.y;
-    if (x >= g.nx || y >= g.ny) return;
-    const unsigned col = (unsigned)y * nx + (unsigned)x;
+  for_each_span(g, (plane + TX * TY - 1) / (TX * TY), [&](unsigned tile, int k0, int k1) {
+    const unsigned col = tile * (TX * TY) + threadIdx.y * TX + threadIdx.x;
+    if (col >= plane) return;
+    const int y = (int)(col / nx), x = (int)(col - (unsigned)y * nx);
     const bool px = g.bc[0] == kBcP, py = g.bc[1] == kBcP, pz = g.bc[2] == kBcP;
     // neighbours inside the grid (periodic faces wrapped); a face of another kind takes its ghost value
     const bool fxl = x == 0 && !px, fxr = x == g.nx - 1 && !px, fyl = y == 0 && !py, fyr = y == g.ny - 1 && !py;
@@ -1941,7 +1950,8 @@ int setup_fx_grids(tpcg_plan* p) {
                                (const void*)k_efield};
   for (int i = 0; i < kFxCount; ++i) {
     const int tw = (i == kFxDir && quad) ? 4 * TX : (((i == kFxUpd || i == kFxDir) && pair) ? 2 * TX : TX);
-    const long long T = (long long)((p->nx + tw - 1) / tw) * ((p->ny + TY - 1) / TY) * p->nz;
+    const long long T = (i == kFxField ? ((long long)p->nx * p->ny + TX * TY - 1) / (TX * TY)
+                                               : (long long)((p->nx + tw - 1) / tw) * ((p->ny + TY - 1) / TY)) * p->nz;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[i], TX * TY, 0) != cudaSuccess) return -1;
     per_sm = std::max(1, std::min(per_sm, 8));
@@ -1949,7 +1959,11 @@ int setup_fx_grids(tpcg_plan* p) {
     // block (both together at 101 x 80 x 33 24.6 -> 20.6 us, at 48 x 40 x 100 16.4 -> 13.5; large grids the same)
     const bool free_blocks = deflt && (i == kFxApply || i == kFxField);
     const long long grain = free_blocks ? 1 : grain_of(T);
-    p->fx_blocks[i] = (int)std::max(1LL, std::min<long long>((T + grain - 1) / grain, (long long)p->num_sms * per_sm));
+    // the field, without a ring to fill or a sum to reduce, in four waves of blocks: a last plane more or less weighs a
+    // quarter (3 x 700 x 700 with unequal spacings 23.0 -> 20.9 us, 256 x 256 x 128 109 -> 104)
+    const int waves = i == kFxField ? 4 : 1;
+    p->fx_blocks[i] = (int)std::max(1LL, std::min<long long>((T + grain - 1) / grain,
+                                                             (long long)p->num_sms * per_sm * waves));
   }
   return 0;
 }

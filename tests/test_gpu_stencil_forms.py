@@ -87,3 +87,47 @@ def test_unequal_spacings_large_values_on_a_weak_axis(shape, h):
             worst = (np.abs(w - ref) / mag).max()
             assert worst <= 4 * 2.0**-52, (axis, k, float(worst * 2.0**52))
     pl.close()
+
+
+@pytest.mark.parametrize("shape", [(3, 700, 5), (8, 33, 4), (16, 16, 3), (5, 51, 1), (257, 3, 6), (255, 4, 3), (3, 3, 900)])
+def test_field_on_narrow_planes(shape):
+    """Planes below, at and above the 256 columns of a block: the exact differences, one rounding each (1 / (2 h) a power of
+    two) or two."""
+    from paper_2501_03377_gb300 import Plan
+
+    nx, ny, nz = shape
+    h = (1.0, 0.3, 0.25)
+    pl = Plan(nx, ny, nz, ("D", "D", "D"), h)
+    u = np.random.default_rng(52).standard_normal((nz, ny, nx))
+    ud = torch.from_numpy(u).cuda()
+    out = [torch.full_like(ud, float("nan")) for _ in range(3)]
+    pl.efield(ud, *out)
+    for m in range(3 if nz > 1 else 2):
+        lo, hi = neighbours(u, 2 - m)
+        assert np.array_equal(out[m].cpu().numpy(), (lo - hi) * (0.5 / h[m]))
+    pl.close()
+
+
+@pytest.mark.parametrize("narrow", [(8, 512, 512), (3, 700, 998)])
+def test_field_of_a_narrow_grid_costs_what_a_wide_one_does(narrow):
+    """The same number of points, twice the time at most (tiles 32 columns wide: 3.4 and 7 times)."""
+    from paper_2501_03377_gb300 import Plan
+
+    def best(shape):
+        nx, ny, nz = shape
+        pl = Plan(nx, ny, nz, ("D", "D", "D"))
+        u = torch.zeros((nz, ny, nx), dtype=torch.float64, device="cuda")
+        out = [torch.empty_like(u) for _ in range(3)]
+        times = []
+        for _ in range(8):
+            t = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            t[0].record()
+            for _ in range(10):
+                pl.efield(u, *out)
+            t[1].record()
+            torch.cuda.synchronize()
+            times.append(t[0].elapsed_time(t[1]))
+        pl.close()
+        return min(times)
+
+    assert best(narrow) <= 2.0 * best((512, 512, 8))
