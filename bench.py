@@ -34,6 +34,8 @@ if ROOT not in sys.path:
 
 METRIC = "256\u00b3 solves/s at rel-res 1e-10, TC-mixed vs FP64 PCG; serving p50/p99 ms"
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12  # SMs x FP64 FMA/clk/SM x 2 flop x max SM clock
+# The FP64 form's products of axes up to 256 points: exact FP16 digit products per FP64 product
+DIGIT_PRODUCTS = 28
 
 
 def parse():
@@ -558,8 +560,8 @@ def kernel_work(kind, plan_prec, N, dims, iters_total, applies_total, solves, ch
     lpb = {"fp16": 2, "bf16": 2, "tf32": 4, "bf16x3": 4}.get(plan_prec, 0)
     if kind == "modeprod_f64":
         npass = 6 if t > 1 else 4
-        if max(n, q, t) <= 256:  # 28 exact FP16 digit products per FP64 product, on the tensor cores
-            return applies_total * 28 * 4.0 * N * (n + q + t) / 1e12, "TFLOP", "tensor", applies_total * npass
+        if max(n, q, t) <= 256:  # as FP16 digit products on the tensor cores (DIGIT_PRODUCTS)
+            return applies_total * 4.0 * N * (n + q + t) / 1e12, "TFLOP", "tensor", applies_total * npass
         return applies_total * 4.0 * N * (n + q + t + 0.25) / 1e12, "TFLOP", "alu", applies_total * npass
     if kind == "modeprod_tc":
         # the per-point figure of the scope table for one application of the mixed preconditioner: about
@@ -799,11 +801,11 @@ def run_ours(args, rank, world, torch):
         secs = kstats[kind]["total_ms"] / 1e3
         achieved = amount / secs
         if unit == "TFLOP":
-            peak = FP64_PEAK_TFLOPS if bound == "alu" else bf16_sus
+            peak = FP64_PEAK_TFLOPS if bound == "alu" else bf16_sus / DIGIT_PRODUCTS
             return {"kernel": kind, "bound": bound, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": None,
                     "peak_source": "derived FP64: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz" if bound == "alu"
-                    else f"{peak_src} bf16 sustained"}
+                    else f"{peak_src} bf16 sustained / {DIGIT_PRODUCTS} FP16 digit products per FP64 product"}
         traffic = NCU_TRAFFIC_PER_LAUNCH.get(prec, {}).get(kind) if nz == 128 else None
         return {"kernel": kind, "bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                 "frac": achieved / hbm_peak, "traffic": traffic,

@@ -97,3 +97,11 @@ def test_kernel_work_counts_the_algorithmic_bytes():
     assert amount * 1e9 == pytest.approx(2 * 28 * N)
     amount, _, _, _ = bench.kernel_work("init_residual", "bf16x3", N, dims, 3, 4, 1, 2)
     assert amount * 1e9 == pytest.approx(1 * 20 * N)
+
+
+def test_kernel_work_counts_the_fp64_products_once():
+    """The digit products are how the tensor cores form an FP64 product: part of the peak, not of the work."""
+    N, dims = 256 * 256 * 128, (256, 256, 128)
+    amount, unit, _, worked = bench.kernel_work("modeprod_f64", "fp64", N, dims, 1, 3, 1, 1)
+    assert unit == "TFLOP" and worked == 18
+    assert abs(amount - 3 * 4.0 * N * 640 / 1e12) <= 1e-12 * amount
