@@ -1843,7 +1843,6 @@ __global__ void __launch_bounds__(256) k_dot_rz(long long N, const double* __res
 struct FaceData {
   double v[6];      // face data, start and end face per axis (0: homogeneous)
   double h[3];      // spacing per axis
-  double inv2h[3];  // 1 / (2 h)
 };
 
 // (lo - hi) * 2^e2 when the factor is a power of two (one FP64 operation, the scaling on the exponent field), else
@@ -2111,13 +2110,12 @@ void launch_efield(const tpcg_plan* p, const Geom& g, const double* U, const dou
   for (int m = 0; m < 6; ++m) fd.v[m] = bval ? bval[m] : 0.0;
   for (int m = 0; m < 3; ++m) {
     fd.h[m] = p->h[m];
-    fd.inv2h[m] = 0.5 / p->h[m];
   }
   FieldScale sc[3];
   for (int m = 0; m < 3; ++m) {
     int e = 0;
-    sc[m].f = fd.inv2h[m];
-    sc[m].pow2 = std::frexp(fd.inv2h[m], &e) == 0.5 ? 1 : 0;
+    sc[m].f = 0.5 / p->h[m];
+    sc[m].pow2 = std::frexp(sc[m].f, &e) == 0.5 ? 1 : 0;
     sc[m].e2 = e - 1;
   }
   k_efield<<<p->fx_blocks[kFxField], p->st_block, 0, p->stream>>>(g, U, fd, sc[0], sc[1], sc[2], ex, ey, ez);

@@ -15,10 +15,13 @@
 // of it is exact, and the digit products of one level s = i + j share an
 // accumulator: the four leading levels stay within 2^24 for any input; levels 4
 // to 6 could pass it only if nearly every digit of a row and of a column took its
-// largest value with matching signs, and then lose one unit of a level, 2^-48 of
-// row times column, the size of the FP64 accumulation's own bound.  Levels 7 to
-// 12 are dropped: together with the 55-bit rounding of the operands about 2^-54
-// of |row| |column|, below the error of the FP64 dot product (some 2^-51 here).
+// largest value with matching signs, and each accumulation past it then loses at
+// most one unit of its level (level 4: 2^-46 of row max times column max, level 5
+// 2^-54).  Levels 7 to 12 are dropped: of row max times column max at worst
+// l 2^-53.4, the a-priori bound of the FP64 dot product of l terms; for digits
+// without a pattern some sqrt(6 l) 2^-57.6, 2^-52.3 at l = 256.  The operands'
+// rounding to 55 bits is at worst l 2^-55.  All of it is relative to the largest
+// entries: an entry 2^-k of its row's largest keeps 55 - k bits.
 // The seven accumulators are put together in 64-bit integers and rounded to
 // FP64 once.
 //
@@ -38,8 +41,7 @@
 // pass along a 256-point axis (120 GFLOP of digit products, 63 us at 1.9 PFLOP/s; the MMAs alone 50) and 78-82 along
 // the 128-point one, against 898 with MMAs whose descriptors one thread puts together, one producer warp, a ring of
 // seven images, eight epilogue warps and a division per point for G.  What is left: with the eigenbasis not
-// reloaded 534, without the epilogue's arithmetic 472, without either 412.  Sharing the eigenbasis stream by TMA
-// multicast in clusters of two or four changed nothing (950 against 953 and 1057 us when it was tried).
+// reloaded 534, without the epilogue's arithmetic 472, without either 412.
 #include <cuda_fp16.h>
 
 #include <algorithm>
