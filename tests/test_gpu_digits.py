@@ -89,3 +89,23 @@ def test_zero_rows_and_zero_input():
     ref = reference(pl, r)
     pl.precond(torch.from_numpy(r).cuda(), zd)
     assert rel_err(zd.cpu().numpy(), ref) <= 1e-12
+
+
+@pytest.mark.parametrize("shape", [(130, 200, 200), (40, 208, 200), (200, 256, 40)])
+def test_precond_many_tiles_a_block(shape):
+    """Passes of 5 to 10 data tiles per block, with one and two column blocks and with an eigenbasis that stays resident:
+    the rings, the accumulators and the eight row-exponent buffers go round."""
+    from paper_2501_03377_gb300 import Plan
+
+    nx, ny, nz = shape
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert max(ny * nz, nx * nz, nx * ny) > 4 * 32 * sms
+    pl = Plan(nx, ny, nz, ("P", "D", "N"))
+    r = synth.random_field(nx, ny, nz, seed=34)
+    # rows and planes of their own magnitude: a row's exponent read from another tile's buffer shows
+    r *= np.exp2(np.random.default_rng(35).integers(-40, 40, (nz, ny, 1)))
+    rd = torch.from_numpy(r).cuda()
+    zd = torch.full_like(rd, float("nan"))
+    pl.precond(rd, zd)
+    assert rel_err(zd.cpu().numpy(), reference(pl, r)) <= 1e-12
+    pl.close()

@@ -56,3 +56,21 @@ def test_application_that_gave_up_is_reported_once(hooks, prec):
     torch.cuda.synchronize()
     assert torch.equal(z, ref)
     pl.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp16", "bf16x3"])
+@pytest.mark.parametrize("timeout", [0, 1])
+def test_chunk_without_progress_ends_the_solve(hooks, prec, timeout):
+    """A read-back in which no iteration completed, or a wait gave up, ends the solve in two steps (its end and the report
+    of it) with an error; the plan solves again afterwards."""
+    from paper_2501_03377_gb300 import binding
+
+    pl, eta, u = plan_and_fields(prec)
+    steps = ctypes.c_int(0)
+    ptr = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    st = hooks.hook_stalled_chunk(pl.handle, ptr(eta), ptr(u), timeout, ctypes.byref(steps))
+    assert st == (binding.TPCG_ERR_TIMEOUT if timeout else binding.TPCG_ERR_NOT_CONVERGED)
+    assert steps.value == 2
+    st, info = pl.solve(eta, u, tol=1e-10, maxit=50, zero_guess=True)
+    assert st == 0 and info["rel_res_true"] <= 1e-10
+    pl.close()

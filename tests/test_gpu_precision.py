@@ -101,3 +101,22 @@ def test_cg_scalars_match_fp64_dots(prec, shape, bcs):
         assert e_rho <= bound_rho, (s, e_rho)
         assert e_alpha <= bound_wp + bound_rho, (s, e_alpha)
         assert e_beta <= 2 * bound_rho, (s, e_beta)
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16", "tf32", "bf16x3"])
+@pytest.mark.parametrize("shape", [(130, 70, 24), (201, 33, 7), (255, 19, 5)])
+def test_rho_of_odd_extents(shape, prec):
+    """The last pass's <R, Z> where its rows are unaligned and hold several column chunks per warp; bounds as above."""
+    nx, ny, nz = shape
+    bcs = ("P", "D", "N")
+    eta = synth.defect_rhs(nx, ny, nz, bcs, 20, 1.5, seed=33, noise_std=1e-3)
+    L = o.kron_sum(shape, bcs)
+    ulp = {"fp16": 2.0 ** -11, "tf32": 2.0 ** -11, "bf16x3": 2.0 ** -16}.get(prec, 2.0 ** -8)
+    bound_rho = max(1e-5, 50 * ulp / np.sqrt(nx * ny * nz))
+    for s in (1, 2):
+        st, info, sc, R1, Z, P = _run(prec, shape, bcs, s, eta)
+        assert sc["iter"] == s
+        wp, rho, rn = _fp64_scalars(L, R1, Z, P, sc["alpha"], o.is_singular(shape, bcs))
+        assert rn >= 1e-9 * info["eta_norm"]
+        assert abs(sc["rho"] - rho) <= bound_rho * rho, (s, abs(sc["rho"] - rho) / rho)
+        assert abs(sc["wp"] - wp) <= 1e-7 * wp
