@@ -237,11 +237,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
         // Every copy this warp issued has landed (bounded) before the CTA may leave, also where another warp gives up
         // after the last one was issued: of a whole sequence the last ring of images, which no later one overtakes.
         const int from = it < total ? it - kOzProd - kOzStages + 1 : total - kOzStages;
-        for (int j = it - kOzProd; j >= 0 && j >= from; j -= kOzProd) {
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try_wait(wfull(j % kOzStages), (uint32_t)((j / kOzStages) & 1)) && gtimer() - t0 < kWaitLimitNs) {
-          }
-        }
+        for (int j = it - kOzProd; j >= 0 && j >= from; j -= kOzProd)
+          wait_landed(wfull(j % kOzStages), (uint32_t)((j / kOzStages) & 1));
       }
       __syncwarp();
     } else {

@@ -231,11 +231,7 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
       }
     }
     if (lane == 0) {  // every issued load completes (bounded) before the CTA may exit, whoever gave up
-      for (int j = (it1 > NS1 ? it1 - NS1 : 0); j < it1; ++j) {
-        const unsigned long long t0 = gtimer();
-        while (!mbar_try_wait(full1(j % NS1), (uint32_t)((j / NS1) & 1)) && gtimer() - t0 < kWaitLimitNs) {
-        }
-      }
+      for (int j = (it1 > NS1 ? it1 - NS1 : 0); j < it1; ++j) wait_landed(full1(j % NS1), (uint32_t)((j / NS1) & 1));
     }
     __syncwarp();
   } else if (warp == kFrontalRing2Warp) {
@@ -253,11 +249,7 @@ __global__ void __launch_bounds__(kFrontalThreads, 1)
             tma_load_2d(sR2 + (uint32_t)s * kBlk, &tmA2, kt * 64, b * 128, full2(s));
           }
       {
-        for (int j = (it2 > NS2 ? it2 - NS2 : 0); j < it2; ++j) {
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try_wait(full2(j % NS2), (uint32_t)((j / NS2) & 1)) && gtimer() - t0 < kWaitLimitNs) {
-          }
-        }
+        for (int j = (it2 > NS2 ? it2 - NS2 : 0); j < it2; ++j) wait_landed(full2(j % NS2), (uint32_t)((j / NS2) & 1));
       }
     }
     __syncwarp();
@@ -581,14 +573,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1)
       }
     }
     if (lane == 0) {  // every issued load completes (bounded) before the CTA may exit, whoever gave up
-      for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
-        const unsigned long long t0 = gtimer();
-        while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {
-        }
-      }
-      const unsigned long long t0 = gtimer();
-      while (!mbar_try_wait(vbar, 0) && gtimer() - t0 < kWaitLimitNs) {
-      }
+      for (int j = (it > NS ? it - NS : 0); j < it; ++j) wait_landed(full(j % NS), (uint32_t)((j / NS) & 1));
+      wait_landed(vbar, 0);
     }
     __syncwarp();
   } else if (warp == 1) {

@@ -391,14 +391,8 @@ __global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::va
       // drain: every issued load has completed (bounded) before the CTA may exit, also where another warp gives up
       // after the last one was issued
       {
-        for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {
-          }
-        }
-        const unsigned long long t0 = gtimer();
-        while (!a.wstream && !mbar_try_wait(vbar, 0) && gtimer() - t0 < kWaitLimitNs) {
-        }
+        for (int j = (it > NS ? it - NS : 0); j < it; ++j) wait_landed(full(j % NS), (uint32_t)((j / NS) & 1));
+        if (!a.wstream) wait_landed(vbar, 0);
       }
     }
     __syncwarp();
@@ -504,12 +498,8 @@ __global__ void __launch_bounds__(TcWarps<FINAL, std::is_same<InT, Bf16Pair>::va
       }
       {  // every issued load completes before the CTA may exit
         for (int hh = 0; hh < 2; ++hh)
-          for (int k = (issued[hh] > a.rhalf ? issued[hh] - a.rhalf : 0); k < issued[hh]; ++k) {
-            const unsigned long long t0 = gtimer();
-            while (!mbar_try_wait(rfull(hh * kRHalf + (k % a.rhalf)), (uint32_t)((k / a.rhalf) & 1)) &&
-                   gtimer() - t0 < kWaitLimitNs) {
-            }
-          }
+          for (int k = (issued[hh] > a.rhalf ? issued[hh] - a.rhalf : 0); k < issued[hh]; ++k)
+            wait_landed(rfull(hh * kRHalf + (k % a.rhalf)), (uint32_t)((k / a.rhalf) & 1));
       }
     }
     __syncwarp();
@@ -994,14 +984,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
       }
       {  // every issued load completes before the CTA may exit (see k_modeprod_tc)
-        for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {
-          }
-        }
-        const unsigned long long t0 = gtimer();
-        while (!mbar_try_wait(vbar, 0) && gtimer() - t0 < kWaitLimitNs) {
-        }
+        for (int j = (it > NS ? it - NS : 0); j < it; ++j) wait_landed(full(j % NS), (uint32_t)((j / NS) & 1));
+        wait_landed(vbar, 0);
       }
     }
     __syncwarp();
@@ -1297,14 +1281,8 @@ __global__ void __launch_bounds__(kPairSplitThreads, 1)
         }
       }
       {  // every issued load completes before the CTA may exit (see k_modeprod_tc)
-        for (int j = (it > NS ? it - NS : 0); j < it; ++j) {
-          const unsigned long long t0 = gtimer();
-          while (!mbar_try_wait(full(j % NS), (uint32_t)((j / NS) & 1)) && gtimer() - t0 < kWaitLimitNs) {
-          }
-        }
-        const unsigned long long t0 = gtimer();
-        while (!mbar_try_wait(vbar, 0) && gtimer() - t0 < kWaitLimitNs) {
-        }
+        for (int j = (it > NS ? it - NS : 0); j < it; ++j) wait_landed(full(j % NS), (uint32_t)((j / NS) & 1));
+        wait_landed(vbar, 0);
       }
     }
     __syncwarp();

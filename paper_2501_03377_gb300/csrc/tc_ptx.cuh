@@ -63,6 +63,14 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, cons
   }
 }
 
+// The copies of a phase have landed, or the limit has passed: what a warp waits for before its CTA may leave.
+__device__ __forceinline__ void wait_landed(uint32_t bar, uint32_t parity) {
+  if (mbar_try_wait(bar, parity)) return;  // (reading the timer takes longer than the rest)
+  const unsigned long long t0 = gtimer();
+  while (!mbar_try_wait(bar, parity) && gtimer() - t0 < kWaitLimitNs) {
+  }
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
