@@ -298,6 +298,11 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
       __syncwarp();
     }
     __syncwarp();
+    // The warps of a warpgroup meet between two setmaxnreg, or what each of them holds is undefined: a producer warp with
+    // few images could otherwise ask for its registers back while a neighbour still held its own and a converter waited
+    // for them, without end.  The MMA warp is the last here: every converter has its registers by then.
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 72;");
   } else if (warp < kOzEpi0) {  // two warpgroups
     asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
     // ---------------- converters: warp w takes rows 4w .. 4w+3 of a tile; a lane holds elements 64 kt + 2 lane
@@ -378,6 +383,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
       }
     }
     __syncwarp();
+    asm volatile("bar.sync %0, 128;" ::"r"(2 + ((warp - kOzConv0) >> 2)) : "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
   } else {
     // ---------------- epilogue: thread = output column of the block; the four warps of a TMEM lane quadrant take
     // eight of the 32 rows each
@@ -467,12 +474,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_modeprod_oz(OzArgs a) {
     }
   }
 
-  // The registers go back to the launch's split behind a barrier: the warps of a warpgroup have to meet between two
-  // setmaxnreg, or what each of them holds is undefined.  A producer warp with few images could otherwise ask for its
-  // registers back before a neighbour had given its own away, and a converter then wait for them without end.
   __syncthreads();
-  if (warp <= kOzProd) asm volatile("setmaxnreg.inc.sync.aligned.u32 72;");
-  else if (warp < kOzEpi0) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
   if (warp == kOzProd) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
